@@ -185,10 +185,10 @@ def rank_kpoint(base, rank):
     return tuple(float(v) + 0.01 * rank for v in base)
 
 
-KERNEL_SOURCES = ("matvec.h", "matvec_impl.cuh", "matvec_kernels.cuh", "matvec_pk.cuh", "fft_pk.cuh",
-                  "fft_smem.cuh", "fft_reg.cuh", "nfs_complex.cuh", "cg_state.cuh", "tuning.h")
+KERNEL_SOURCES = ("matvec.h", "matvec_impl.cuh", "matvec_kernels.cuh", "fft_pk.cuh", "fft_reg.cuh",
+                  "nfs_complex.cuh", "cg_state.cuh", "tuning.h")
 PASS_COUNTERS = os.path.join(ROOT, "profiles", "pseudo96_matvec_c64_counters.json")
-PASS_KERNELS = ("k_pk_pass1", "k_pk_pass2", "k_pass3_fft_xy_project")
+PASS_KERNELS = ("k_rows_in", "k_columns", "k_rows_out")
 
 
 def kernel_sources_hash():

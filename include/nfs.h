@@ -165,18 +165,17 @@ int nfs_setup(nfs_ctx** out, const int grid[3], const double* lattice, const dou
 /* Au = A_r u (eq. factor_mtx / eq. spd_LS) in the given element type.  u and
  * Au are device pointers to 4n complex numbers and must not overlap.
  * NFS_C128_DS: complex128 vectors, product in double-single arithmetic (~1e-14;
- * MIXED contexts only, else NFS_EINVAL); it uses the context's CG workspace,
- * so it must not overlap an nfs_cg_solve or nfs_eigs on the same context. */
+ * MIXED contexts only, else NFS_EINVAL). */
 int nfs_matvec(nfs_ctx* ctx, int dtype, const void* u, void* Au);
 
-/* Run only the passes of nfs_matvec selected by `mask` (bit 0: pass 1,
- * spectral assembly + inverse DFT along x, y; bit 1: pass 2, inverse DFT
- * along z + material product + forward DFT along z; bit 2: pass 3, forward
- * DFT along y, x + projection onto P_r^*, Q_r^*; where the xy plane does not
- * fit in shared memory -- complex128 at 128 -- passes 1 and 3 are two kernels
- * each).  Passes communicate through the context's field workspace, so mask 7
- * equals nfs_matvec; other masks exist to time the passes one by one.  Same
- * arguments as nfs_matvec (NFS_C128 and NFS_C64 only). */
+/* Run only the kernels of nfs_matvec selected by `mask` (bit 0: spectral
+ * assembly, inverse DFT along x and the first stage of the one along y; bit 1:
+ * inverse DFT along z, the second stage along y, the material product and the
+ * same transforms forward; bit 2: the rest of the forward DFT along y, the one
+ * along x, and the projection onto P_r^*, Q_r^*).  They communicate through the
+ * context's field workspace, so mask 7 equals nfs_matvec; other masks exist to
+ * time the kernels one by one.  Same arguments as nfs_matvec (NFS_C128 and
+ * NFS_C64 only). */
 int nfs_matvec_passes(nfs_ctx* ctx, int dtype, int mask, const void* u, void* Au);
 
 /* out = B_r v = i [Sigma_r^{-1} v2; -Sigma_r^{-1} v1] (eq. NFSEP_spd_1), with

@@ -1,9 +1,9 @@
 """Autotuner for the complex64 A_r product's kernel schedule.
 
-The schedule knobs are compile-time (template parameters of the pass
-kernels): the radix split N = N1 * N2 of each line length (NFS_N1_<N>), the
-z-pass tile width and thread count, the CTAs per SM requested for the plane
-and z passes, and one or two complex elements per lane.  This tool builds
+The schedule knobs are compile-time (template parameters of the product's
+kernels): the radix split N = N1 * N2 of the z lines (NFS_N1_<N>) and of the x
+and y lines (NFS_N2_<N>), the x slots of a column CTA and of the workspace's
+runs, and the threads of the row kernels.  This tool builds
 variants of libnfs.so with candidate settings (in parallel, in a scratch
 directory), times the complex64 product of each on seeded smoothed chiral
 fields of the requested grid sizes, checks each variant against the
@@ -38,21 +38,17 @@ KNOBS = {
     "NFS_N1_64": [8, 16, 4],
     "NFS_N1_96": [12, 8, 16, 6],
     "NFS_N1_128": [16, 8],
-    "NFS_PLANE_MINB": [3, 2],
-    "NFS_Z_MINB": [3, 2],
-    "NFS_ZTILE_C64": [16, 8],
-    "NFS_C64_PAIRS": [0, 1],
-    "NFS_PASS1_FUSED_LOAD": [0, 1],
-    "NFS_SPLIT_C64": [0, 1],
-    "NFS_PK": [1, 0],
-    "NFS_PK1_FUSED": [0, 1],
-    "NFS_PK3": [0, 1],
+    "NFS_N2_48": [12, 8],
+    "NFS_N2_96": [12, 8],
+    "NFS_X": [2, 4],
+    "NFS_XL": [4, 2, 8],
+    "NFS_ROWS_NT": [192, 288],
 }
 MIN_GAIN = 0.03  # relative improvement a knob change must show to be taken
 
 # knobs that only matter for some sizes
 KNOB_SIZES = {"NFS_N1_32": {32}, "NFS_N1_48": {48}, "NFS_N1_64": {64}, "NFS_N1_96": {96}, "NFS_N1_128": {128},
-              "NFS_PK1_FUSED": {96}, "NFS_PK3": {96}}
+              "NFS_N2_48": {48}, "NFS_N2_96": {96}}
 
 
 def time_variant(lib, size, reps=60):

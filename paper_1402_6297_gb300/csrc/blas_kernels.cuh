@@ -6,9 +6,7 @@
 // Reductions are deterministic: a grid of blocks per problem fixed by the
 // vector length and the problem count (at most kRedBlocks) writes one
 // partial per block, and a one-block kernel sums the partials in a fixed
-// order.  Every CG kernel reads its problem's device `done` flag first and
-// returns at once when it is set, so launched iterations past convergence (or
-// for problems already converged) cost only empty launches.
+// order.
 #pragma once
 #include <cstdint>
 #include <type_traits>
@@ -49,13 +47,10 @@ __device__ __forceinline__ double sum_partials(const double* part, int count = k
 }
 
 // part[p * pstride + b] = block b's share of Re(conj(x_p) y_p); grid (blocks, P).
-// skip (optional): problem p is skipped when skip[p * sstride] is nonzero.
 template <typename C>
 __global__ void __launch_bounds__(kRedThreads)
-k_dot_re(const C* __restrict__ x, const C* __restrict__ y, long long N, double* __restrict__ part, long long pstride,
-         const int* __restrict__ skip, int sstride) {
+k_dot_re(const C* __restrict__ x, const C* __restrict__ y, long long N, double* __restrict__ part, long long pstride) {
   const int p = blockIdx.y;
-  if (skip && skip[(long long)p * sstride]) return;
   x += (long long)p * N;
   y += (long long)p * N;
   Acc<C> acc;
@@ -88,116 +83,45 @@ k_residual_parts(const double2* __restrict__ Ay, const double2* __restrict__ By,
   }
 }
 
-// CG start, one block per problem: rr = the sum of the nred partials in
-// part_a; stop once r^* r <= tol2[p].
+// CG start, one block per problem: r^* r = the sum of the nred partials of
+// k_dot_re in part_a becomes the only partial of the nb in part_b.
+template <typename R>
 __global__ void __launch_bounds__(kRedThreads)
-k_cg_init(CGState* st, const double* __restrict__ tol2, int maxit, int npart_a, int nred) {
+k_cg_init(CGState* st, const double* __restrict__ tol2, int maxit, int nred, int nb) {
+  using P = typename RedAccFor<R>::partial;
   st += blockIdx.x;
   const double rr = sum_partials(st->part_a, nred);
+  P* pb = reinterpret_cast<P*>(st->part_b);
+  for (int i = threadIdx.x; i < nb; i += kRedThreads) {
+    P v;
+    scalar_from(i == 0 ? rr : 0.0, v);  // (thread 0 holds the sum)
+    pb[i] = v;
+  }
   if (threadIdx.x == 0) {
-    const double t2 = tol2[blockIdx.x];
-    st->npart_a = npart_a;
     st->rr = rr;
-    st->tol2 = t2;
     st->it = 0;
     st->maxit = maxit;
-    st->status = 0;
-    st->alpha = st->beta = 0.0;
-    st->arrived = 0;
-    st->done = (rr <= t2) ? 1 : 0;
-    if (!(rr == rr)) { st->done = 1; st->status = -7; }
+    st->done = st->status = 0;
+    st->stop = st->halt = st->broken = 0;
+    scalar_from((double)INFINITY, *reinterpret_cast<P*>(&st->rr_last));
+    scalar_from(tol2[blockIdx.x], *reinterpret_cast<P*>(&st->tol2));
   }
 }
 
-// One CG step after the product, for every problem (grid (kUpdBlocks, P)):
-// alpha = rr / p^*Ap (every block sums the npart_a partials of p^* A p in the
-// same order, so all blocks agree; block 0 records it), x += alpha p,
-// r -= alpha Ap, and block b's partial of the new r^* r.  The last block to
-// finish (counted with an atomic, no waiting) sums the partials in fixed
-// order and sets beta = rr_new / rr, the convergence flag and the iteration
-// count for the next launch.  Vectors move in 16-byte loads.
-template <typename C>
-__global__ void __launch_bounds__(kUpdThreads)
-k_cg_update_xr(C* __restrict__ x, C* __restrict__ r, const C* __restrict__ p, const C* __restrict__ Ap, long long N,
-               CGState* st) {
-  const int pb = blockIdx.y;
-  st += pb;
-  if (st->done) return;
-  using V = typename std::conditional<sizeof(C) == 8, float4, double2>::type;
-  constexpr int EPV = 16 / (int)sizeof(C);
-  V* x4 = reinterpret_cast<V*>(x + (long long)pb * N);
-  V* r4 = reinterpret_cast<V*>(r + (long long)pb * N);
-  const V* p4 = reinterpret_cast<const V*>(p + (long long)pb * N);
-  const V* a4 = reinterpret_cast<const V*>(Ap + (long long)pb * N);
-  using R = typename RealOf<C>::type;
-  __shared__ double s_alpha;
-  __shared__ int s_ok, s_last;
-  double pAp;
-  {
-    double v = 0.0;
-    for (int i = threadIdx.x; i < st->npart_a; i += kUpdThreads) v += st->part_a[i];
-    pAp = block_sum<kUpdThreads>(v);  // valid in thread 0
-  }
+// End of a chunk of CG steps, one block per problem: the state that the host
+// reads, from the nb partials of r^* r (k_rows_in reaches the same decision from
+// the same partials when another chunk follows).
+template <typename R>
+__global__ void __launch_bounds__(kRedThreads) k_cg_check(CGState* st, int nb) {
+  using P = typename RedAccFor<R>::partial;
+  st += blockIdx.x;
+  const P rr = sum_partials_all<R, kRedThreads>(st->part_b, nb);
   if (threadIdx.x == 0) {
-    s_alpha = st->rr / pAp;
-    s_ok = (pAp > 0.0) && (s_alpha == s_alpha);  // also catches NaN
-    if (blockIdx.x == 0) {
-      st->pAp = pAp;
-      st->alpha = s_alpha;
-      if (!s_ok) {
-        st->status = -7;
-        st->done = 1;
-      }
-    }
-  }
-  __syncthreads();
-  if (!s_ok) return;  // breakdown: leave x, r untouched (uniform per block)
-  const R al = (R)s_alpha;
-  Acc<C> acc;
-  const long long NV = N / EPV;
-  for (long long i = (long long)blockIdx.x * kUpdThreads + threadIdx.x; i < NV;
-       i += (long long)gridDim.x * kUpdThreads) {
-    const V pi = p4[i], ai = a4[i];
-    V xi = x4[i], ri = r4[i];
-    if constexpr (EPV == 2) {
-      xi.x += al * pi.x; xi.y += al * pi.y; xi.z += al * pi.z; xi.w += al * pi.w;
-      ri.x -= al * ai.x; ri.y -= al * ai.y; ri.z -= al * ai.z; ri.w -= al * ai.w;
-      acc.add(ri.x * ri.x + ri.y * ri.y + ri.z * ri.z + ri.w * ri.w);
-    } else {
-      xi.x += al * pi.x; xi.y += al * pi.y;
-      ri.x -= al * ai.x; ri.y -= al * ai.y;
-      acc.add(ri.x * ri.x + ri.y * ri.y);
-    }
-    x4[i] = xi;
-    r4[i] = ri;
-  }
-  const double s = block_sum<kUpdThreads>(acc.total());
-  if (threadIdx.x == 0) {
-    st->part_b[blockIdx.x] = s;
-    __threadfence();
-    s_last = atomicAdd(&st->arrived, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!s_last) return;
-  // the last block: new residual norm, convergence, beta
-  __threadfence();
-  double v = 0.0;
-  for (int i = threadIdx.x; i < (int)gridDim.x; i += kUpdThreads) v += ((volatile double*)st->part_b)[i];
-  const double rr = block_sum<kUpdThreads>(v);
-  if (threadIdx.x == 0) {
-    st->arrived = 0;
-    st->it += 1;
-    if (!(rr == rr)) {
-      st->status = -7;
-      st->done = 1;
-    } else if (rr <= st->tol2) {
-      st->done = 1;
-    } else if (st->it >= st->maxit) {
-      st->status = -6;
-      st->done = 1;
-    }
-    st->beta = rr / st->rr;
-    st->rr = rr;
+    st->rr = scalar_double(rr);
+    const bool bad = st->broken || scalar_nan(rr);
+    const bool conv = scalar_le(rr, *reinterpret_cast<const P*>(&st->tol2));
+    st->status = bad ? -7 : conv ? 0 : st->it >= st->maxit ? -6 : 0;
+    st->done = bad || conv || st->it >= st->maxit;
   }
 }
 
@@ -209,6 +133,11 @@ template <typename C>
 __global__ void k_sub(const C* __restrict__ a, const C* __restrict__ b, C* __restrict__ y, long long total) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x)
     y[i] = csub(a[i], b[i]);
+}
+
+__global__ void k_add(const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ y, long long n) {
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    y[i] = a[i] + b[i];
 }
 
 // Refinement residual per problem p (skip64, skip32: the masks of the two

@@ -9,8 +9,8 @@
 // addition costs two packed additions for two complex numbers, a product with
 // a constant twiddle four packed multiply/fma instructions for two, and a
 // product with +-i only swaps the two registers (the sign goes into the next
-// addition).  In the A_r product the two lines are the two fields P_r u1 and
-// Q_r u2 of the same component (passes 1, 3) or of the same column (pass 2).
+// addition).  In the A_r product the two lines are the two fields of a pair
+// that the material couples (matvec_kernels.cuh).
 //
 // Sign convention as fft_reg.cuh: forward (INV = false) is
 // X[k] = sum_n x[n] exp(-2 pi i n k / L), inverse unnormalised with +.
@@ -72,9 +72,14 @@ __device__ __forceinline__ cp2 pscale(cp2 a, unsigned long long s) { return {vmu
 __device__ __forceinline__ cp2 pmul(cp2 a, unsigned long long c, unsigned long long s, unsigned long long ms) {
   return {vfma(a.im, ms, vmul(a.re, c)), vfma(a.im, c, vmul(a.re, s))};
 }
-// a * w for a twiddle table entry w = {(c, c), (s, s)} (direction folded in)
+// a * w for a twiddle table entry w = {(c, c), (s, s)}
 __device__ __forceinline__ cp2 pmul_tw(cp2 a, cp2 w) {
   return {vsub(vmul(a.re, w.re), vmul(a.im, w.im)), vfma(a.im, w.re, vmul(a.re, w.im))};
+}
+
+// a * conj(w)
+__device__ __forceinline__ cp2 pmul_tw_conj(cp2 a, cp2 w) {
+  return {vfma(a.im, w.im, vmul(a.re, w.re)), vsub(vmul(a.im, w.re), vmul(a.re, w.im))};
 }
 
 // a * exp(s 2 pi i j / 48), s = +1 inverse, -1 forward; j is a compile-time
@@ -179,16 +184,5 @@ struct PDFT {
     }
   }
 };
-
-// Stage A of a split line DFT (N = N1 N2, see fft_smem.cuh): the radix-N1
-// DFT of the items elements n1 N2 + n2 and the twiddles w_N^{n2 k1}; tw is the
-// table of the transform's direction, tw[m] = {(cos, cos), (+-sin, +-sin)} of
-// 2 pi m / N.
-template <bool INV, int N1>
-__device__ __forceinline__ void pk_stage_a(cp2 (&r)[N1], const cp2* tw, int n2) {
-  PDFT<N1, INV>::run(r);
-#pragma unroll
-  for (int k1 = 1; k1 < N1; ++k1) r[k1] = pmul_tw(r[k1], tw[n2 * k1]);
-}
 
 }  // namespace nfs

@@ -144,7 +144,7 @@ struct DFT {
 };
 
 // Two-level split of a line length N = N1 * N2 used by the shared-memory
-// line FFT (see fft_smem.cuh).  The first factor of each length is a tuning
+// line DFTs along z (matvec_kernels.cuh).  The first factor of each length is a tuning
 // choice (NFS_N1_<N>, picked by autotune.py into tuning.h); both factors must
 // be register DFT lengths (divisors of 48).
 #ifndef NFS_N1_24
@@ -171,9 +171,9 @@ struct SplitOf {
   static constexpr int N1 = F1, N2 = N / F1;
 };
 template <int N> struct LineSplit;
-template <> struct LineSplit<8>   { static constexpr int N1 = 8,  N2 = 1; };
-template <> struct LineSplit<12>  { static constexpr int N1 = 12, N2 = 1; };
-template <> struct LineSplit<16>  { static constexpr int N1 = 16, N2 = 1; };
+template <> struct LineSplit<8>   { static constexpr int N1 = 2,  N2 = 4; };
+template <> struct LineSplit<12>  { static constexpr int N1 = 3,  N2 = 4; };
+template <> struct LineSplit<16>  { static constexpr int N1 = 4,  N2 = 4; };
 template <> struct LineSplit<24>  : SplitOf<24, NFS_N1_24> {};
 template <> struct LineSplit<32>  : SplitOf<32, NFS_N1_32> {};
 template <> struct LineSplit<48>  : SplitOf<48, NFS_N1_48> {};

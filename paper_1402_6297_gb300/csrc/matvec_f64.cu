@@ -1,12 +1,13 @@
-// complex128 instantiation of the three-pass A_r product; the eigenvalue
-// gradient and eigenvector-field passes that share its pass-1 fields; the
+// complex128 instantiation of the A_r product; the eigenvalue gradient and the
+// eigenvector fields, which are other per-voxel steps of its column kernel; the
 // residual of the original GEP.
 #include <algorithm>
 #include <cmath>
 #include "matvec_impl.cuh"
 
 namespace nfs {
-NFS_INSTANTIATE_MATVEC(double)
+NFS_INSTANTIATE_ROWS(double)
+NFS_INSTANTIATE_COLUMNS(double)
 
 // Gradient of omega with respect to the per-component permittivity and the
 // chirality, for one eigenvector y of B_r y = theta A_r y (mu = 1):
@@ -17,191 +18,91 @@ NFS_INSTANTIATE_MATVEC(double)
 //   d/d eps_c   : -|s_c|^2 / Phi_c^2
 //   d/d gamma_c : 2 Re(conj(s_c) i p_c) / Phi_c + 2 gamma_c |s_c|^2 / Phi_c^2   (chiral)
 // and for the pseudochiral pair (a, b) with one gamma per voxel the two
-// coupled components' terms add (s_a = i gamma p_b + q_a, s_b = i gamma p_a + q_b).
-// `scale` carries weight / (n y^* B_r y): pass 1 leaves sqrt(n) p, sqrt(n) q.
-template <int N3, int TX, int NT>
-__global__ void __launch_bounds__(NT)
-k_grad_z(const double2* __restrict__ fld, const double2* __restrict__ twz, int ncols, const double* __restrict__ inv_phi,
-         const double* __restrict__ gam, int kind, int ax_a, int ax_b, double scale, double* __restrict__ d_eps,
-         double* __restrict__ d_gamma) {
-  using C = double2;
-  constexpr int LINES = 6 * TX;
-  constexpr int PITCH = LINES + 1;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* buf = reinterpret_cast<C*>(smem_raw);
-  C* stw = buf + N3 * PITCH;
-  for (int i = threadIdx.x; i < N3; i += NT) stw[i] = twz[i];
-  const int col0 = blockIdx.x * TX;
-  const long long n = (long long)ncols * N3;
-  for (int idx = threadIdx.x; idx < N3 * LINES; idx += NT) {
-    const int c = idx % TX;
-    const int t = idx / TX;
-    const int f = t % 6, z = t / 6;
-    buf[z * PITCH + f * TX + c] = fld[f * n + (long long)z * ncols + col0 + c];
-  }
-  __syncthreads();
-  smem_fft<true, N3, LINES, NT, 1, PITCH>(buf, stw);
-  for (int idx = threadIdx.x; idx < N3 * TX; idx += NT) {
-    const int c = idx % TX, z = idx / TX;
-    const long long v = (long long)z * ncols + col0 + c;
-    const C* row = buf + z * PITCH + c;
-    const C p[3] = {row[0], row[TX], row[2 * TX]};
-    const C q[3] = {row[3 * TX], row[4 * TX], row[5 * TX]};
-    double ip[3];
-    for (int k = 0; k < 3; ++k) ip[k] = inv_phi[k * n + v];
-    if (kind == kMediumChiral) {
-      for (int k = 0; k < 3; ++k) {
-        const double g = gam[k * n + v];
-        const C s = mk(q[k].x - g * p[k].y, q[k].y + g * p[k].x);   // q + i g p
-        const double s2 = cabs2(s);
-        const C ipk = cmul_i(p[k]);
-        const double re = s.x * ipk.x + s.y * ipk.y;                  // Re(conj(s) i p)
-        if (d_eps) d_eps[k * n + v] += scale * (-s2 * ip[k] * ip[k]);
-        if (d_gamma) d_gamma[k * n + v] += scale * (2.0 * re * ip[k] + 2.0 * g * s2 * ip[k] * ip[k]);
-      }
-    } else {
-      const double g = gam[v];
-      C s[3] = {q[0], q[1], q[2]};
-      s[ax_a] = cadd(q[ax_a], cmul_i(cscale(p[ax_b], g)));
-      s[ax_b] = cadd(q[ax_b], cmul_i(cscale(p[ax_a], g)));
-      double dg = 0.0;
-      for (int k = 0; k < 3; ++k) {
-        const double s2 = cabs2(s[k]);
-        if (d_eps) d_eps[k * n + v] += scale * (-s2 * ip[k] * ip[k]);
-        if (k == ax_a || k == ax_b) {
-          const C ipo = cmul_i(p[k == ax_a ? ax_b : ax_a]);
-          const double re = s[k].x * ipo.x + s[k].y * ipo.y;
-          dg += 2.0 * re * ip[k] + 2.0 * g * s2 * ip[k] * ip[k];
-        }
-      }
-      if (d_gamma) d_gamma[v] += scale * dg;
+// coupled components' terms add (s_a = i gamma p_b + q_a, s_b = i gamma p_a + q_b);
+// different CTAs form them, so they accumulate in two arrays.
+// `scale` carries weight / (n y^* B_r y): the DFTs leave sqrt(n) p, sqrt(n) q.
+struct GradStep {
+  static constexpr bool kForward = false;
+  const double* inv_phi;
+  const double* gam;
+  int kind, ax_a, ax_b;
+  long long n;
+  double scale;
+  double* d_eps;
+  double* dg;
+  template <int NB>
+  struct Vals {};
+  template <int NB>
+  __device__ __forceinline__ void load(const ColumnPos&, int, Vals<NB>&) const {}
+  template <int NB>
+  __device__ __forceinline__ double apply(const ColumnPos& c, int b, const Vals<NB>&, int, double2& p, double2& q) const {
+    const long long v = c.voxel(b);
+    const bool chiral = kind == kMediumChiral;
+    const bool coupled = chiral || c.j == ax_a || c.j == ax_b;
+    const double ip = inv_phi[c.j * n + v];
+    const double g = coupled ? gam[(chiral ? c.j * n : 0) + v] : 0.0;
+    const double2 s = mk(q.x - g * p.y, q.y + g * p.x);  // q + i g p
+    const double s2 = cabs2(s);
+    if (d_eps) d_eps[c.j * n + v] += scale * (-s2 * ip * ip);
+    if (dg && coupled) {
+      const double2 i_p = cmul_i(p);
+      const double re = s.x * i_p.x + s.y * i_p.y;  // Re(conj(s) i p)
+      dg[(chiral ? c.j * n : c.j == ax_a ? 0 : n) + v] += scale * (2.0 * re * ip + 2.0 * g * s2 * ip * ip);
     }
+    return 0.0;
   }
-}
-
-template <int N3>
-static cudaError_t grad_prep_n3() {
-  constexpr int TX = z_tile(N3, 16);
-  constexpr int NT = z_threads(N3, 16);
-  return cudaFuncSetAttribute(k_grad_z<N3, TX, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)z_smem<double, N3>());
-}
-
-template <int N3>
-static cudaError_t grad_launch_n3(const GradArgs& a) {
-  constexpr int TX = z_tile(N3, 16);
-  constexpr int NT = z_threads(N3, 16);
-  const int ncols = a.n1 * a.n2;
-  k_grad_z<N3, TX, NT><<<ncols / TX, NT, z_smem<double, N3>(), a.stream>>>(
-      a.fld, a.tw3, ncols, a.inv_phi, a.gam, a.kind, a.ax_a, a.ax_b, a.scale, a.d_eps, a.d_gamma);
-  return cudaGetLastError();
-}
-
-cudaError_t grad_prepare(int n1, int n2, int n3) {
-  if (!matvec_supported<double>(n1, n2, n3)) return cudaErrorInvalidValue;
-  switch (n3) {
-#define NFS_CASE(N) case N: return grad_prep_n3<N>();
-    NFS_FOR_EACH_SIZE(NFS_CASE)
-#undef NFS_CASE
-  }
-  return cudaErrorInvalidValue;
-}
+};
 
 cudaError_t grad_launch(const GradArgs& a) {
-  switch (a.n3) {
-#define NFS_CASE(N) case N: return grad_launch_n3<N>(a);
-    NFS_FOR_EACH_SIZE(NFS_CASE)
-#undef NFS_CASE
-  }
-  return cudaErrorInvalidValue;
+  const GradStep step{a.inv_phi, a.gam, a.kind, a.ax_a, a.ax_b, (long long)a.n1 * a.n1 * a.n3, a.scale, a.d_eps, a.dg};
+  return columns_launch<double>(a.fld, step, a.tw1, a.tw3, a.n1, a.n3, 1, nullptr, nullptr, BatchStrides{}, a.stream);
 }
 
 // Physical fields of one eigenvector (Algorithm 1, final step):
 //   x = [E; H] = B^{-1} diag(P_r, Q_r) y,   B = i [[zeta, mu], [-eps, -xi]].
 // By eq. B_inv, B^{-1} [p; q] = [i w; -i f] with the same
 //   w = Phi^{-1} (xi mu^{-1} p + q),   f = mu^{-1} (zeta w + p)
-// that the middle factors of A_r form (material_apply), so this is pass 1,
-// the inverse DFT along z and the material step of the product.  The product
+// that the middle factors of A_r form, so this is k_rows_in and k_columns up to
+// the material step of the product.  The product
 // never needs the Bloch twist D of T = n^{-1/2} D U (eq. mtx_T: it cancels
 // against T^*); the fields do, so it is applied here from the three 1-D
 // diagonals D_l[j] = exp(i 2 pi k.a_l j / n_l).  The two unnormalised DFTs
 // leave sqrt(n) p, sqrt(n) q; inv_sqrt_n removes that factor.
-template <int N3, int TX, int NT>
-__global__ void __launch_bounds__(NT)
-k_fields_z(const double2* __restrict__ fld, const double2* __restrict__ twz, int n1, int ncols, MatView<double> mat,
-           const double2* __restrict__ bloch, double inv_sqrt_n, double2* __restrict__ X) {
-  using C = double2;
-  constexpr int LINES = 6 * TX;
-  constexpr int PITCH = LINES + 1;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* buf = reinterpret_cast<C*>(smem_raw);
-  C* stw = buf + N3 * PITCH;
-  for (int i = threadIdx.x; i < N3; i += NT) stw[i] = twz[i];
-  const int col0 = blockIdx.x * TX;
-  const long long n = (long long)ncols * N3;
-  for (int idx = threadIdx.x; idx < N3 * LINES; idx += NT) {
-    const int c = idx % TX;
-    const int t = idx / TX;
-    const int f = t % 6, z = t / 6;
-    buf[z * PITCH + f * TX + c] = fld[f * n + (long long)z * ncols + col0 + c];
+struct FieldsStep {
+  static constexpr bool kForward = false;
+  ProductStep<double> material;  // scale 1 / sqrt(n)
+  const double2* bloch;
+  double2* X;
+  template <int NB>
+  using Vals = ProductStep<double>::Vals<NB>;
+  template <int NB>
+  __device__ __forceinline__ void load(const ColumnPos& c, int b, Vals<NB>& v) const {
+    material.load<NB>(c, b, v);
   }
-  __syncthreads();
-  smem_fft<true, N3, LINES, NT, 1, PITCH>(buf, stw);
-  const int n2 = ncols / n1;
-  for (int idx = threadIdx.x; idx < N3 * TX; idx += NT) {
-    const int c = idx % TX, z = idx / TX;
-    const int col = col0 + c;
-    const long long v = (long long)z * ncols + col;
-    const C* row = buf + z * PITCH + c;
-    const C p[3] = {row[0], row[TX], row[2 * TX]};
-    const C q[3] = {row[3 * TX], row[4 * TX], row[5 * TX]};
-    C f[3], w[3];
-    material_apply<double>(mat, v, p, q, f, w, inv_sqrt_n);
-    const C d = cmul(cmul(bloch[col % n1], bloch[n1 + col / n1]), bloch[n1 + n2 + z]);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      X[k * n + v] = cmul_i(cmul(d, w[k]));         // E = i D w
-      X[(3 + k) * n + v] = cmul_mi(cmul(d, f[k]));  // H = -i D f
-    }
+  template <int NB>
+  __device__ __forceinline__ double apply(const ColumnPos& c, int b, const Vals<NB>& mv, int k, double2& p, double2& q) const {
+    material.apply<NB>(c, b, mv, k, p, q);  // p <- f of axis s(j), q <- w of axis j
+    const int y = c.a + c.N1 * b;
+    const long long n = material.m.n, v = c.voxel(b);
+    const double2 d = cmul(cmul(bloch[c.x], bloch[c.n1 + y]), bloch[2 * c.n1 + c.z]);
+    const int s = pair_axis(material.m.kind, material.m.ax_a, material.m.ax_b, c.j);
+    X[c.j * n + v] = cmul_i(cmul(d, q));         // E = i D w
+    X[(3 + s) * n + v] = cmul_mi(cmul(d, p));    // H = -i D f
+    return 0.0;
   }
-}
-
-template <int N3>
-static cudaError_t fields_prep_n3() {
-  constexpr int TX = z_tile(N3, 16);
-  constexpr int NT = z_threads(N3, 16);
-  return cudaFuncSetAttribute(k_fields_z<N3, TX, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)z_smem<double, N3>());
-}
-
-template <int N3>
-static cudaError_t fields_launch_n3(const FieldsArgs& a) {
-  constexpr int TX = z_tile(N3, 16);
-  constexpr int NT = z_threads(N3, 16);
-  const int ncols = a.n1 * a.n2;
-  const MatView<double> mat{a.inv_phi, a.gam, a.inv_mu, a.kind, a.ax_a, a.ax_b, (long long)ncols * N3};
-  k_fields_z<N3, TX, NT><<<ncols / TX, NT, z_smem<double, N3>(), a.stream>>>(
-      a.fld, a.tw3, a.n1, ncols, mat, a.bloch, 1.0 / std::sqrt((double)ncols * N3), a.X);
-  return cudaGetLastError();
-}
-
-cudaError_t fields_prepare(int n1, int n2, int n3) {
-  if (!matvec_supported<double>(n1, n2, n3)) return cudaErrorInvalidValue;
-  switch (n3) {
-#define NFS_CASE(N) case N: return fields_prep_n3<N>();
-    NFS_FOR_EACH_SIZE(NFS_CASE)
-#undef NFS_CASE
-  }
-  return cudaErrorInvalidValue;
-}
+};
 
 cudaError_t fields_launch(const FieldsArgs& a) {
-  switch (a.n3) {
-#define NFS_CASE(N) case N: return fields_launch_n3<N>(a);
-    NFS_FOR_EACH_SIZE(NFS_CASE)
-#undef NFS_CASE
-  }
-  return cudaErrorInvalidValue;
+  const long long n = (long long)a.n1 * a.n1 * a.n3;
+  const FieldsStep step{{{a.inv_phi, a.gam, a.inv_mu, nullptr, nullptr, a.kind, a.ax_a, a.ax_b, n},
+                         1.0 / std::sqrt((double)n), 0},
+                        a.bloch, a.X};
+  return columns_launch<double>(a.fld, step, a.tw1, a.tw3, a.n1, a.n3, 1, nullptr, nullptr, BatchStrides{}, a.stream);
+}
+
+cudaError_t fields_prepare(int n1, int n3) {
+  const cudaError_t e = columns_prepare<double, GradStep>(n1, n3);
+  return e != cudaSuccess ? e : columns_prepare<double, FieldsStep>(n1, n3);
 }
 
 // Residual of an eigenpair (omega, x = [E; H]) in the GEP of eq.

@@ -1,21 +1,52 @@
-// The A_r matrix-vector product of the HHPD-NFGEP (eq. factor_mtx, applied
-// as in eq. spd_LS) in three HBM passes:
+// The A_r matrix-vector product of the HHPD-NFGEP (eq. factor_mtx, applied as
+// in eq. spd_LS) in three kernels, for complex64, complex128 and
+// double-single vectors.
 //
-//   pass 1  (cluster of 3 CTAs per (z-plane i3, group)):  spectral assembly
-//           p^ = P_r-coefficients, q^ = Q_r-coefficients per voxel, then the
-//           inverse DFT along x and y.  Group 0 builds p = P_r [u1a; u1b],
-//           group 1 builds q = Q_r [u2a; u2b]; CTA rank c owns component c.
-//           Each CTA assembles all three components of its third of the
-//           plane and the CTAs exchange them through shared memory (Stage).
-//   pass 2  (one CTA per tile of xy columns):  inverse DFT along z, the
-//           per-voxel material product of eq. factor_mtx, forward DFT along z
-//           (the tile goes between global memory and registers directly).
-//   pass 3  (cluster of 3 CTAs per (z-plane, group)):  forward DFT along y
-//           and x, then the projections P_r^* f (group 0) or Q_r^* w (group 1)
-//           from the three transformed components (remote shared loads).
+// A line DFT of length N = N1 N2 runs in two register stages.  Inverse:
+// stage A forms, for every n2 < N2, the radix-N1 DFT of the elements
+// n1 N2 + n2 and the twiddles w_N^{n2 k1}; stage B forms, for every k1 < N1,
+// the radix-N2 DFT of the slots k1 N2 + n2.  Both work in place (they write
+// the slots they read), which leaves element k1 + N1 k2 in slot k1 N2 + k2;
+// nothing in real space cares where an element sits, so it stays there.  The
+// forward transform undoes the two stages in turn: A' over the slots of one
+// k1, then B' over all k1 at one offset, which ends in natural order.
+// No stage has a hazard between its reads and its writes.
 //
-// Planes too large for shared memory take the five-pass form of
-// matvec_split.cuh.
+// Stage A of the y transform needs N1 rows of a plane, stage B then only the
+// N2 slots of one k1, so the y transform is split between the kernels and no
+// kernel holds a plane:
+//
+//   k_rows_in   (CTA: z index i3, n2 = b;  the N1 rows y = n1 N2 + b):  CG
+//               direction, spectral assembly p^ = P_r-coefficients,
+//               q^ = Q_r-coefficients, inverse DFT along x, stage A along y.
+//   k_columns   (CTA: pair j, k1 = a, X slots of x;  all z, the N2 slots of
+//               a):  inverse DFT along z; then per (z, x) stage B along y, the
+//               material product of eq. factor_mtx and stage A' along y, all in
+//               registers; forward DFT along z.
+//   k_rows_out  (CTA: i3, b;  the N1 rows y = b + N2 k):  stage B' along y,
+//               forward DFT along x, the projections P_r^* f, Q_r^* w, and in CG
+//               the step x += alpha p, r -= alpha A_r p.
+//
+// Why this split.  Holding whole xy planes between two plane passes and a z
+// pass (the form measured before) took 12 shared-memory round trips per
+// element against 10 here, read every input in three CTAs (one per component)
+// or exchanged it through a cluster, and needed 149 KB per CTA at 96 x 96, one
+// CTA per SM with its loads, transforms and stores one after another.  Here a
+// CTA holds 56 KB (rows) or 52 KB (columns) at 96^3, several share an SM and
+// overlap, all six fields of a voxel are in one CTA of the row kernels, and on
+// small grids the work spreads over more SMs, which is what complex128 needs:
+// GB300 retires one FP64 warp instruction per ~16 cycles and SM.
+//
+// Pairs.  The material couples p and q of one voxel only inside three pairs:
+// w_j = Phi_j^{-1} (q_j + i g mu^{-1} p_s(j)) and f_s(j) = mu^{-1} (p_s(j) -
+// i g w_j), with s the identity (chiral) or the exchange of the coupled axes
+// (pseudochiral; g = 0 for the third).  A CTA of k_columns therefore owns one
+// pair.  In complex64 the two fields of a pair also share one element: two
+// packed f32x2 registers hold (Re p, Re q) and (Im p, Im q) (fft_pk.cuh), so
+// every butterfly treats both lines in one instruction and every shared access
+// moves 16 bytes.  The other types keep p and q in separate lines.
+//
+// Workspace: E fld[j][f][a][x / XL][z][b][x % XL], f < NF.
 //
 // Basis per spectral voxel (Section 2), with a = (Lambda_1, Lambda_2, Lambda_3),
 // t = (alpha, beta, 1), Lambda_p = t x a, Lambda_q = |a|^2:
@@ -29,21 +60,15 @@
 // The Bloch twist D of T (eq. mtx_T) is a per-voxel unit scalar and commutes
 // with the per-voxel material product, so it cancels between T and T^*: the
 // kernels run plain DFTs.  The two unnormalised DFTs give a factor n, removed
-// in pass 2 (T = D U / sqrt(n)).
-//
-// Field buffer layout: fld[g][c][i3][j2][j1], g in {p/f, q/w}, c in {x, y, z};
-// z is spectral in passes 1 -> 2 and 2 -> 3, x and y are real-space.
+// in the material step (T = D U / sqrt(n)).
 #pragma once
-#include <cooperative_groups.h>
-
 #include <type_traits>
 
 #include "cg_state.cuh"
-#include "fft_smem.cuh"
+#include "fft_pk.cuh"
 #include "matvec.h"
 
 namespace nfs {
-namespace cg = cooperative_groups;
 
 constexpr int kMediumChiral = 0;
 constexpr int kMediumPseudochiral = 1;
@@ -52,35 +77,28 @@ constexpr int kMediumPseudochiral = 1;
 //   inv_phi[3][n] = 1 / Phi_c, Phi = eps - xi mu^{-1} zeta (diagonal here)
 //   gam     chiral [3][n] gamma_c; pseudochiral [n] gamma
 //   inv_mu  [3][n] = 1 / mu_c, or nullptr for mu = 1
+// in natural order, or (complex64 products) in the order k_columns meets them:
+// pair j, voxel (slot order) -> pmat = {1 / Phi_j, g} for two neighbouring b
+// and pmu = mu^{-1}_s(j) likewise (see pair_material_launch).
 template <typename R>
 struct MatView {
   const R* inv_phi;
   const R* gam;
   const R* inv_mu;
+  const float4* pmat;
+  const float2* pmu;
   int kind;
   int ax_a, ax_b;
   long long n;
 };
 
-// 16-byte vector type holding 16 / sizeof(C) complex elements.
-template <typename C> struct Vec16;
-template <> struct Vec16<float2> { using type = float4; };
-template <> struct Vec16<double2> { using type = double2; };
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
-// How the passes move elements between global and shared memory: EPV
-// consecutive elements per lane in one vector V.  One element per lane
-// (8-byte accesses for complex64, still 256 contiguous bytes per warp) keeps
-// every shared-memory access of a warp on consecutive addresses, free of bank
-// conflicts; pairs (16-byte accesses) halve the instruction count but make
-// 8-byte shared accesses stride 16 bytes, a two-way conflict.
-#ifndef NFS_C64_PAIRS
-#define NFS_C64_PAIRS 0
-#endif
-template <typename C>
-struct Lane {
-  static constexpr int EPV = (sizeof(C) == 8 && NFS_C64_PAIRS) ? 2 : 1;
-  using V = typename std::conditional<EPV == 2, float4, C>::type;
-};
+// Partner axis of pair j: s(j).
+__host__ __device__ __forceinline__ int pair_axis(int kind, int ax_a, int ax_b, int j) {
+  if (kind == kMediumChiral) return j;
+  return j == ax_a ? ax_b : (j == ax_b ? ax_a : j);
+}
 
 // Sum of one double per thread over the block (result valid in thread 0).
 template <int NT>
@@ -99,6 +117,118 @@ __device__ __forceinline__ double block_sum_dbl(double v) {
   }
   __syncthreads();
   return r;
+}
+
+// ---------------------------------------------------------------------------
+// schedule
+// ---------------------------------------------------------------------------
+
+// N = N1 N2 of the x and y transforms (N1 rows per CTA of the row kernels, N2
+// slots of y per CTA of k_columns), X, the x slots of a CTA of k_columns, and
+// XL, the x slots that lie together in the workspace.
+// N2 = 8 keeps the items of every stage within a thread's registers up to 128;
+// 96 and 48 take 12 in complex64: 8 rows instead of 12 fit four CTAs per SM and
+// divide evenly (7.6 CTAs per SM instead of 5.05).  Measured on GB300 at 96^3,
+// rows in / columns / rows out in us: 17.7 / 23.2 / 18.9 against 21.7 / 21.6 /
+// 19.7 with N2 = 8.  XL = 4: the row kernels reach the workspace in runs of XL
+// elements, k_columns in runs of X; XL = X = 2 gave 20.1 / 20.9 / 21.5, XL = 8
+// 16.7 / 28.4 / 17.9 (products: 63.8 us with XL = 4, 66.8, 67.5).  X = 2 against
+// X = 4: a product of 63.8 against 68.4 us (smaller CTAs, more of them per SM).
+// The smallest grids take N2 = 4 and X = 1 to have CTAs for the whole GPU (8^3:
+// 32 row CTAs and 48 column CTAs).
+#ifndef NFS_N2_48
+#define NFS_N2_48 12
+#endif
+#ifndef NFS_N2_96
+#define NFS_N2_96 12
+#endif
+#ifndef NFS_X
+#define NFS_X 2
+#endif
+#ifndef NFS_XL
+#define NFS_XL 4
+#endif
+template <typename R, int N> struct PlaneSplit {
+  static constexpr bool F32 = sizeof(cplx<R>) == 8;
+  static constexpr int N2 = N < 24 ? 4 : (F32 && N == 48) ? NFS_N2_48 : (F32 && N == 96) ? NFS_N2_96 : 8, N1 = N / N2;
+  static constexpr int X = N < 24 ? 1 : NFS_X;
+  static constexpr int XL = NFS_XL;
+};
+
+// N = N1 N2 of the z transforms.  The packed elements take the shortest lengths
+// in one stage; complex128 and double-single ones in two, so that more lanes of
+// the few warps work on a small tile (an FP64 warp instruction occupies its
+// pipe for ~16 cycles whether 8 or 32 lanes are active).
+template <typename R, int N> struct DepthSplit : LineSplit<N> {};
+template <> struct DepthSplit<float, 8> { static constexpr int N1 = 8, N2 = 1; };
+template <> struct DepthSplit<float, 12> { static constexpr int N1 = 12, N2 = 1; };
+template <> struct DepthSplit<float, 16> { static constexpr int N1 = 16, N2 = 1; };
+
+// Elements of the workspace and of shared memory, and how many of them hold
+// the two fields of a pair.
+template <typename R> struct ElemOf {
+  using E = cplx<R>;
+  static constexpr int NF = 2;
+};
+template <> struct ElemOf<float> {
+  using E = cp2;
+  static constexpr int NF = 1;
+};
+
+// One register DFT on elements of either kind.
+template <int L, bool INV> __device__ __forceinline__ void edft(cp2* x) { PDFT<L, INV>::run(x); }
+template <int L, bool INV, typename C> __device__ __forceinline__ void edft(C* x) { DFT<L, INV>::run(x); }
+
+// Twiddles: the table holds exp(-2 pi i m / N); packed elements keep each one
+// as {(cos, cos), (-sin, -sin)}.
+__device__ __forceinline__ cp2 tw_entry(float2 w) { return {splat(w.x), splat(w.y)}; }
+template <typename C> __device__ __forceinline__ C tw_entry(C w) { return w; }
+template <bool INV> __device__ __forceinline__ cp2 etwiddle(cp2 a, cp2 w) { return INV ? pmul_tw_conj(a, w) : pmul_tw(a, w); }
+template <bool INV, typename C> __device__ __forceinline__ C etwiddle(C a, C w) { return INV ? cmulc(w, a) : cmul(a, w); }
+
+// Elements of a pair from and to its two complex fields (scalar elements: one
+// field per element, `stride` apart).
+__device__ __forceinline__ void put_pair(cp2* line0, int stride, float2 p, float2 q) {
+  (void)stride;
+  *line0 = {f2pk(p.x, q.x), f2pk(p.y, q.y)};
+}
+template <typename C> __device__ __forceinline__ void put_pair(C* line0, int stride, C p, C q) {
+  line0[0] = p;
+  line0[stride] = q;
+}
+__device__ __forceinline__ void get_pair(const cp2* line0, int stride, float2& p, float2& q) {
+  (void)stride;
+  const cp2 v = *line0;
+  const float2 re = pk2f(v.re), im = pk2f(v.im);
+  p = mk(re.x, im.x);
+  q = mk(re.y, im.y);
+}
+template <typename C> __device__ __forceinline__ void get_pair(const C* line0, int stride, C& p, C& q) {
+  p = line0[0];
+  q = line0[stride];
+}
+
+// Vector elements in memory to and from the type computed in.
+template <typename R, typename V> __device__ __forceinline__ cplx<R> from_vec(V v) {
+  if constexpr (std::is_same<cplx<R>, V>::value) return v;
+  else return cplx<R>{R(v.x), R(v.y)};
+}
+template <typename R> __device__ __forceinline__ vecc<R> to_vec(cplx<R> v) {
+  if constexpr (std::is_same<cplx<R>, vecc<R>>::value) return v;
+  else return vecc<R>{(double)v.x, (double)v.y};
+}
+
+template <typename C> __device__ __forceinline__ void cswap(C& a, C& b) {
+  const C t = a;
+  a = b;
+  b = t;
+}
+// Exchange the entries of the coupled pair (a, b) of a pseudochiral medium.
+template <typename C> __device__ __forceinline__ void swap_axes(C* v, int ax_a, int ax_b) {
+  const int s = ax_a + ax_b;  // 1: x-y, 2: x-z, 3: y-z
+  if (s == 1) cswap(v[0], v[1]);
+  else if (s == 2) cswap(v[0], v[2]);
+  else cswap(v[1], v[2]);
 }
 
 template <typename R>
@@ -165,561 +295,609 @@ __global__ void k_basis_table(const cplx<R>* __restrict__ lam, int n1, int n2, i
 }
 
 // ---------------------------------------------------------------------------
-// pass 1
+// stages over lines in shared memory: element e of line l at buf[l LS + e ES]
+// (work items take the line index fastest across threads; the callers'
+// pitches are odd, so the 16-byte accesses of 8 neighbouring lanes hit 8
+// different bank groups)
 // ---------------------------------------------------------------------------
 
-// Element range [e0, e1) of cluster rank r over a plane of NE elements, with
-// even boundaries so that 16-byte vectors never straddle two ranks.
-template <int NE>
-__device__ __forceinline__ int third_bound(int r) {
-  return r >= 3 ? NE : ((r * NE) / 3) & ~1;
-}
-
-template <typename R>
-__device__ __forceinline__ cplx<R> pick3(int k, cplx<R> a, cplx<R> b, cplx<R> c) {
-  return k == 0 ? a : (k == 1 ? b : c);
-}
-
-// Shared-memory staging of pass 1's exchange.  Rank r computes all three
-// components of its third of the plane; its own component goes to its final
-// place, the other two to staging gaps of its plane buffer (outside its own
-// third's final positions), from which the partner CTAs load them.
-template <int NX, int NY>
-struct Stage {
-  static constexpr int PITCH = NX + 1, NE = NX * NY, TOTAL = NY * PITCH;
-  __host__ __device__ static constexpr int pos(int e) { return (e / NX) * PITCH + e % NX; }
-  __host__ __device__ static constexpr int e0(int r) { return r >= 3 ? NE : ((r * NE) / 3) & ~1; }
-  // start of the staging run of rank r's values of component r + k (k = 1, 2)
-  __host__ __device__ static constexpr int base(int r, int k) {
-    const int s = e0(r + 1) - e0(r);
-    const int lo = pos(e0(r)), hi = pos(e0(r + 1) - 1) + 1, rhi = (hi + 1) & ~1;
-    if (lo >= s && TOTAL - rhi >= s) return k == 1 ? 0 : rhi;
-    if (TOTAL - rhi >= 2 * s) return k == 1 ? rhi : rhi + s;
-    return k == 1 ? 0 : s;
+// Inverse stage A (or, FWD = true, forward stage B'): radix N1 over the slots
+// n1 N2 + n2 of one n2; the inverse stage multiplies by its twiddles.
+template <bool FWD, int N1, int N2, int NLINES, int NT, int LS, int ES, typename E>
+__device__ __forceinline__ void stage_strided(E* buf, const E* tw) {
+  constexpr int ITEMS = NLINES * N2;
+#pragma unroll 1
+  for (int it = threadIdx.x; it < ITEMS; it += NT) {
+    const int l = it % NLINES, n2 = it / NLINES;
+    E* base = buf + l * LS + n2 * ES;
+    E r[N1];
+#pragma unroll
+    for (int n1 = 0; n1 < N1; ++n1) r[n1] = base[n1 * N2 * ES];
+    edft<N1, !FWD>(r);
+    if (!FWD) {
+#pragma unroll
+      for (int k1 = 1; k1 < N1; ++k1) r[k1] = etwiddle<true>(r[k1], tw[n2 * k1]);
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < N1; ++k1) base[k1 * N2 * ES] = r[k1];
   }
-};
+}
 
-// Pass 1's input handling: 0 loads every input block first (all loads in
-// flight together), 1 handles one block at a time (fewer live registers).
-#ifndef NFS_PASS1_FUSED_LOAD
-#define NFS_PASS1_FUSED_LOAD 0
-#endif
+// Inverse stage B (or, FWD = true, forward stage A'): radix N2 over the slots
+// k1 N2 + n2 of one k1; the forward stage multiplies by its twiddles.
+template <bool FWD, int N1, int N2, int NLINES, int NT, int LS, int ES, typename E>
+__device__ __forceinline__ void stage_group(E* buf, const E* tw) {
+  constexpr int ITEMS = NLINES * N1;
+#pragma unroll 1
+  for (int it = threadIdx.x; it < ITEMS; it += NT) {
+    const int l = it % NLINES, k1 = it / NLINES;
+    E* base = buf + l * LS + k1 * N2 * ES;
+    E r[N2];
+#pragma unroll
+    for (int i = 0; i < N2; ++i) r[i] = base[i * ES];
+    edft<N2, !FWD>(r);
+    if (FWD) {
+#pragma unroll
+      for (int i = 1; i < N2; ++i) r[i] = etwiddle<false>(r[i], tw[k1 * i]);
+    }
+#pragma unroll
+    for (int i = 0; i < N2; ++i) base[i * ES] = r[i];
+  }
+}
 
-template <typename R, int NX, int NY, int NT, int MINB>
-__global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(NT, MINB)
-k_pass1_assemble_ifft_xy(const cplx<R>* u, cplx<R>* __restrict__ fld,
-                         const cplx<R>* __restrict__ lam, const cplx<R>* __restrict__ twx,
-                         const cplx<R>* __restrict__ twy, int n3, R alpha, R beta,
-                         const int* __restrict__ skip, const cplx<R>* __restrict__ cg_r,
-                         const double* __restrict__ cg_beta, const cplx<R>* __restrict__ basis, BatchStrides bs) {
+// ---------------------------------------------------------------------------
+// k_rows_in: grid (N2 NF, n3, P); scalar elements: a CTA takes one field of
+// each pair (P_r u1 or Q_r u2)
+// ---------------------------------------------------------------------------
+template <typename R, int N>
+constexpr size_t rows_smem() {
+  return (size_t)(3 * PlaneSplit<R, N>::N1 * (N + 1) + N) * 16;
+}
+
+template <typename R, int N, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB)
+k_rows_in(const vecc<R>* u, typename ElemOf<R>::E* __restrict__ fld, const cplx<R>* __restrict__ lam,
+          const cplx<R>* __restrict__ twx, R alpha, R beta, int kind, int ax_a, int ax_b, const int* __restrict__ skip,
+          const cplx<R>* __restrict__ basis, BatchStrides bs, CgFuse<R> cg) {
   using C = cplx<R>;
-  constexpr int PITCH = NX + 1;
-  constexpr int NE = NX * NY;
-  constexpr int EPV = Lane<C>::EPV;
+  using E = typename ElemOf<R>::E;
+  using S = PlaneSplit<R, N>;
+  constexpr int NF = ElemOf<R>::NF, N1 = S::N1, N2 = S::N2, X = S::X, XL = S::XL;
+  constexpr int PITCH = N + 1;
+  constexpr int LINES = 3 * N1;  // line j N1 + row
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* plane = reinterpret_cast<C*>(smem_raw);
-  C* stx = plane + NY * PITCH;
-  C* sty = stx + NX;
-  cg::cluster_group cl = cg::this_cluster();
-  const int prob = blockIdx.z / n3;
-  if (skip != nullptr && skip[(long long)prob * bs.sskip]) return;  // uniform across the cluster
-  const int rank = (int)cl.block_rank();
-  const int grp = blockIdx.y;
-  const int i3 = blockIdx.z % n3;
+  E* buf = reinterpret_cast<E*>(smem_raw);
+  E* tw = buf + LINES * PITCH;
+  const int b = blockIdx.x % N2, fsel = blockIdx.x / N2, i3 = blockIdx.y, prob = blockIdx.z, n3 = gridDim.y;
+  if (skip != nullptr && skip[(long long)prob * bs.sskip]) return;
+  constexpr bool CGT = !std::is_same<R, df>::value;  // (the double-single product never runs CG)
+  CGState* st = (CGT && cg.st != nullptr) ? cg.st + prob : nullptr;
+  if (st != nullptr) u = cg.p;
   u += prob * bs.su;
   fld += prob * bs.sfld;
   lam += (long long)prob * bs.slam;
   if (basis != nullptr) basis += prob * bs.sbasis;
-  if (cg_r != nullptr) {
-    cg_r += prob * bs.su;
-    cg_beta += prob * bs.sstate;
-  }
-  for (int i = threadIdx.x; i < NX; i += NT) stx[i] = twx[i];
-  for (int i = threadIdx.x; i < NY; i += NT) sty[i] = twy[i];
-
-  const long long n = (long long)NE * n3;
-  const int e0 = third_bound<NE>(rank), e1 = third_bound<NE>(rank + 1);
-  const C* ua = u + (2 * grp) * n + (long long)i3 * NE + e0;
-  const C* ub = ua + n;
-  // this rank's inputs, loaded into registers (both halves in flight together)
-  using V = typename Lane<C>::V;
-  constexpr int NVMAX = (NE / 3 + 2) / EPV;
-  constexpr int PER = (NVMAX + NT - 1) / NT;
-  const int nv = (e1 - e0) / EPV;
-#if NFS_PASS1_FUSED_LOAD
-  // one block of inputs at a time: load, CG update, assembly and staging, so
-  // that only one block's inputs are live (no register spills at 96 x 96
-  // with three CTAs per SM)
-  const C a3 = lam[NX + NY + i3];
-  using SG = Stage<NX, NY>;
-  const int sb1 = SG::base(rank, 1), sb2 = SG::base(rank, 2);
-  const int r1 = rank == 2 ? 0 : rank + 1, r2 = rank == 0 ? 2 : rank - 1;
-  const R bt = cg_r != nullptr ? (R)*cg_beta : (R)0;
-  const long long goff = (2 * grp) * n + (long long)i3 * NE + e0;
+  const vecc<R>* r_in = st != nullptr ? cg.r + prob * bs.su : nullptr;
+  const long long n = (long long)N * N * n3;
+  // the quarters of u that this CTA needs: all, or the two of its field
+  constexpr int NQ = 4 / NF;
+  const int q0 = NF == 1 ? 0 : 2 * fsel;
+  // the first voxel's inputs are on their way while the tables are staged and
+  // (in CG) the partials of r^* r are summed; each later voxel's while the one
+  // before it is assembled
+  constexpr int NV = N1 * N;
+  vecc<R> v[NQ], g[NQ];
+  auto fetch = [&](int vi) {
+    if (vi < NV) {
+      const long long e = ((long long)i3 * N + (vi / N) * N2 + b) * N + vi % N + q0 * n;
 #pragma unroll
-  for (int b = 0; b < PER; ++b) {
-    const int v = b * NT + (int)threadIdx.x;
-    if (v < nv) {
-      V ra = reinterpret_cast<const V*>(ua)[v];
-      V rb = reinterpret_cast<const V*>(ub)[v];
-      if (cg_r != nullptr) {
-        // CG direction update fused into the load: u = r + beta u, stored back
-        const V qa = ldg_c(reinterpret_cast<const V*>(cg_r + goff) + v);
-        const V qb = ldg_c(reinterpret_cast<const V*>(cg_r + goff + n) + v);
-        if constexpr (EPV == 2) {
-          ra = make_float4(qa.x + bt * ra.x, qa.y + bt * ra.y, qa.z + bt * ra.z, qa.w + bt * ra.w);
-          rb = make_float4(qb.x + bt * rb.x, qb.y + bt * rb.y, qb.z + bt * rb.z, qb.w + bt * rb.w);
-        } else {
-          ra = mk(qa.x + bt * ra.x, qa.y + bt * ra.y);
-          rb = mk(qb.x + bt * rb.x, qb.y + bt * rb.y);
-        }
-        reinterpret_cast<V*>(const_cast<C*>(ua))[v] = ra;
-        reinterpret_cast<V*>(const_cast<C*>(ub))[v] = rb;
-      }
+      for (int q = 0; q < NQ; ++q) v[q] = u[q * n + e];
+      if (r_in != nullptr) {
 #pragma unroll
-      for (int h = 0; h < EPV; ++h) {
-        const int e = e0 + v * EPV + h;
-        C va, vb;
-        if constexpr (EPV == 2) {
-          va = h == 0 ? mk(ra.x, ra.y) : mk(ra.z, ra.w);
-          vb = h == 0 ? mk(rb.x, rb.y) : mk(rb.z, rb.w);
-        } else {
-          va = ra;
-          vb = rb;
-        }
-        const int i1 = e % NX, i2 = e / NX;
-        Basis<R> B;
-        voxel_basis<R>(basis, n, (long long)i3 * NE + e, lam[i1], lam[NX + i2], a3, alpha, beta, B);
-        C o[3];
-        if (grp == 0) {
-#pragma unroll
-          for (int k = 0; k < 3; ++k) o[k] = csub(cmul(B.x[k], vb), cmul(B.c[k], va));
-        } else {
-#pragma unroll
-          for (int k = 0; k < 3; ++k) o[k] = cadd(cmulc(B.x[k], va), cmulc(B.c[k], vb));
-        }
-        const int sidx = i2 * PITCH + i1;
-        plane[sidx] = pick3<R>(rank, o[0], o[1], o[2]);
-        plane[sb1 + (e - e0)] = pick3<R>(r1, o[0], o[1], o[2]);
-        plane[sb2 + (e - e0)] = pick3<R>(r2, o[0], o[1], o[2]);
+        for (int q = 0; q < NQ; ++q) g[q] = ldg_c(r_in + q * n + e);
       }
     }
-  }
-#else
-  V ra[PER], rb[PER];
-#pragma unroll
-  for (int b = 0; b < PER; ++b) {
-    const int v = b * NT + (int)threadIdx.x;
-    if (v < nv) {
-      ra[b] = reinterpret_cast<const V*>(ua)[v];
-      rb[b] = reinterpret_cast<const V*>(ub)[v];
-    }
-  }
-  if (cg_r != nullptr) {
-    // CG direction update fused into the load: u = r + beta u, stored back
-    const R bt = (R)*cg_beta;
-    const long long off = (2 * grp) * n + (long long)i3 * NE + e0;
-    const V* rva = reinterpret_cast<const V*>(cg_r + off);
-    const V* rvb = reinterpret_cast<const V*>(cg_r + off + n);
-    V* wa = reinterpret_cast<V*>(const_cast<C*>(ua));
-    V* wb = reinterpret_cast<V*>(const_cast<C*>(ub));
-#pragma unroll
-    for (int b = 0; b < PER; ++b) {
-      const int v = b * NT + (int)threadIdx.x;
-      if (v < nv) {
-        const V qa = ldg_c(rva + v), qb = ldg_c(rvb + v);
-        if constexpr (EPV == 2) {
-          ra[b] = make_float4(qa.x + bt * ra[b].x, qa.y + bt * ra[b].y, qa.z + bt * ra[b].z, qa.w + bt * ra[b].w);
-          rb[b] = make_float4(qb.x + bt * rb[b].x, qb.y + bt * rb[b].y, qb.z + bt * rb[b].z, qb.w + bt * rb[b].w);
-        } else {
-          ra[b] = mk(qa.x + bt * ra[b].x, qa.y + bt * ra[b].y);
-          rb[b] = mk(qb.x + bt * rb[b].x, qb.y + bt * rb[b].y);
-        }
-        wa[v] = ra[b];
-        wb[v] = rb[b];
+  };
+  fetch(threadIdx.x);
+  for (int i = threadIdx.x; i < N; i += NT) tw[i] = tw_entry(twx[i]);
+  R bt = (R)0;
+  if constexpr (CGT) {
+    if (st != nullptr) {
+      using P = typename RedAccFor<R>::partial;
+      const P tol2 = *reinterpret_cast<const P*>(&st->tol2), last = *reinterpret_cast<const P*>(&st->rr_last);
+      const bool over = st->halt || st->it >= st->maxit;
+      const P rr = sum_partials_all<R, NT>(st->part_b, gridDim.x * n3);
+      const bool stop = over || scalar_nan(rr) || scalar_le(rr, tol2);
+      if (blockIdx.x == 0 && i3 == 0 && threadIdx.x == 0) {
+        st->stop = stop;
+        *reinterpret_cast<P*>(&st->rr_now) = rr;
       }
+      if (stop) return;
+      bt = (R)scalar_ratio(rr, last);
     }
   }
-  const C a3 = lam[NX + NY + i3];
-  // exchange through shared memory: all three components of this third are
-  // computed here; this rank's goes to its final place, the other two to
-  // staging runs that the partner CTAs load after the cluster barrier
-  using SG = Stage<NX, NY>;
-  const int sb1 = SG::base(rank, 1), sb2 = SG::base(rank, 2);
-  const int r1 = rank == 2 ? 0 : rank + 1, r2 = rank == 0 ? 2 : rank - 1;
+  const C a3 = lam[2 * N + i3];
+#pragma unroll 1
+  for (int vi = threadIdx.x; vi < NV; vi += NT) {
+    const int row = vi / N, x = vi % N, y = row * N2 + b;
+    const long long e = ((long long)i3 * N + y) * N + x;
+    C w[NQ];
 #pragma unroll
-  for (int b = 0; b < PER; ++b) {
-    const int v = b * NT + (int)threadIdx.x;
-    if (v < nv) {
+    for (int q = 0; q < NQ; ++q) w[q] = from_vec<R>(v[q]);
+    if constexpr (CGT) {
+      if (r_in != nullptr) {
+        // CG direction p = r + beta p, stored back
 #pragma unroll
-      for (int h = 0; h < EPV; ++h) {
-        const int e = e0 + v * EPV + h;
-        C va, vb;
-        if constexpr (EPV == 2) {
-          va = h == 0 ? mk(ra[b].x, ra[b].y) : mk(ra[b].z, ra[b].w);
-          vb = h == 0 ? mk(rb[b].x, rb[b].y) : mk(rb[b].z, rb[b].w);
-        } else {
-          va = ra[b];
-          vb = rb[b];
-        }
-        const int i1 = e % NX, i2 = e / NX;
-        Basis<R> B;
-        voxel_basis<R>(basis, n, (long long)i3 * NE + e, lam[i1], lam[NX + i2], a3, alpha, beta, B);
-        C o[3];
-        if (grp == 0) {
-          // p^ = -c u1a + x u1b
-#pragma unroll
-          for (int k = 0; k < 3; ++k) o[k] = csub(cmul(B.x[k], vb), cmul(B.c[k], va));
-        } else {
-          // q^ = conj(x) u2a + conj(c) u2b
-#pragma unroll
-          for (int k = 0; k < 3; ++k) o[k] = cadd(cmulc(B.x[k], va), cmulc(B.c[k], vb));
-        }
-        const int sidx = i2 * PITCH + i1;
-        plane[sidx] = pick3<R>(rank, o[0], o[1], o[2]);
-        plane[sb1 + (e - e0)] = pick3<R>(r1, o[0], o[1], o[2]);
-        plane[sb2 + (e - e0)] = pick3<R>(r2, o[0], o[1], o[2]);
-      }
-    }
-  }
-#endif
-  cl.sync();  // staging complete in every CTA of the cluster
-  {
-    // load this rank's component of the two other thirds from the partners'
-    // staging runs, then (after every CTA has read) put them in place
-    using V = typename Lane<C>::V;
-    constexpr int S_MAX = (NE / 3 + 2) / EPV;
-    constexpr int PER2 = (S_MAX + NT - 1) / NT;
-    V g[2][PER2];
-    int gt[2], gn[2];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int t = q == 0 ? r1 : r2;               // partner rank (its third)
-      const int k = q == 0 ? 2 : 1;                 // this rank = t + k (mod 3)
-      const V* src = reinterpret_cast<const V*>(cl.map_shared_rank(plane, t) + SG::base(t, k));
-      gt[q] = t;
-      gn[q] = (SG::e0(t + 1) - SG::e0(t)) / EPV;
-#pragma unroll
-      for (int b = 0; b < PER2; ++b) {
-        const int v = b * NT + (int)threadIdx.x;
-        if (v < gn[q]) g[q][b] = src[v];
-      }
-    }
-    cl.sync();  // every CTA has read its partners' staging
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int te0 = SG::e0(gt[q]);
-#pragma unroll
-      for (int b = 0; b < PER2; ++b) {
-        const int v = b * NT + (int)threadIdx.x;
-        if (v < gn[q]) {
-#pragma unroll
-          for (int h = 0; h < EPV; ++h) {
-            const int e = te0 + v * EPV + h;
-            C val;
-            if constexpr (EPV == 2) {
-              val = h == 0 ? mk(g[q][b].x, g[q][b].y) : mk(g[q][b].z, g[q][b].w);
-            } else {
-              val = g[q][b];
-            }
-            plane[(e / NX) * PITCH + (e % NX)] = val;
-          }
+        for (int q = 0; q < NQ; ++q) {
+          w[q] = mk(g[q].x + bt * w[q].x, g[q].y + bt * w[q].y);
+          const_cast<C*>(u)[(q0 + q) * n + e] = w[q];
         }
       }
     }
-    __syncthreads();
+    fetch(vi + NT);
+    Basis<R> B;
+    voxel_basis<R>(basis, n, e, lam[x], lam[N + y], a3, alpha, beta, B);
+    E* cell = buf + row * PITCH + x;
+    if constexpr (NF == 1) {
+      C p[3], q[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        p[k] = csub(cmul(B.x[k], w[1]), cmul(B.c[k], w[0]));   // p^ = -c u1a + x u1b
+        q[k] = cadd(cmulc(B.x[k], w[2]), cmulc(B.c[k], w[3]));  // q^ = conj(x) u2a + conj(c) u2b
+      }
+      if (kind != kMediumChiral) swap_axes(p, ax_a, ax_b);
+#pragma unroll
+      for (int j = 0; j < 3; ++j) put_pair(cell + j * N1 * PITCH, 0, p[j], q[j]);
+    } else {
+      C o[3];
+      if (fsel == 0) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) o[k] = csub(cmul(B.x[k], w[1]), cmul(B.c[k], w[0]));
+        if (kind != kMediumChiral) swap_axes(o, ax_a, ax_b);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) o[k] = cadd(cmulc(B.x[k], w[0]), cmulc(B.c[k], w[1]));
+      }
+#pragma unroll
+      for (int j = 0; j < 3; ++j) cell[j * N1 * PITCH] = o[j];
+    }
   }
-  smem_fft<true, NX, NY, NT, PITCH, 1>(plane, stx);  // along x (rows)
-  // along y (columns), the results leaving for global memory from registers
-  C* out = fld + ((long long)(grp * 3 + rank) * n3 + i3) * NE;
-  smem_fft_io<true, NY, NX, NT, 1, PITCH, false, true>(plane, sty, NoGet{},
-                                                      [&](int i1, int i2, C v) { out[i2 * NX + i1] = v; });
+  __syncthreads();
+  stage_strided<false, N1, N2, LINES, NT, PITCH, 1>(buf, tw);  // along x
+  __syncthreads();
+  stage_group<false, N1, N2, LINES, NT, PITCH, 1>(buf, tw);
+  __syncthreads();
+  // stage A along y over the rows, results to the workspace
+#pragma unroll 1
+  for (int it = threadIdx.x; it < 3 * N; it += NT) {
+    const int j = it / N, x = it % N;
+    E r[N1];
+#pragma unroll
+    for (int k = 0; k < N1; ++k) r[k] = buf[(j * N1 + k) * PITCH + x];
+    edft<N1, true>(r);
+    E* o = fld + (long long)(j * NF + fsel) * n + ((long long)(x / XL) * n3 + i3) * (N2 * XL) + b * XL + x % XL;
+#pragma unroll
+    for (int a = 0; a < N1; ++a) {
+      if (a > 0) r[a] = etwiddle<true>(r[a], tw[a * b]);
+      o[(long long)a * N * n3 * N2] = r[a];
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
-// pass 2: the material product of eq. factor_mtx, per real-space voxel:
-//   w = Phi^{-1} (xi mu^{-1} p + q),   f = mu^{-1} (zeta w + p)
+// k_columns: grid (N / X, N1, 3 P)
 // ---------------------------------------------------------------------------
 
+// The voxel whose fields a column CTA holds at slot (a, b) of y, slot xs of x
+// and slot zs of z (natural index).
+template <int N2>
+__device__ __forceinline__ int slot_index(int s, int N1) { return s / N2 + N1 * (s % N2); }
+
+// Where a column CTA sits, for the per-voxel steps.
+struct ColumnPos {
+  int j, a, xs, zs, prob;  // pair, k1 of y, slot of x, slot of z, problem
+  int x, z;                // natural indices of xs and zs
+  int n1, N1, n3;          // plane edge, its first factor, z length
+  __device__ __forceinline__ long long voxel(int b) const { return ((long long)z * n1 + a + N1 * b) * n1 + x; }
+};
+
+// The material product of a pair at one voxel:
+//   w = 1/Phi (q + i g im p),  f = im (p - i g w),  both times `scale`;
+// returns Re(conj(p) f + conj(q) w) for the CG curvature.
 template <typename R>
-__device__ __forceinline__ void material_apply(const MatView<R>& m, long long v, const cplx<R>* p,
-                                               const cplx<R>* q, cplx<R>* f, cplx<R>* w, R scale) {
-  using C = cplx<R>;
-  R ip[3], im[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    ip[c] = m.inv_phi[c * m.n + v];
-    im[c] = m.inv_mu ? m.inv_mu[c * m.n + v] : (R)1;
-  }
-  if (m.kind == kMediumChiral) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const R g = m.gam[c * m.n + v];
-      // xi mu^{-1} p = i g im p;  w = ip (q + i g im p)
-      const R gi = g * im[c];
-      const C s = mk(q[c].x - gi * p[c].y, q[c].y + gi * p[c].x);
-      const C wc = cscale(s, ip[c]);
-      // zeta w = -i g w;  f = im (p - i g w)
-      const C fc = mk(p[c].x + g * wc.y, p[c].y - g * wc.x);
-      w[c] = cscale(wc, scale);
-      f[c] = cscale(fc, im[c] * scale);
-    }
-  } else {
-    const R g = m.gam[v];
-    const int a = m.ax_a, b = m.ax_b;
-    // partner component of each axis in the coupled pair (-1: uncoupled)
-    C wc[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const int o = c == a ? b : (c == b ? a : -1);
-      C xmp = mk((R)0, (R)0);
-      if (o >= 0) {
-        // (xi mu^{-1} p)_c = i g im_o p_o
-        const C po = pick3<R>(o, p[0], p[1], p[2]);
-        const R imo = o == 0 ? im[0] : (o == 1 ? im[1] : im[2]);
-        xmp = cmul_i(cscale(po, g * imo));
-      }
-      wc[c] = cscale(cadd(q[c], xmp), ip[c]);
-    }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const int o = c == a ? b : (c == b ? a : -1);
-      C zw = mk((R)0, (R)0);
-      if (o >= 0) zw = cmul_mi(cscale(pick3<R>(o, wc[0], wc[1], wc[2]), g));  // (zeta w)_c = -i g w_o
-      w[c] = cscale(wc[c], scale);
-      f[c] = cscale(cadd(p[c], zw), im[c] * scale);
-    }
-  }
+__device__ __forceinline__ R pair_material(R ip, R g, R im, R scale, cplx<R>& p, cplx<R>& q) {
+  const R gi = g * im;
+  const cplx<R> wc = cscale(mk(q.x - gi * p.y, q.y + gi * p.x), ip);
+  const cplx<R> fc = mk(p.x + g * wc.y, p.y - g * wc.x);
+  const cplx<R> w = cscale(wc, scale), f = cscale(fc, im * scale);
+  const R s = p.x * f.x + p.y * f.y + q.x * w.x + q.y * w.y;
+  p = f;
+  q = w;
+  return s;
 }
 
-template <typename R, int N3, int TX, int NT, int MINB>
+// The step of the A_r product: load() fetches the material of the NB voxels
+// from slot b of y on, ahead of its use; apply() forms the product of the voxel
+// at slot b, entry k of the loaded values.
+template <typename R>
+struct ProductStep {
+  static constexpr bool kForward = true;
+  MatView<R> m;
+  R inv_n;
+  long long smat;
+  template <int NB>
+  struct Vals {
+    R ip[NB], g[NB], im[NB];
+  };
+  template <int NB>
+  __device__ __forceinline__ void load(const ColumnPos& c, int b, Vals<NB>& v) const {
+    if constexpr (std::is_same<R, float>::value) {
+      // [j][a][x][b / 2][z]: {1/Phi, g} of b and b + 1
+      const long long at = (((long long)(c.j * c.N1 + c.a) * c.n1 + c.xs) * (NB / 2)) * c.n3 + c.zs;
+      const float4* t = m.pmat + c.prob * smat + at;
+#pragma unroll
+      for (int k = 0; k < NB / 2; ++k) {
+        const float4 w = __ldg(t + (long long)k * c.n3);
+        v.ip[2 * k] = w.x;
+        v.g[2 * k] = w.y;
+        v.ip[2 * k + 1] = w.z;
+        v.g[2 * k + 1] = w.w;
+      }
+      if (m.pmu != nullptr) {
+        const float2* s = m.pmu + c.prob * smat + at;
+#pragma unroll
+        for (int k = 0; k < NB / 2; ++k) {
+          const float2 w = __ldg(s + (long long)k * c.n3);
+          v.im[2 * k] = w.x;
+          v.im[2 * k + 1] = w.y;
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < NB; ++k) v.im[k] = 1.0f;
+      }
+    } else {
+      const int s = pair_axis(m.kind, m.ax_a, m.ax_b, c.j);
+      const bool none = m.kind != kMediumChiral && s == c.j;  // the uncoupled component
+#pragma unroll
+      for (int k = 0; k < NB; ++k) {
+        const long long vox = c.voxel(b + k);
+        v.ip[k] = m.inv_phi[c.prob * smat + c.j * m.n + vox];
+        v.im[k] = m.inv_mu ? m.inv_mu[c.prob * smat + s * m.n + vox] : (R)1;
+        v.g[k] = none ? (R)0 : m.gam[c.prob * smat + (m.kind == kMediumChiral ? c.j * m.n : 0) + vox];
+      }
+    }
+  }
+  template <int NB>
+  __device__ __forceinline__ R apply(const ColumnPos&, int, const Vals<NB>& v, int k, cplx<R>& p, cplx<R>& q) const {
+    return pair_material<R>(v.ip[k], v.g[k], v.im[k], inv_n, p, q);
+  }
+};
+
+template <typename R, int N2, int X, int N3>
+constexpr size_t columns_smem() {
+  return (size_t)(N3 * (ElemOf<R>::NF * N2 * X + 1) + N3 + N2) * 16;
+}
+
+// The plane edge N1 N2 is a run-time value (it only sets strides).
+template <typename R, int N2, int X, int XL, int N3, int NT, int MINB, class Step>
 __global__ void __launch_bounds__(NT, MINB)
-k_pass2_z_material(cplx<R>* __restrict__ fld, MatView<R> mat, const cplx<R>* __restrict__ twz, int ncols,
-                   R inv_n, const int* __restrict__ skip, double* __restrict__ dot_part, BatchStrides bs) {
+k_columns(typename ElemOf<R>::E* __restrict__ fld, Step step, const cplx<R>* __restrict__ twy,
+          const cplx<R>* __restrict__ twz, const int* __restrict__ skip, CGState* st, BatchStrides bs) {
   using C = cplx<R>;
-  constexpr int LINES = 6 * TX;
+  using E = typename ElemOf<R>::E;
+  using S = DepthSplit<R, N3>;
+  constexpr int NF = ElemOf<R>::NF, Z1 = S::N1, Z2 = S::N2;
+  constexpr int L = N2 * X;
+  constexpr int LINES = NF * L;  // line f L + b X + x % X
   constexpr int PITCH = LINES + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* buf = reinterpret_cast<C*>(smem_raw);
-  C* stw = buf + N3 * PITCH;
-  const int tiles = ncols / TX;
-  const int prob = blockIdx.x / tiles;
+  E* buf = reinterpret_cast<E*>(smem_raw);
+  E* tz = buf + N3 * PITCH;
+  E* ty = tz + N3;  // w_N^{a b}, b < N2
+  const int xt = blockIdx.x, a = blockIdx.y, j = blockIdx.z % 3, prob = blockIdx.z / 3;
   if (skip != nullptr && skip[(long long)prob * bs.sskip]) return;
-  fld += prob * bs.sfld;
-  mat.inv_phi += prob * bs.smat;
-  mat.gam += prob * bs.smat;
-  if (mat.inv_mu) mat.inv_mu += prob * bs.smat;
-  for (int i = threadIdx.x; i < N3; i += NT) stw[i] = twz[i];
-  const int col0 = (blockIdx.x % tiles) * TX;
-  const long long n = (long long)ncols * N3;
-  // line l = f * TX + c of the tile is field f, column col0 + c; its element
-  // z lives at fld[f n + z ncols + col0 + c] (consecutive lines, consecutive
-  // addresses within a field)
-  C* tile = fld + col0;
-  auto gaddr = [&](int l, int z) { return tile + (long long)(l / TX) * n + (long long)z * ncols + (l % TX); };
+  const int stop = st != nullptr ? st[prob].stop : 0;
+  for (int i = threadIdx.x; i < N3; i += NT) tz[i] = tw_entry(twz[i]);
+  if (threadIdx.x < N2) ty[threadIdx.x] = tw_entry(twy[a * threadIdx.x]);
+  const int N1 = gridDim.y, N = N1 * N2;
+  const long long n = (long long)N * N * N3;
+  static_assert(XL % X == 0, "a column tile lies within one run of the workspace");
+  E* tile = fld + prob * bs.sfld + (long long)j * NF * n + ((long long)a * N + xt * X / XL * XL) * (N3 * N2) + xt * X % XL;
+  auto gaddr = [&](int l, int z) { return tile + (l / L) * n + z * (N2 * XL) + l % L / X * XL + l % X; };
+  if (stop) return;
   __syncthreads();  // twiddles
-  smem_fft_io<true, N3, LINES, NT, 1, PITCH, true, false>(buf, stw, [&](int l, int z) { return ldg_c(gaddr(l, z)); },
-                                                         NoPut{});
-  // CG curvature from the real-space fields (Parseval; the DFTs carry the
-  // factor n that inv_n removes): u^* A_r u = sum Re(conj(P) f + conj(Q) w)
-  RedAccFor<R> dot_acc;
-  for (int idx = threadIdx.x; idx < N3 * TX; idx += NT) {
-    const int c = idx % TX, z = idx / TX;
-    C* row = buf + z * PITCH + c;
-    C p[3] = {row[0], row[TX], row[2 * TX]};
-    C q[3] = {row[3 * TX], row[4 * TX], row[5 * TX]};
-    C fo[3], wo[3];
-    material_apply<R>(mat, (long long)z * ncols + col0 + c, p, q, fo, wo, inv_n);
-    if (dot_part != nullptr) {
-      R sacc = 0;
+  // inverse stage A along z from the workspace
+  {
+    constexpr int ITEMS = LINES * Z2;
+#pragma unroll 1
+    for (int it = threadIdx.x; it < ITEMS; it += NT) {
+      const int l = it % LINES, n2 = it / LINES;
+      const E* g = gaddr(l, n2);
+      E r[Z1];
 #pragma unroll
-      for (int k = 0; k < 3; ++k)
-        sacc += p[k].x * fo[k].x + p[k].y * fo[k].y + q[k].x * wo[k].x + q[k].y * wo[k].y;
-      dot_acc.add(static_cast<typename RedAccFor<R>::value_type>(sacc));
+      for (int k = 0; k < Z1; ++k) r[k] = g[k * Z2 * (N2 * XL)];
+      edft<Z1, true>(r);
+      E* o = buf + n2 * PITCH + l;
+#pragma unroll
+      for (int k = 0; k < Z1; ++k) o[k * Z2 * PITCH] = (k > 0 && Z2 > 1) ? etwiddle<true>(r[k], tz[n2 * k]) : r[k];
     }
-    row[0] = fo[0];
-    row[TX] = fo[1];
-    row[2 * TX] = fo[2];
-    row[3 * TX] = wo[0];
-    row[4 * TX] = wo[1];
-    row[5 * TX] = wo[2];
   }
-  if (dot_part != nullptr) {
-    const double tot = dot_acc.template block_total<NT>();  // (its barriers also order the material writes)
-    if (threadIdx.x == 0) dot_part[(long long)prob * bs.sstate + blockIdx.x % tiles] = tot;
-  } else {
+  __syncthreads();
+  if constexpr (Z2 > 1) {
+    stage_group<false, Z1, Z2, LINES, NT, 1, PITCH>(buf, tz);
     __syncthreads();
   }
-  smem_fft_io<false, N3, LINES, NT, 1, PITCH, false, true>(buf, stw, NoGet{},
-                                                          [&](int l, int z, C v) { *gaddr(l, z) = v; });
+  // stage B along y, the material step, stage A' along y
+  RedAccFor<R> dot;
+  auto position = [&](int xi, int zs) {
+    return ColumnPos{j,  a, xt * X + xi, zs, prob, slot_index<N2>(xt * X + xi, N1), slot_index<Z2>(zs, Z1), N, N1, N3};
+  };
+  if constexpr (NF == 1) {
+    // all in registers: items (x slot, z slot), the z slot fastest across
+    // threads (odd pitch)
+    constexpr int ITEMS = X * N3;
+#pragma unroll 1
+    for (int it = threadIdx.x; it < ITEMS; it += NT) {
+      const int xi = it / N3, zs = it % N3;
+      const ColumnPos pos = position(xi, zs);
+      typename Step::template Vals<N2> mv;
+      step.template load<N2>(pos, 0, mv);
+      E* cell = buf + zs * PITCH + xi;
+      E v[N2];
+#pragma unroll
+      for (int k = 0; k < N2; ++k) v[k] = cell[k * X];
+      edft<N2, true>(v);
+      R sacc = (R)0;
+#pragma unroll
+      for (int k = 0; k < N2; ++k) {
+        C p, q;
+        get_pair(&v[k], 0, p, q);
+        const R s = step.template apply<N2>(pos, k, mv, k, p, q);
+        if (st != nullptr) sacc = sacc + s;
+        put_pair(&v[k], 0, p, q);
+      }
+      if (st != nullptr) dot.add(static_cast<typename RedAccFor<R>::value_type>(sacc));
+      edft<N2, false>(v);
+#pragma unroll
+      for (int k = 0; k < N2; ++k) cell[k * X] = k > 0 ? etwiddle<false>(v[k], ty[k]) : v[k];
+    }
+  } else {
+    // one step after the other over the tile, each with as many items as it
+    // has: these types are bound by their arithmetic, and a small tile leaves
+    // most lanes of a warp idle when one item does all three (8^3 complex128,
+    // whose 48 CTAs have 8 such items each)
+    constexpr int DITEMS = NF * X * N3;
+#pragma unroll 1
+    for (int it = threadIdx.x; it < DITEMS; it += NT) {
+      E* cell = buf + (it % N3) * PITCH + it / N3 % X + it / (N3 * X) * L;
+      E v[N2];
+#pragma unroll
+      for (int k = 0; k < N2; ++k) v[k] = cell[k * X];
+      edft<N2, true>(v);
+#pragma unroll
+      for (int k = 0; k < N2; ++k) cell[k * X] = v[k];
+    }
+    __syncthreads();
+    constexpr int VITEMS = L * N3;
+#pragma unroll 1
+    for (int it = threadIdx.x; it < VITEMS; it += NT) {
+      const int zs = it % N3, l = it / N3;
+      const ColumnPos pos = position(l % X, zs);
+      typename Step::template Vals<1> mv;
+      step.template load<1>(pos, l / X, mv);
+      E* cell = buf + zs * PITCH + l;
+      C p = cell[0], q = cell[L];
+      const R s = step.template apply<1>(pos, l / X, mv, 0, p, q);
+      if (st != nullptr) dot.add(static_cast<typename RedAccFor<R>::value_type>(s));
+      cell[0] = p;
+      cell[L] = q;
+    }
+    if constexpr (Step::kForward) {
+      __syncthreads();
+#pragma unroll 1
+      for (int it = threadIdx.x; it < DITEMS; it += NT) {
+        E* cell = buf + (it % N3) * PITCH + it / N3 % X + it / (N3 * X) * L;
+        E v[N2];
+#pragma unroll
+        for (int k = 0; k < N2; ++k) v[k] = cell[k * X];
+        edft<N2, false>(v);
+#pragma unroll
+        for (int k = 0; k < N2; ++k) cell[k * X] = k > 0 ? etwiddle<false>(v[k], ty[k]) : v[k];
+      }
+    }
+  }
+  if constexpr (Step::kForward) {
+    if (st != nullptr) {
+      // this CTA's share of p^* A_r p (Parseval: from the real-space fields; the
+      // DFTs carry the factor n that the step removes)
+      const auto tot = dot.template block_total<NT>();
+      if (threadIdx.x == 0)
+        reinterpret_cast<typename RedAccFor<R>::partial*>(st[prob].part_a)[(j * gridDim.y + a) * gridDim.x + xt] = tot;
+      if (NT == 32) __syncthreads();  // (otherwise block_total's barriers order the tile's writes)
+    } else {
+      __syncthreads();
+    }
+    if constexpr (Z2 > 1) {
+      stage_group<true, Z1, Z2, LINES, NT, 1, PITCH>(buf, tz);
+      __syncthreads();
+    }
+    // forward stage B' along z, results to the workspace
+    constexpr int ITEMS = LINES * Z2;
+#pragma unroll 1
+    for (int it = threadIdx.x; it < ITEMS; it += NT) {
+      const int l = it % LINES, n2 = it / LINES;
+      const E* s = buf + n2 * PITCH + l;
+      E r[Z1];
+#pragma unroll
+      for (int k = 0; k < Z1; ++k) r[k] = s[k * Z2 * PITCH];
+      edft<Z1, false>(r);
+      E* g = gaddr(l, n2);
+#pragma unroll
+      for (int k = 0; k < Z1; ++k) g[k * Z2 * (N2 * XL)] = r[k];
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
-// pass 3
+// k_rows_out: grid (N2 NF, n3, P), as k_rows_in
 // ---------------------------------------------------------------------------
-template <typename R, int NX, int NY, int NT, int MINB>
-__global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(NT, MINB)
-k_pass3_fft_xy_project(const cplx<R>* __restrict__ fld, cplx<R>* __restrict__ Au,
-                       const cplx<R>* __restrict__ lam, const cplx<R>* __restrict__ twx,
-                       const cplx<R>* __restrict__ twy, int n3, R alpha, R beta,
-                       const int* __restrict__ skip, const cplx<R>* __restrict__ basis, BatchStrides bs,
-                       CgFuse<R> cg) {
+template <typename R, int N, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB)
+k_rows_out(const typename ElemOf<R>::E* __restrict__ fld, vecc<R>* __restrict__ Au, const cplx<R>* __restrict__ lam,
+           const cplx<R>* __restrict__ twx, R alpha, R beta, int kind, int ax_a, int ax_b,
+           const int* __restrict__ skip, const cplx<R>* __restrict__ basis, BatchStrides bs, CgFuse<R> cg) {
   using C = cplx<R>;
-  constexpr int PITCH = NX + 1;
-  constexpr int NE = NX * NY;
-  constexpr int EPV = Lane<C>::EPV;
+  using E = typename ElemOf<R>::E;
+  using S = PlaneSplit<R, N>;
+  constexpr int NF = ElemOf<R>::NF, N1 = S::N1, N2 = S::N2, X = S::X, XL = S::XL;
+  constexpr int PITCH = N + 1;
+  constexpr int LINES = 3 * N1;
+  constexpr int NV = N1 * N;
+  static_assert(3 * N1 * (N / X) <= kMaxPartials, "one partial of p^* A p per CTA of k_columns");
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* plane = reinterpret_cast<C*>(smem_raw);
-  C* stx = plane + NY * PITCH;
-  C* sty = stx + NX;
-  cg::cluster_group cl = cg::this_cluster();
-  const int prob = blockIdx.z / n3;
+  E* buf = reinterpret_cast<E*>(smem_raw);
+  E* tw = buf + LINES * PITCH;
+  const int b = blockIdx.x % N2, fsel = blockIdx.x / N2, i3 = blockIdx.y, prob = blockIdx.z, n3 = gridDim.y;
   if (skip != nullptr && skip[(long long)prob * bs.sskip]) return;
-  const int rank = (int)cl.block_rank();
-  const int grp = blockIdx.y;
-  const int i3 = blockIdx.z % n3;
+  constexpr bool CGT = !std::is_same<R, df>::value;  // (the double-single product never runs CG)
+  CGState* st = (CGT && cg.st != nullptr) ? cg.st + prob : nullptr;
+  const bool first = blockIdx.x == 0 && i3 == 0 && threadIdx.x == 0;
+  const long long n = (long long)N * N * n3;
+  constexpr int NQ = 4 / NF;  // quarters of the result that this CTA forms, from q0 on
+  const int q0 = NF == 1 ? 0 : 2 * fsel;
+  int stop = 0;
+  RedAccFor<R> pap_acc;
+  if constexpr (CGT) {
+    if (st != nullptr) {
+      stop = st->stop;
+      cg.x += prob * bs.su + q0 * n;
+      cg.r += prob * bs.su + q0 * n;
+      cg.p += prob * bs.su + q0 * n;
+      // the CG vectors of this CTA's rows do not all stay in L2 between two
+      // steps at 96^3: fetch them there while the transforms run
+      constexpr int LINE = 128 / (int)sizeof(C);  // elements of a cache line
+      constexpr int PER = (N + LINE - 1) / LINE;  // lines of a row
+      for (int i = threadIdx.x; i < NQ * N1 * PER; i += NT) {
+        const int q = i / (N1 * PER), row = i / PER % N1, l = i % PER;
+        const long long e = q * n + ((long long)i3 * N + b + N2 * row) * N + l * LINE;
+        prefetch_l2(cg.p + e);
+        prefetch_l2(cg.r + e);
+        prefetch_l2(cg.x + e);
+      }
+      const auto* pa = reinterpret_cast<const typename RedAccFor<R>::partial*>(st->part_a);
+#pragma unroll 2
+      for (int i = threadIdx.x; i < 3 * N1 * (N / X); i += NT) pap_acc.add_partial(pa[i]);
+    }
+  }
   fld += prob * bs.sfld;
   Au += prob * bs.su;
   lam += (long long)prob * bs.slam;
   if (basis != nullptr) basis += prob * bs.sbasis;
-  for (int i = threadIdx.x; i < NX; i += NT) stx[i] = twx[i];
-  for (int i = threadIdx.x; i < NY; i += NT) sty[i] = twy[i];
-  const C* in = fld + ((long long)(grp * 3 + rank) * n3 + i3) * NE;
-  // fused CG step: alpha from pass 2's partials of p^* A p, summed in the same
-  // fixed order by every CTA (so all agree); no state is written until the
-  // last CTA of the launch (the `done` flag every CTA reads at its start must
-  // not change while the launch runs)
-  __shared__ double s_cg_alpha;
-  __shared__ int s_cg_ok, s_cg_last;
-  // (only complex64 and complex128 run CG; the double-single product never does)
-  constexpr bool CGT = std::is_same<R, float>::value || std::is_same<R, double>::value;
-  CGState* cst = (CGT && cg.st != nullptr) ? cg.st + prob : nullptr;
-  if (cst != nullptr) {
-    RedAccFor<R> pa;
-    for (int i = threadIdx.x; i < cst->npart_a; i += NT) pa.add_double(cst->part_a[i]);
-    const double pAp = pa.template block_total<NT>();
-    if (threadIdx.x == 0) {
-      s_cg_alpha = cst->rr / pAp;
-      s_cg_ok = (pAp > 0.0) && (s_cg_alpha == s_cg_alpha);  // also catches NaN
-      if (blockIdx.x == 0 && blockIdx.y == 0 && i3 == 0) {
-        cst->pAp = pAp;
-        cst->alpha = s_cg_alpha;
-      }
-    }
-  }
-  __syncthreads();  // twiddles (and alpha)
-  // the 2-D DFT along y first (columns, read from global memory straight into
-  // registers), then along x
-  smem_fft_io<false, NY, NX, NT, 1, PITCH, true, false>(plane, sty,
-                                                       [&](int i1, int i2) { return ldg_c(in + i2 * NX + i1); }, NoPut{});
-  smem_fft<false, NX, NY, NT, PITCH, 1>(plane, stx);
-  cl.sync();
-  const C* src0 = cl.map_shared_rank(plane, 0);
-  const C* src1 = cl.map_shared_rank(plane, 1);
-  const C* src2 = cl.map_shared_rank(plane, 2);
-  const long long n = (long long)NE * n3;
-  C* o0 = Au + (2 * grp) * n + (long long)i3 * NE;
-  C* o1 = o0 + n;
-  const C a3 = lam[NX + NY + i3];
-  const int e0 = third_bound<NE>(rank), e1 = third_bound<NE>(rank + 1);
-  using V = typename Lane<C>::V;
-  V* o0v = reinterpret_cast<V*>(o0);
-  V* o1v = reinterpret_cast<V*>(o1);
-  const bool cg_on = cst != nullptr;
-  const bool cg_upd = cg_on && s_cg_ok;
-  const R cg_al = cg_on ? (R)s_cg_alpha : (R)0;
-  const long long cg_off = prob * bs.su + (2 * grp) * n + (long long)i3 * NE;
-  RedAccFor<R> cg_acc;
-  // EPV consecutive elements per lane (e0, e1 even)
-  for (int ev = e0 / EPV + (int)threadIdx.x; ev < e1 / EPV; ev += NT) {
-    C r0[EPV], r1[EPV];
+  for (int i = threadIdx.x; i < N; i += NT) tw[i] = tw_entry(twx[i]);
+  // stage B' along y from the workspace: row k of the CTA is y = b + N2 k
+#pragma unroll 1
+  for (int it = threadIdx.x; it < 3 * N; it += NT) {
+    const int j = it / N, x = it % N;
+    const E* g = fld + (long long)(j * NF + fsel) * n + ((long long)(x / XL) * n3 + i3) * (N2 * XL) + b * XL + x % XL;
+    E r[N1];
 #pragma unroll
-    for (int h = 0; h < EPV; ++h) {
-      const int e = ev * EPV + h;
-      const int i1 = e % NX, i2 = e / NX;
-      const int s = i2 * PITCH + i1;
-      const C f[3] = {src0[s], src1[s], src2[s]};
-      Basis<R> B;
-      voxel_basis<R>(basis, n, (long long)i3 * NE + e, lam[i1], lam[NX + i2], a3, alpha, beta, B);
-      if (grp == 0) {
-        // P_r^* f = [-sum conj(c) f ; sum conj(x) f]
-        r0[h] = cneg(cadd(cadd(cmulc(B.c[0], f[0]), cmulc(B.c[1], f[1])), cmulc(B.c[2], f[2])));
-        r1[h] = cadd(cadd(cmulc(B.x[0], f[0]), cmulc(B.x[1], f[1])), cmulc(B.x[2], f[2]));
-      } else {
-        // Q_r^* w = [sum x w ; sum c w]
-        r0[h] = cadd(cadd(cmul(B.x[0], f[0]), cmul(B.x[1], f[1])), cmul(B.x[2], f[2]));
-        r1[h] = cadd(cadd(cmul(B.c[0], f[0]), cmul(B.c[1], f[1])), cmul(B.c[2], f[2]));
-      }
-    }
-    if (cg_on) {
-      // x += alpha p, r -= alpha A_r p (this CTA's third of its two quarters)
-      if constexpr (CGT) if (cg_upd) {
+    for (int a = 0; a < N1; ++a) r[a] = g[(long long)a * N * n3 * N2];
+    edft<N1, false>(r);
 #pragma unroll
-        for (int h = 0; h < EPV; ++h) {
-          const long long i0 = cg_off + ev * EPV + h, i1 = i0 + n;
-          const C pa = cg.p[i0], pb = cg.p[i1];
-          C xa = cg.x[i0], xb = cg.x[i1], ra = cg.r[i0], rb = cg.r[i1];
-          xa = mk(xa.x + cg_al * pa.x, xa.y + cg_al * pa.y);
-          xb = mk(xb.x + cg_al * pb.x, xb.y + cg_al * pb.y);
-          ra = mk(ra.x - cg_al * r0[h].x, ra.y - cg_al * r0[h].y);
-          rb = mk(rb.x - cg_al * r1[h].x, rb.y - cg_al * r1[h].y);
-          cg.x[i0] = xa;
-          cg.x[i1] = xb;
-          cg.r[i0] = ra;
-          cg.r[i1] = rb;
-          cg_acc.add(static_cast<typename RedAccFor<R>::value_type>(ra.x * ra.x + ra.y * ra.y + rb.x * rb.x +
-                                                                   rb.y * rb.y));
-        }
-      }
-    } else if constexpr (EPV == 2) {
-      o0v[ev] = make_float4(r0[0].x, r0[0].y, r0[1].x, r0[1].y);
-      o1v[ev] = make_float4(r1[0].x, r1[0].y, r1[1].x, r1[1].y);
-    } else {
-      o0v[ev] = r0[0];
-      o1v[ev] = r1[0];
-    }
+    for (int k = 0; k < N1; ++k) buf[(j * N1 + k) * PITCH + x] = r[k];
   }
-  if (cg_on) {
-    // this CTA's partial of the new r^* r; the last CTA to arrive (atomic
-    // count, no waiting) sums them in fixed order and sets beta, the
-    // iteration count and the convergence state for the next launch
-    const int ncta = 6 * n3;
-    const int cta = rank + 3 * (grp + 2 * i3);
-    const double part = cg_acc.template block_total<NT>();
-    if (threadIdx.x == 0) {
-      cst->part_b[cta] = part;
-      __threadfence();
-      s_cg_last = atomicAdd(&cst->arrived, 1u) == (unsigned)ncta - 1;
-    }
-    __syncthreads();
-    if (s_cg_last) {
-      __threadfence();
-      RedAccFor<R> rb_acc;
-      for (int i = threadIdx.x; i < ncta; i += NT) rb_acc.add_double(((volatile double*)cst->part_b)[i]);
-      const double rr = rb_acc.template block_total<NT>();
-      if (threadIdx.x == 0) {
-        cst->arrived = 0;
-        if (!s_cg_ok) {
-          cst->status = -7;  // breakdown: x, r left untouched
-          cst->done = 1;
+  if (stop) {
+    if (first) st->halt = 1;
+    return;
+  }
+  __syncthreads();
+  stage_group<true, N1, N2, LINES, NT, PITCH, 1>(buf, tw);  // along x
+  __syncthreads();
+  stage_strided<true, N1, N2, LINES, NT, PITCH, 1>(buf, tw);
+  R cg_al = (R)0;
+  bool ok = false;
+  if constexpr (CGT) {
+    if (st != nullptr) {
+      using P = typename RedAccFor<R>::partial;
+      const P pAp = pap_acc.template block_total<NT>();
+      const P rr = *reinterpret_cast<const P*>(&st->rr_now);
+      cg_al = (R)scalar_ratio(rr, pAp);
+      ok = scalar_positive(pAp) && cg_al == cg_al;  // also catches NaN
+      if (first) {
+        if (ok) {
+          st->it += 1;
+          *reinterpret_cast<P*>(&st->rr_last) = rr;
         } else {
-          cst->it += 1;
-          if (!(rr == rr)) {
-            cst->status = -7;
-            cst->done = 1;
-          } else if (rr <= cst->tol2) {
-            cst->done = 1;
-          } else if (cst->it >= cst->maxit) {
-            cst->status = -6;
-            cst->done = 1;
-          }
-          cst->beta = rr / cst->rr;
-          cst->rr = rr;
+          st->broken = st->halt = 1;  // breakdown: x, r left untouched
+        }
+      }
+      if (!ok) return;
+    }
+  }
+  __syncthreads();
+  RedAccFor<R> rr_acc;
+  const C a3 = lam[2 * N + i3];
+#pragma unroll 1
+  for (int vi = threadIdx.x; vi < NV; vi += NT) {
+    const int row = vi / N, x = vi % N, y = b + N2 * row;
+    const long long e = ((long long)i3 * N + y) * N + x;
+    vecc<R> pv[NQ], xv[NQ], rv[NQ];
+    if constexpr (CGT) {
+      if (ok) {
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+          pv[q] = cg.p[e + q * n];
+          rv[q] = cg.r[e + q * n];
+          xv[q] = cg.x[e + q * n];
         }
       }
     }
+    Basis<R> B;
+    voxel_basis<R>(basis, n, e, lam[x], lam[N + y], a3, alpha, beta, B);
+    // P_r^* f = [-sum conj(c) f ; sum conj(x) f],  Q_r^* w = [sum x w ; sum c w]
+    const E* cell = buf + row * PITCH + x;
+    C o[NQ];
+    C f[3], w[3];
+    if constexpr (NF == 1) {
+#pragma unroll
+      for (int j = 0; j < 3; ++j) get_pair(cell + j * N1 * PITCH, 0, f[j], w[j]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 3; ++j) f[j] = w[j] = cell[j * N1 * PITCH];
+    }
+    if (NF == 1 || fsel == 0) {
+      if (kind != kMediumChiral) swap_axes(f, ax_a, ax_b);
+      o[0] = cneg(cadd(cadd(cmulc(B.c[0], f[0]), cmulc(B.c[1], f[1])), cmulc(B.c[2], f[2])));
+      o[1] = cadd(cadd(cmulc(B.x[0], f[0]), cmulc(B.x[1], f[1])), cmulc(B.x[2], f[2]));
+    }
+    if (NF == 1 || fsel == 1) {
+      o[NQ - 2] = cadd(cadd(cmul(B.x[0], w[0]), cmul(B.x[1], w[1])), cmul(B.x[2], w[2]));
+      o[NQ - 1] = cadd(cadd(cmul(B.c[0], w[0]), cmul(B.c[1], w[1])), cmul(B.c[2], w[2]));
+    }
+    if (ok) {
+      if constexpr (CGT) {
+        R s = (R)0;
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+          xv[q] = mk(xv[q].x + cg_al * pv[q].x, xv[q].y + cg_al * pv[q].y);
+          rv[q] = mk(rv[q].x - cg_al * o[q].x, rv[q].y - cg_al * o[q].y);
+          cg.x[e + q * n] = xv[q];
+          cg.r[e + q * n] = rv[q];
+          s += rv[q].x * rv[q].x + rv[q].y * rv[q].y;
+        }
+        rr_acc.add(s);
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) Au[(q0 + q) * n + e] = to_vec<R>(o[q]);
+    }
   }
-  cl.sync();  // keep this CTA's plane alive until the cluster finished reading it
+  if constexpr (CGT) {
+    if (st != nullptr) {
+      const auto part = rr_acc.template block_total<NT>();
+      if (threadIdx.x == 0) reinterpret_cast<typename RedAccFor<R>::partial*>(st->part_b)[i3 * gridDim.x + blockIdx.x] = part;
+    }
+  }
 }
 
 }  // namespace nfs

@@ -42,7 +42,7 @@ using nfs::kRedThreads;
 
 namespace {
 struct GraphEntry {
-  const void* key[5];
+  const void* key[4];
   cudaGraphExec_t exec;
 };
 // A batch of GMRES steps as a replayable graph: steps j0 .. j0 + nsteps - 1
@@ -77,7 +77,8 @@ struct nfs_ctx {
   float2* tw32[3] = {nullptr, nullptr, nullptr};
   // material, per problem (stride mat_len): inv_phi [3n] | gam [3n or n] | inv_mu [3n]
   double* mat64 = nullptr;
-  float* mat32 = nullptr;
+  float4* pmat = nullptr;  // complex64 order of the material (mixed contexts and products; stride 3n / 2)
+  float2* pmu = nullptr;
   double2* basis64 = nullptr;  // per problem [6][n]: c and x of every voxel (complex128 products)
   // Bloch twist of T (eq. mtx_T), per problem (stride nl): the diagonals
   // D_l[j] = exp(i 2 pi k.a_l j / n_l), l = 1, 2, 3; and k.a_l itself
@@ -102,7 +103,6 @@ struct nfs_ctx {
   void* fld = nullptr;  // 6n complex128 each (complex64 uses 12n entries of it)
   double2 *x64 = nullptr, *r64 = nullptr, *p64 = nullptr, *Ap64 = nullptr, *t64 = nullptr, *t64b = nullptr;
   float2 *x32 = nullptr, *r32 = nullptr, *p32 = nullptr, *Ap32 = nullptr;
-  float2* p32b = nullptr;  // second CG direction buffer when pass 1 cannot update in place
   CGState* st = nullptr;
   CGState* st_host = nullptr;  // pinned mirror of the scalar part
   // small per-problem arrays (device + pinned host): tolerances, scales, flags
@@ -206,23 +206,21 @@ nfs::BatchStrides strides(const nfs_ctx* c, long long sfld) {
   b.su = c->N;
   b.sfld = sfld;
   b.smat = c->mat_len;
-  b.sstate = nfs::kStateDoubles;
   b.slam = c->nl;
-  b.sskip = nfs::kStateInts;
   return b;
 }
 
 template <typename R>
-nfs::MatvecArgs<R> margs(nfs_ctx* c, const nfs::cplx<R>* u, nfs::cplx<R>* Au, const int* skip);
+nfs::MatvecArgs<R> margs(nfs_ctx* c, const nfs::vecc<R>* u, nfs::vecc<R>* Au, const int* skip);
 
 template <>
 nfs::MatvecArgs<double> margs<double>(nfs_ctx* c, const double2* u, double2* Au, const int* skip) {
   nfs::MatvecArgs<double> a{};
-  a.u = u; a.Au = Au; a.fld = (double2*)c->fld; a.lam = c->lam64;
-  a.tw1 = c->tw64[0]; a.tw2 = c->tw64[1]; a.tw3 = c->tw64[2];
+  a.u = u; a.Au = Au; a.fld = c->fld; a.lam = c->lam64;
+  a.tw1 = c->tw64[0]; a.tw3 = c->tw64[2];
   a.inv_phi = c->mat64; a.gam = c->mat64 + 3 * c->n; a.inv_mu = c->has_mu ? c->mat64 + 3 * c->n + c->gam_len : nullptr;
   a.kind = c->kind; a.ax_a = c->ax_a; a.ax_b = c->ax_b;
-  a.n1 = c->n1; a.n2 = c->n2; a.n3 = c->n3; a.alpha = c->opt.alpha; a.beta = c->opt.beta;
+  a.n1 = c->n1; a.n3 = c->n3; a.alpha = c->opt.alpha; a.beta = c->opt.beta;
   a.skip = skip; a.stream = c->stream;
   a.basis = c->basis64;
   a.P = c->P;
@@ -234,25 +232,26 @@ nfs::MatvecArgs<double> margs<double>(nfs_ctx* c, const double2* u, double2* Au,
 template <>
 nfs::MatvecArgs<float> margs<float>(nfs_ctx* c, const float2* u, float2* Au, const int* skip) {
   nfs::MatvecArgs<float> a{};
-  a.u = u; a.Au = Au; a.fld = (float2*)c->fld; a.lam = c->lam32;
-  a.tw1 = c->tw32[0]; a.tw2 = c->tw32[1]; a.tw3 = c->tw32[2];
-  a.inv_phi = c->mat32; a.gam = c->mat32 + 3 * c->n; a.inv_mu = c->has_mu ? c->mat32 + 3 * c->n + c->gam_len : nullptr;
+  a.u = u; a.Au = Au; a.fld = c->fld; a.lam = c->lam32;
+  a.tw1 = c->tw32[0]; a.tw3 = c->tw32[2];
+  a.pmat = c->pmat; a.pmu = c->pmu;
   a.kind = c->kind; a.ax_a = c->ax_a; a.ax_b = c->ax_b;
-  a.n1 = c->n1; a.n2 = c->n2; a.n3 = c->n3; a.alpha = (float)c->opt.alpha; a.beta = (float)c->opt.beta;
+  a.n1 = c->n1; a.n3 = c->n3; a.alpha = (float)c->opt.alpha; a.beta = (float)c->opt.beta;
   a.skip = skip; a.stream = c->stream;
   a.P = c->P;
-  a.bs = strides(c, 12 * c->n);  // the complex128-sized workspace holds 12 n complex64 per problem
+  a.bs = strides(c, 3 * c->n);  // a workspace element holds two complex64 numbers
+  a.bs.smat = 3 * c->n / 2;
   return a;
 }
 
 template <>
-nfs::MatvecArgs<nfs::df> margs<nfs::df>(nfs_ctx* c, const nfs::dfc* u, nfs::dfc* Au, const int* skip) {
+nfs::MatvecArgs<nfs::df> margs<nfs::df>(nfs_ctx* c, const double2* u, double2* Au, const int* skip) {
   nfs::MatvecArgs<nfs::df> a{};
-  a.u = u; a.Au = Au; a.fld = (nfs::dfc*)c->fld; a.lam = c->lamdf;
-  a.tw1 = c->twdf[0]; a.tw2 = c->twdf[1]; a.tw3 = c->twdf[2];
+  a.u = u; a.Au = Au; a.fld = c->fld; a.lam = c->lamdf;
+  a.tw1 = c->twdf[0]; a.tw3 = c->twdf[2];
   a.inv_phi = c->matdf; a.gam = c->matdf + 3 * c->n; a.inv_mu = c->has_mu ? c->matdf + 3 * c->n + c->gam_len : nullptr;
   a.kind = c->kind; a.ax_a = c->ax_a; a.ax_b = c->ax_b;
-  a.n1 = c->n1; a.n2 = c->n2; a.n3 = c->n3; a.alpha = nfs::df(c->opt.alpha); a.beta = nfs::df(c->opt.beta);
+  a.n1 = c->n1; a.n3 = c->n3; a.alpha = nfs::df(c->opt.alpha); a.beta = nfs::df(c->opt.beta);
   a.skip = skip; a.stream = c->stream;
   a.basis = c->basisdf;
   a.P = c->P;
@@ -264,29 +263,15 @@ nfs::MatvecArgs<nfs::df> margs<nfs::df>(nfs_ctx* c, const nfs::dfc* u, nfs::dfc*
 // P products (problem p's vectors at u + p N); skip (optional): problem p is
 // skipped when skip[p * sskip] is nonzero.
 template <typename R>
-int matvec(nfs_ctx* c, cudaStream_t s, const nfs::cplx<R>* u, nfs::cplx<R>* Au, const int* skip = nullptr,
+int matvec(nfs_ctx* c, cudaStream_t s, const nfs::vecc<R>* u, nfs::vecc<R>* Au, const int* skip = nullptr,
            int sskip = 0) {
   nfs::MatvecArgs<R> a = margs<R>(c, u, Au, skip);
   a.stream = s;
   a.bs.sskip = sskip;
   cudaError_t e = nfs::matvec_launch<R>(a);
   if (e != cudaSuccess) return cuda_fail(e, "matvec launch");
-  c->launches += nfs::product_kernels<R>(c->n1);
-  if (sizeof(nfs::cplx<R>) == 8) c->mv32 += c->P; else c->mv64 += c->P;
-  return NFS_OK;
-}
-
-// FP64-accuracy products of complex128 vectors through the double-single
-// product (mixed contexts): u is converted into the free CG direction buffer
-// p64, the result is written into out and converted there in place.
-int matvec_refine(nfs_ctx* c, cudaStream_t s, const double2* u, double2* out, const int* skip, int sskip) {
-  const long long reals = 2 * c->P * c->N;
-  nfs::dfc* uin = reinterpret_cast<nfs::dfc*>(c->p64);
-  nfs::dfc* res = reinterpret_cast<nfs::dfc*>(out);
-  CK(nfs::double_to_df(reinterpret_cast<const double*>(u), reinterpret_cast<nfs::df*>(uin), reals, s));
-  TRY(matvec<nfs::df>(c, s, uin, res, skip, sskip));
-  CK(nfs::df_to_double(reinterpret_cast<const nfs::df*>(res), reinterpret_cast<double*>(out), reals, s));
-  c->launches += 2;
+  c->launches += nfs::kProductKernels;
+  if (sizeof(R) == 4) c->mv32 += c->P; else c->mv64 += c->P;
   return NFS_OK;
 }
 
@@ -329,7 +314,7 @@ int red_blocks(long long N, int P) {
 template <typename C>
 int dots_re(nfs_ctx* c, cudaStream_t s, const C* x, const C* y, std::vector<double>& out) {
   const int nb = red_blocks(c->N, c->P);
-  nfs::k_dot_re<C><<<dim3(nb, c->P), kRedThreads, 0, s>>>(x, y, c->N, c->dscratch, nb, nullptr, 0);
+  nfs::k_dot_re<C><<<dim3(nb, c->P), kRedThreads, 0, s>>>(x, y, c->N, c->dscratch, nb);
   CK(cudaGetLastError());
   c->launches += 1;
   CK(cudaMemcpyAsync(c->hscratch, c->dscratch, (size_t)nb * c->P * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -371,66 +356,38 @@ int put_flags(nfs_ctx* c, cudaStream_t s, int off, const std::vector<int>& v) {
 #endif
 constexpr int kCgChunk = NFS_CG_CHUNK;
 
-// Enqueue kCgChunk iterations for all problems: pass 1 (which first forms
-// p = r + beta p), passes 2 and 3 (pass 2 also emits the p^* A p partials,
-// from the real-space fields) and the x/r update (which forms alpha, and in
-// its last block beta).
+// Enqueue kCgChunk iterations for all problems, three kernels each (see
+// CgFuse), and the check that sets the state for the host.
 template <typename R>
-cudaError_t enqueue_cg_chunk(nfs_ctx* c, cudaStream_t s, nfs::cplx<R>* x, nfs::cplx<R>* r, nfs::cplx<R>* p,
-                             nfs::cplx<R>* Ap) {
-  using C = nfs::cplx<R>;
-  nfs::MatvecArgs<R> a = margs<R>(c, p, Ap, &c->st->done);
+cudaError_t enqueue_cg_chunk(nfs_ctx* c, cudaStream_t s, nfs::cplx<R>* x, nfs::cplx<R>* r, nfs::cplx<R>* p) {
+  nfs::MatvecArgs<R> a = margs<R>(c, nullptr, nullptr, nullptr);
   a.stream = s;
-  a.cg_r = r;
-  a.cg_beta = &c->st->beta;
-  a.dot_part = c->st->part_a;
-  // kernels that cannot form p = r + beta p in place alternate between p and
-  // a second buffer (kCgChunk is even: p holds the direction after a chunk)
-  C* p2 = nullptr;
-  if (sizeof(R) == 4 && nfs::cg_needs_p_out<R>(c->n1)) p2 = reinterpret_cast<C*>(c->p32b);
-  static_assert(kCgChunk % 2 == 0, "the direction must end a chunk in p");
-  // where pass 3 can take the x/r step itself, no update kernel runs and A p
-  // is never stored
-  const bool fused = nfs::cg_fusable<R>(c->n1);
+  a.cg.x = x;
+  a.cg.r = r;
+  a.cg.p = p;
+  a.cg.st = c->st;
   for (int i = 0; i < kCgChunk; ++i) {
-    C* pn = p;
-    if (p2 != nullptr) {
-      a.u = (i % 2 == 0) ? p : p2;
-      pn = (i % 2 == 0) ? p2 : p;
-      a.p_out = pn;
-    }
-    if (fused) {
-      a.cg.x = x;
-      a.cg.r = r;
-      a.cg.p = pn;
-      a.cg.st = c->st;
-    }
     cudaError_t e = nfs::matvec_launch<R>(a);
     if (e != cudaSuccess) return e;
-    if (!fused) {
-      nfs::k_cg_update_xr<C><<<dim3(nfs::kUpdBlocks, c->P), nfs::kUpdThreads, 0, s>>>(x, r, pn, Ap, c->N, c->st);
-      e = cudaGetLastError();
-      if (e != cudaSuccess) return e;
-    }
   }
-  return cudaSuccess;
+  nfs::k_cg_check<R><<<c->P, kRedThreads, 0, s>>>(c->st, nfs::cg_partials<R>(c->n1, c->n3));
+  return cudaGetLastError();
 }
 
 // The chunk as a CUDA graph, captured once per (precision, buffers) on the
 // context's work stream and replayed: one launch per chunk instead of
-// 4 kCgChunk kernel launches.
+// 3 kCgChunk kernel launches.
 template <typename R>
-int cg_chunk_graph(nfs_ctx* c, nfs::cplx<R>* x, nfs::cplx<R>* r, nfs::cplx<R>* p, nfs::cplx<R>* Ap,
-                   cudaGraphExec_t* out) {
-  const void* key[5] = {x, r, p, Ap, (const void*)(uintptr_t)sizeof(R)};
+int cg_chunk_graph(nfs_ctx* c, nfs::cplx<R>* x, nfs::cplx<R>* r, nfs::cplx<R>* p, cudaGraphExec_t* out) {
+  const void* key[4] = {x, r, p, (const void*)(uintptr_t)sizeof(R)};
   for (const GraphEntry& g : c->graphs)
-    if (std::equal(key, key + 5, g.key)) {
+    if (std::equal(key, key + 4, g.key)) {
       *out = g.exec;
       return NFS_OK;
     }
   cudaGraph_t graph = nullptr;
   CK(cudaStreamBeginCapture(c->work, cudaStreamCaptureModeThreadLocal));
-  cudaError_t e = enqueue_cg_chunk<R>(c, c->work, x, r, p, Ap);
+  cudaError_t e = enqueue_cg_chunk<R>(c, c->work, x, r, p);
   cudaError_t e2 = cudaStreamEndCapture(c->work, &graph);
   if (e != cudaSuccess) {
     if (graph) cudaGraphDestroy(graph);
@@ -442,7 +399,7 @@ int cg_chunk_graph(nfs_ctx* c, nfs::cplx<R>* x, nfs::cplx<R>* r, nfs::cplx<R>* p
   cudaGraphDestroy(graph);
   if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate");
   GraphEntry g;
-  std::copy(key, key + 5, g.key);
+  std::copy(key, key + 4, g.key);
   g.exec = exec;
   c->graphs.push_back(g);
   *out = exec;
@@ -455,26 +412,25 @@ int cg_chunk_graph(nfs_ctx* c, nfs::cplx<R>* x, nfs::cplx<R>* r, nfs::cplx<R>* p
 // its problem's device `done` flag is set, and the host reads the flags
 // between chunks.
 template <typename R>
-int cg_run(nfs_ctx* c, nfs::cplx<R>* x, nfs::cplx<R>* r, nfs::cplx<R>* p, nfs::cplx<R>* Ap,
-           const std::vector<double>& tol2, int maxit, std::vector<int>& iters, std::vector<int>& status) {
+int cg_run(nfs_ctx* c, nfs::cplx<R>* x, nfs::cplx<R>* r, nfs::cplx<R>* p, const std::vector<double>& tol2, int maxit,
+           std::vector<int>& iters, std::vector<int>& status) {
   using C = nfs::cplx<R>;
   cudaStream_t s = c->work;
   CK(cudaStreamSynchronize(s));  // earlier work is not the loop's
   const double t0 = now_s();
   CK(cudaMemsetAsync(p, 0, c->P * c->N * sizeof(C), s));  // with beta = 0 the first pass 1 sets p = r
   const int nb = red_blocks(c->N, c->P);
-  nfs::k_dot_re<C><<<dim3(nb, c->P), kRedThreads, 0, s>>>(r, r, c->N, c->st->part_a, nfs::kStateDoubles, nullptr, 0);
+  nfs::k_dot_re<C><<<dim3(nb, c->P), kRedThreads, 0, s>>>(r, r, c->N, c->st->part_a, nfs::kStateDoubles);
   TRY(put_small(c, s, 0, tol2));
-  nfs::k_cg_init<<<c->P, kRedThreads, 0, s>>>(c->st, c->d_small, maxit,
-                                               nfs::matvec_dot_partials<R>(c->n1, c->n2, c->n3), nb);
+  nfs::k_cg_init<R><<<c->P, kRedThreads, 0, s>>>(c->st, c->d_small, maxit, nb, nfs::cg_partials<R>(c->n1, c->n3));
   CK(cudaGetLastError());
   c->launches += 2;
   cudaGraphExec_t exec = nullptr;
-  TRY(cg_chunk_graph<R>(c, x, r, p, Ap, &exec));
+  TRY(cg_chunk_graph<R>(c, x, r, p, &exec));
   const size_t head = offsetof(CGState, part_a);
   for (;;) {
     CK(cudaGraphLaunch(exec, s));
-    c->launches += (nfs::product_kernels<R>(c->n1) + (nfs::cg_fusable<R>(c->n1) ? 0 : 1)) * kCgChunk;
+    c->launches += nfs::kProductKernels * kCgChunk + 1;
     CK(cudaMemcpy2DAsync(c->st_host, sizeof(CGState), c->st, sizeof(CGState), head, c->P, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     bool all = true;
@@ -534,7 +490,7 @@ int solve(nfs_ctx* c, const double2* b, double2* x, bool x_zero, const std::vect
     std::vector<double> tol2(P);
     for (int q = 0; q < P; ++q) tol2[q] = need[q] ? tol * tol * bb[q] : INFINITY;
     std::vector<int> it, st;
-    TRY(cg_run<double>(c, x, c->r64, c->p64, c->Ap64, tol2, c->opt.cg_maxit, it, st));
+    TRY(cg_run<double>(c, x, c->r64, c->p64, tol2, c->opt.cg_maxit, it, st));
     for (int q = 0; q < P; ++q) {
       if (!need[q]) continue;
       so.iters[q] = it[q];
@@ -588,7 +544,7 @@ int solve(nfs_ctx* c, const double2* b, double2* x, bool x_zero, const std::vect
     c->launches += 1;
     CK(cudaMemsetAsync(c->x32, 0, tot * sizeof(float2), s));
     std::vector<int> it, st;
-    TRY(cg_run<float>(c, c->x32, c->r32, c->p32, c->Ap32, itol2, c->opt.cg_maxit, it, st));
+    TRY(cg_run<float>(c, c->x32, c->r32, c->p32, itol2, c->opt.cg_maxit, it, st));
     TRY(put_small(c, s, 2 * P, nrm));
     nfs::k_axpy_promote<<<nb, 256, 0, s>>>(x, c->d_small + 2 * P, c->x32, c->N, tot);
     CK(cudaGetLastError());
@@ -596,7 +552,7 @@ int solve(nfs_ctx* c, const double2* b, double2* x, bool x_zero, const std::vect
     // next residual: complex128 product of x, or complex64 product of d
     TRY(put_flags(c, s, 2 * P, skip64));
     TRY(put_flags(c, s, 3 * P, skip32));
-    if (any64) TRY(matvec_refine(c, s, x, c->Ap64, c->d_flags + 2 * P, 1));
+    if (any64) TRY(matvec<nfs::df>(c, s, x, c->Ap64, c->d_flags + 2 * P, 1));
     if (any32) TRY(matvec<float>(c, s, c->x32, c->Ap32, c->d_flags + 3 * P, 1));
     nfs::k_refine_residual<<<nb, 256, 0, s>>>(c->r64, b, c->Ap64, c->Ap32, c->d_small + 2 * P, c->d_flags + 2 * P,
                                               c->d_flags + 3 * P, c->N, tot);
@@ -830,7 +786,7 @@ int final_rayleigh_ritz(nfs_ctx* c, int p, int nev, const int* flags, std::vecto
     CK(cudaMemcpyAsync(c->t64 + (long long)p * N, c->V + p * vstride + (long long)i * N, N * sizeof(double2),
                        cudaMemcpyDeviceToDevice, c->work));
     if (c->lamdf)
-      TRY(matvec_refine(c, c->work, c->t64, c->t64b, d_skip, 1));
+      TRY(matvec<nfs::df>(c, c->work, c->t64, c->t64b, d_skip, 1));
     else
       TRY(matvec<double>(c, c->work, c->t64, c->t64b, d_skip, 1));
     TRY(multi_dot(c, c->V, 0, nev, c->t64b, d, flags));
@@ -1373,9 +1329,9 @@ void free_ctx(nfs_ctx* c) {
   for (GraphEntry& g : c->graphs) cudaGraphExecDestroy(g.exec);
   for (GmresGraph& g : c->gm_graphs) cudaGraphExecDestroy(g.exec);
   void* ptrs[] = {c->lam64, c->lam32, c->tw64[0], c->tw64[1], c->tw64[2], c->tw32[0], c->tw32[1], c->tw32[2],
-                  c->mat64, c->mat32, c->basis64, c->bloch64, c->lamdf, c->twdf[0], c->twdf[1], c->twdf[2], c->matdf,
+                  c->mat64, c->pmat, c->pmu, c->basis64, c->bloch64, c->lamdf, c->twdf[0], c->twdf[1], c->twdf[2], c->matdf,
                   c->basisdf, c->fld, c->x64, c->r64, c->p64, c->Ap64, c->t64, c->t64b, c->x32, c->r32,
-                  c->p32, c->p32b, c->Ap32, c->st, c->d_small, c->d_flags, c->dscratch, c->V, c->MV, c->V32, c->MV32,
+                  c->p32, c->Ap32, c->st, c->d_small, c->d_flags, c->dscratch, c->V, c->MV, c->V32, c->MV32,
                   c->MV32lo, c->dY, c->binv64, c->zv, c->gv, c->zY};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -1420,8 +1376,7 @@ int prepare_problem(const int grid[3], const double* lattice, const double k[3],
     return NFS_EINVAL;
   const int n1 = grid[0], n2 = grid[1], n3 = grid[2];
   if (!size_ok(n1) || !size_ok(n2) || !size_ok(n3) || n1 != n2) return NFS_EUNSUPPORTED;
-  if (!nfs::matvec_supported<double>(n1, n2, n3) || !nfs::matvec_supported<float>(n1, n2, n3))
-    return NFS_EUNSUPPORTED;
+  if (!nfs::matvec_supported(n1, n2, n3)) return NFS_EUNSUPPORTED;
   double a_len[3] = {1.0, 1.0, 1.0};
   if (lattice) {
     for (int r = 0; r < 3; ++r)
@@ -1600,13 +1555,12 @@ int setup_class(nfs_ctx** out, int P, const int grid[3], const nfs_material* con
   {
     const size_t ml = (size_t)c->mat_len;
     TRYC(dalloc(c, &c->mat64, (size_t)P * ml));
-    TRYC(dalloc(c, &c->mat32, (size_t)P * ml));
-    std::vector<float> m32(ml);
-    for (int p = 0; p < P; ++p) {
-      for (size_t i = 0; i < ml; ++i) m32[i] = (float)prep[p].m64[i];
+    for (int p = 0; p < P; ++p)
       CKC(cudaMemcpy(c->mat64 + (size_t)p * ml, prep[p].m64.data(), ml * sizeof(double), cudaMemcpyHostToDevice));
-      CKC(cudaMemcpy(c->mat32 + (size_t)p * ml, m32.data(), ml * sizeof(float), cudaMemcpyHostToDevice));
-    }
+    TRYC(dalloc(c, &c->pmat, (size_t)P * 3 * c->n / 2));
+    if (c->has_mu) TRYC(dalloc(c, &c->pmu, (size_t)P * 3 * c->n / 2));
+    CKC(nfs::pair_material_launch(c->mat64, c->mat_len, n1, n3, c->kind, c->ax_a, c->ax_b, c->gam_len, c->has_mu,
+                                  c->pmat, c->pmu, P, 0));
   }
   {
     std::vector<double2> d((size_t)P * nl);
@@ -1652,7 +1606,6 @@ int setup_class(nfs_ctx** out, int P, const int grid[3], const nfs_material* con
     TRYC(dalloc(c, &c->r32, PN));
     TRYC(dalloc(c, &c->p32, PN));
     TRYC(dalloc(c, &c->Ap32, PN));
-    if (nfs::cg_needs_p_out<float>(n1)) TRYC(dalloc(c, &c->p32b, PN));
   }
   TRYC(dalloc(c, &c->st, P));
   CKC(cudaMallocHost((void**)&c->st_host, (size_t)P * sizeof(CGState)));
@@ -1663,11 +1616,10 @@ int setup_class(nfs_ctx** out, int P, const int grid[3], const nfs_material* con
   TRYC(dalloc(c, &c->d_flags, (size_t)kFlagSlots * P));
   CKC(cudaMallocHost((void**)&c->h_flags, (size_t)kFlagSlots * P * sizeof(int)));
   TRYC(ensure_scratch(c, (size_t)kRedBlocks * 2 * 64 * P + 4096));
-  CKC(nfs::matvec_prepare<double>(n1, n2, n3));
-  CKC(nfs::matvec_prepare<float>(n1, n2, n3));
-  if (o.precision == NFS_PREC_MIXED) CKC(nfs::matvec_prepare<nfs::df>(n1, n2, n3));
-  CKC(nfs::grad_prepare(n1, n2, n3));
-  CKC(nfs::fields_prepare(n1, n2, n3));
+  CKC(nfs::matvec_prepare<double>(n1, n3));
+  CKC(nfs::matvec_prepare<float>(n1, n3));
+  if (o.precision == NFS_PREC_MIXED) CKC(nfs::matvec_prepare<nfs::df>(n1, n3));
+  CKC(nfs::fields_prepare(n1, n3));
   // an explicit basis size: the eigensolver's memory is taken here, so that
   // no later call allocates
   if (o.ncv > 0) TRYC(reserve_lanczos(c, (int)std::min<long long>(o.ncv, c->N - 1)));
@@ -1768,7 +1720,7 @@ extern "C" int nfs_matvec(nfs_ctx* c, int dtype, const void* u, void* Au) {
   if (dtype == NFS_C64) return matvec<float>(c, c->stream, (const float2*)u, (float2*)Au);
   if (dtype == NFS_C128_DS) {
     if (!c->lamdf) return NFS_EINVAL;  // FP64 contexts hold no double-single tables
-    return matvec_refine(c, c->stream, (const double2*)u, (double2*)Au, nullptr, 0);
+    return matvec<nfs::df>(c, c->stream, (const double2*)u, (double2*)Au);
   }
   return NFS_EINVAL;
 }
@@ -1884,8 +1836,12 @@ extern "C" int nfs_eig_grad(nfs_ctx* c, int m, const double* weights, const void
   TRY(join_caller(c));
   cudaStream_t s = c->work;
   const long long n = c->n, N = c->N;
+  // the two coupled pairs of a pseudochiral medium accumulate apart (in the
+  // work vector x64, 2n of its 8n doubles) and are added at the end
+  const bool chiral = c->kind == NFS_MEDIUM_CHIRAL;
+  double* dg = chiral ? d_gamma : (d_gamma ? reinterpret_cast<double*>(c->x64) : nullptr);
   if (d_eps) CK(cudaMemsetAsync(d_eps, 0, 3 * n * sizeof(double), s));
-  if (d_gamma) CK(cudaMemsetAsync(d_gamma, 0, c->gam_len * sizeof(double), s));
+  if (dg) CK(cudaMemsetAsync(dg, 0, (chiral ? 3 : 2) * n * sizeof(double), s));
   const double2* Y = (const double2*)Yv;
   std::vector<double> yBy;
   for (int j = 0; j < m; ++j) {
@@ -1897,17 +1853,22 @@ extern "C" int nfs_eig_grad(nfs_ctx* c, int m, const double* weights, const void
     const double scale = weights[j] / ((double)n * yBy[0]);
     nfs::MatvecArgs<double> a = margs<double>(c, y, nullptr, nullptr);
     a.stream = s;
-    cudaError_t e = nfs::pass1_launch<double>(a);
-    if (e != cudaSuccess) return cuda_fail(e, "grad pass 1");
+    cudaError_t e = nfs::matvec_launch_mask<double>(a, 1);
+    if (e != cudaSuccess) return cuda_fail(e, "grad rows");
     nfs::GradArgs g{};
-    g.fld = (const double2*)c->fld; g.tw3 = c->tw64[2];
+    g.fld = c->fld; g.tw1 = c->tw64[0]; g.tw3 = c->tw64[2];
     g.inv_phi = c->mat64; g.gam = c->mat64 + 3 * n;
     g.kind = c->kind; g.ax_a = c->ax_a; g.ax_b = c->ax_b;
-    g.n1 = c->n1; g.n2 = c->n2; g.n3 = c->n3;
-    g.scale = scale; g.d_eps = d_eps; g.d_gamma = d_gamma; g.stream = s;
+    g.n1 = c->n1; g.n3 = c->n3;
+    g.scale = scale; g.d_eps = d_eps; g.dg = dg; g.stream = s;
     e = nfs::grad_launch(g);
     if (e != cudaSuccess) return cuda_fail(e, "grad launch");
-    c->launches += 2 + nfs::plane_pass_kernels<double>(c->n1);  // B_r, pass 1, gradient
+    c->launches += 3;  // B_r, rows, gradient
+  }
+  if (!chiral && d_gamma) {
+    nfs::k_add<<<grid_blocks(n, 256), 256, 0, s>>>(dg, dg + n, d_gamma, n);
+    CK(cudaGetLastError());
+    c->launches += 1;
   }
   CK(cudaStreamSynchronize(s));
   return NFS_OK;
@@ -1921,20 +1882,18 @@ extern "C" int nfs_eig_fields(nfs_ctx* c, int m, const void* Yv, void* Xv) {
   const double2* Y = (const double2*)Yv;
   double2* X = (double2*)Xv;
   for (int j = 0; j < m; ++j) {
-    // pass 1 of the complex128 product: the sqrt(n)-scaled untwisted (p, q),
-    // transformed along x and y
     nfs::MatvecArgs<double> a = margs<double>(c, Y + (long long)j * N, nullptr, nullptr);
-    cudaError_t e = nfs::pass1_launch<double>(a);
-    if (e != cudaSuccess) return cuda_fail(e, "fields pass 1");
+    cudaError_t e = nfs::matvec_launch_mask<double>(a, 1);
+    if (e != cudaSuccess) return cuda_fail(e, "fields rows");
     nfs::FieldsArgs f{};
-    f.fld = (const double2*)c->fld; f.tw3 = c->tw64[2]; f.bloch = c->bloch64;
+    f.fld = c->fld; f.tw1 = c->tw64[0]; f.tw3 = c->tw64[2]; f.bloch = c->bloch64;
     f.inv_phi = a.inv_phi; f.gam = a.gam; f.inv_mu = a.inv_mu;
     f.kind = c->kind; f.ax_a = c->ax_a; f.ax_b = c->ax_b;
-    f.n1 = c->n1; f.n2 = c->n2; f.n3 = c->n3;
+    f.n1 = c->n1; f.n3 = c->n3;
     f.X = X + (long long)j * 6 * n; f.stream = c->stream;
     e = nfs::fields_launch(f);
     if (e != cudaSuccess) return cuda_fail(e, "fields launch");
-    c->launches += 1 + nfs::plane_pass_kernels<double>(c->n1);
+    c->launches += 2;
   }
   return NFS_OK;
 }
@@ -1980,22 +1939,22 @@ extern "C" int nfs_gep_residual(nfs_ctx* c, int m, const double* omega, const vo
 
 namespace {
 
-// M y (- sigma v) on the given stream: Sigma^{1/2}, pass 1, the B^{-1} z-pass,
-// pass 3, halves exchanged and Sigma^{1/2} (t64 and Ap64 are its temporaries)
+// M y (- sigma v) on the given stream: Sigma^{1/2}, k_rows_in, the column kernel
+// with B^{-1}, k_rows_out, halves exchanged and Sigma^{1/2} (t64 and Ap64 are its temporaries)
 int nfsep_apply(nfs_ctx* c, cudaStream_t s, const double2* y, double2* out, const double2* v, double2 sigma) {
   cudaError_t e = nfs::nfsep_prescale(y, c->t64, c->lam64, c->n1, c->n2, c->n3, s);
   if (e != cudaSuccess) return cuda_fail(e, "nfsep prescale");
   nfs::MatvecArgs<double> a = margs<double>(c, c->t64, c->Ap64, nullptr);
   a.stream = s;
-  e = nfs::pass1_launch<double>(a);
-  if (e != cudaSuccess) return cuda_fail(e, "nfsep pass 1");
-  e = nfs::nfsep_pass2((double2*)c->fld, c->binv64, c->tw64[2], c->n1, c->n2, c->n3, s);
-  if (e != cudaSuccess) return cuda_fail(e, "nfsep pass 2");
+  e = nfs::matvec_launch_mask<double>(a, 1);
+  if (e != cudaSuccess) return cuda_fail(e, "nfsep rows");
+  e = nfs::nfsep_columns(c->fld, c->binv64, c->tw64[0], c->tw64[2], c->n1, c->n3, s);
+  if (e != cudaSuccess) return cuda_fail(e, "nfsep columns");
   e = nfs::matvec_launch_mask<double>(a, 4);
-  if (e != cudaSuccess) return cuda_fail(e, "nfsep pass 3");
+  if (e != cudaSuccess) return cuda_fail(e, "nfsep rows out");
   e = nfs::nfsep_post(c->Ap64, out, c->lam64, c->n1, c->n2, c->n3, v, sigma, s);
   if (e != cudaSuccess) return cuda_fail(e, "nfsep post");
-  c->launches += 3 + 2 * nfs::plane_pass_kernels<double>(c->n1);
+  c->launches += 2 + nfs::kProductKernels;
   return NFS_OK;
 }
 
@@ -2040,7 +1999,7 @@ struct DevBasis : virtual nfs::host::KrylovOps {
     return NFS_OK;
   }
   int norm(double& nrm) override {
-    nfs::k_dot_re<double2><<<dim3(kRedBlocks, 1), kRedThreads, 0, s>>>(w, w, N, c->dscratch, kRedBlocks, nullptr, 0);
+    nfs::k_dot_re<double2><<<dim3(kRedBlocks, 1), kRedThreads, 0, s>>>(w, w, N, c->dscratch, kRedBlocks);
     CK(cudaGetLastError());
     c->launches += 1;
     CK(cudaMemcpyAsync(c->hscratch, c->dscratch, kRedBlocks * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -2365,7 +2324,7 @@ extern "C" int nfs_setup_biiso(nfs_ctx** out, const int grid[3], const double* l
   const int rc = [&]() -> int {
     TRY(dalloc(c, &c->binv64, binv.size()));
     CK(cudaMemcpy(c->binv64, binv.data(), binv.size() * sizeof(double2), cudaMemcpyHostToDevice));
-    CK(nfs::nfsep_prepare(c->n3));
+    CK(nfs::nfsep_prepare(c->n1, c->n3));
     return NFS_OK;
   }();
   if (rc != NFS_OK) {
@@ -2445,12 +2404,12 @@ extern "C" int nfs_nfsep_fields(nfs_ctx* c, int m, const void* Yv, void* Xv) {
                                         c->n3, c->stream);
     if (e != cudaSuccess) return cuda_fail(e, "nfsep fields prescale");
     nfs::MatvecArgs<double> a = margs<double>(c, c->t64, nullptr, nullptr);
-    e = nfs::pass1_launch<double>(a);
-    if (e != cudaSuccess) return cuda_fail(e, "nfsep fields pass 1");
-    e = nfs::nfsep_fields((const double2*)c->fld, c->binv64, c->tw64[2], c->bloch64, c->n1, c->n2, c->n3,
+    e = nfs::matvec_launch_mask<double>(a, 1);
+    if (e != cudaSuccess) return cuda_fail(e, "nfsep fields rows");
+    e = nfs::nfsep_fields(c->fld, c->binv64, c->tw64[0], c->tw64[2], c->bloch64, c->n1, c->n3,
                           (double2*)Xv + (long long)j * 6 * n, c->stream);
     if (e != cudaSuccess) return cuda_fail(e, "nfsep fields");
-    c->launches += 2 + nfs::plane_pass_kernels<double>(c->n1);
+    c->launches += 3;
   }
   return NFS_OK;
 }

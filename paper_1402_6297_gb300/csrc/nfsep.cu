@@ -1,7 +1,7 @@
 // Kernels of the null space free standard problem for any nonsingular B
-// (see nfsep.h).  The DFT passes are those of the A_r product
-// (matvec_kernels.cuh); only the per-voxel step between the z transforms and
-// the scalings around the product differ.
+// (see nfsep.h).  The DFT kernels are those of the A_r product
+// (matvec_kernels.cuh); only the per-voxel step of the column kernel and the
+// scalings around the product differ.
 #include <algorithm>
 #include <cmath>
 
@@ -38,88 +38,50 @@ __global__ void k_nfsep_post(const double2* __restrict__ a, double2* __restrict_
   }
 }
 
-// (e_c, h_c) = B_c^{-1} (p_c, q_c) for the three components of one voxel
-struct BinvVoxel {
-  const double2* b;
-  long long n, v;
-  __device__ __forceinline__ void apply(int k, double2 p, double2 q, double scale, double2& e, double2& h) const {
-    const double2* bk = b + (long long)(4 * k) * n + v;
-    e = cscale(cadd(cmul(bk[0], p), cmul(bk[n], q)), scale);
-    h = cscale(cadd(cmul(bk[2 * n], p), cmul(bk[3 * n], q)), scale);
+// (e_c, h_c) = B_c^{-1} (p_c, q_c) for component c = the pair of one voxel
+struct BinvStep {
+  const double2* binv;
+  long long n;
+  double scale;
+  template <int NB>
+  struct Vals {};
+  template <int NB>
+  __device__ __forceinline__ void load(const ColumnPos&, int, Vals<NB>&) const {}
+  __device__ __forceinline__ void solve(const ColumnPos& c, long long v, double2 p, double2 q, double2& e,
+                                        double2& h) const {
+    const double2* b = binv + 4 * c.j * n + v;
+    e = cscale(cadd(cmul(b[0], p), cmul(b[n], q)), scale);
+    h = cscale(cadd(cmul(b[2 * n], p), cmul(b[3 * n], q)), scale);
   }
 };
 
-template <int N3, int TX, int NT>
-__global__ void __launch_bounds__(NT)
-k_pass2_z_nfsep(double2* __restrict__ fld, const double2* __restrict__ binv, const double2* __restrict__ twz, int ncols,
-                double inv_n) {
-  using C = double2;
-  constexpr int LINES = 6 * TX;
-  constexpr int PITCH = LINES + 1;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* buf = reinterpret_cast<C*>(smem_raw);
-  C* stw = buf + N3 * PITCH;
-  for (int i = threadIdx.x; i < N3; i += NT) stw[i] = twz[i];
-  const int col0 = blockIdx.x * TX;
-  const long long n = (long long)ncols * N3;
-  C* tile = fld + col0;
-  // line l = f * TX + c: field f, column col0 + c
-  auto gaddr = [&](int l, int z) { return tile + (long long)(l / TX) * n + (long long)z * ncols + (l % TX); };
-  __syncthreads();  // twiddles
-  smem_fft_io<true, N3, LINES, NT, 1, PITCH, true, false>(buf, stw, [&](int l, int z) { return ldg_c(gaddr(l, z)); },
-                                                         NoPut{});
-  for (int idx = threadIdx.x; idx < N3 * TX; idx += NT) {
-    const int c = idx % TX, z = idx / TX;
-    C* row = buf + z * PITCH + c;
-    const BinvVoxel bv{binv, n, (long long)z * ncols + col0 + c};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      C e, h;
-      bv.apply(k, row[k * TX], row[(3 + k) * TX], inv_n, e, h);
-      row[k * TX] = h;        // projected by P_r^* in pass 3 (group 0)
-      row[(3 + k) * TX] = e;  // projected by Q_r^* in pass 3 (group 1)
-    }
+struct NfsepStep : BinvStep {
+  static constexpr bool kForward = true;
+  template <int NB>
+  __device__ __forceinline__ double apply(const ColumnPos& c, int b, const Vals<NB>&, int, double2& p, double2& q) const {
+    double2 e, h;
+    solve(c, c.voxel(b), p, q, e, h);
+    p = h;  // projected by P_r^*
+    q = e;  // projected by Q_r^*
+    return 0.0;
   }
-  __syncthreads();
-  smem_fft_io<false, N3, LINES, NT, 1, PITCH, false, true>(buf, stw, NoGet{},
-                                                          [&](int l, int z, C v) { *gaddr(l, z) = v; });
-}
+};
 
-template <int N3, int TX, int NT>
-__global__ void __launch_bounds__(NT)
-k_fields_z_nfsep(const double2* __restrict__ fld, const double2* __restrict__ binv, const double2* __restrict__ twz,
-                 int n1, int ncols, const double2* __restrict__ bloch, double inv_sqrt_n, double2* __restrict__ X) {
-  using C = double2;
-  constexpr int LINES = 6 * TX;
-  constexpr int PITCH = LINES + 1;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* buf = reinterpret_cast<C*>(smem_raw);
-  C* stw = buf + N3 * PITCH;
-  for (int i = threadIdx.x; i < N3; i += NT) stw[i] = twz[i];
-  const int col0 = blockIdx.x * TX;
-  const long long n = (long long)ncols * N3;
-  const C* tile = fld + col0;
-  auto gaddr = [&](int l, int z) { return tile + (long long)(l / TX) * n + (long long)z * ncols + (l % TX); };
-  __syncthreads();
-  smem_fft_io<true, N3, LINES, NT, 1, PITCH, true, false>(buf, stw, [&](int l, int z) { return ldg_c(gaddr(l, z)); },
-                                                         NoPut{});
-  const int n2 = ncols / n1;
-  for (int idx = threadIdx.x; idx < N3 * TX; idx += NT) {
-    const int c = idx % TX, z = idx / TX;
-    const int col = col0 + c;
-    const long long v = (long long)z * ncols + col;
-    const C* row = buf + z * PITCH + c;
-    const BinvVoxel bv{binv, n, v};
-    const C d = cmul(cmul(bloch[col % n1], bloch[n1 + col / n1]), bloch[n1 + n2 + z]);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      C e, h;
-      bv.apply(k, row[k * TX], row[(3 + k) * TX], inv_sqrt_n, e, h);
-      X[k * n + v] = cmul(d, e);
-      X[(3 + k) * n + v] = cmul(d, h);
-    }
+struct NfsepFieldsStep : BinvStep {
+  static constexpr bool kForward = false;
+  const double2* bloch;
+  double2* X;
+  template <int NB>
+  __device__ __forceinline__ double apply(const ColumnPos& c, int b, const Vals<NB>&, int, double2& p, double2& q) const {
+    const long long v = c.voxel(b);
+    double2 e, h;
+    solve(c, v, p, q, e, h);
+    const double2 d = cmul(cmul(bloch[c.x], bloch[c.n1 + c.a + c.N1 * b]), bloch[2 * c.n1 + c.z]);
+    X[c.j * n + v] = cmul(d, e);
+    X[(3 + c.j) * n + v] = cmul(d, h);
+    return 0.0;
   }
-}
+};
 
 __global__ void k_zaxpy_basis(double2* __restrict__ w, const double2* __restrict__ V, long long N,
                               const double* __restrict__ c, int m, double sign) {
@@ -358,36 +320,6 @@ __global__ void k_gmres_store(const double2* __restrict__ w, double2* __restrict
 
 int blocks_for(long long work) { return (int)std::max<long long>(1, std::min<long long>((work + 255) / 256, 152LL * 16)); }
 
-template <int N3>
-cudaError_t prep_n3() {
-  constexpr int TX = z_tile(N3, 16);
-  constexpr int NT = z_threads(N3, 16);
-  cudaError_t e = cudaFuncSetAttribute(k_pass2_z_nfsep<N3, TX, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)z_smem<double, N3>());
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_fields_z_nfsep<N3, TX, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)z_smem<double, N3>());
-}
-
-template <int N3>
-cudaError_t pass2_n3(double2* fld, const double2* binv, const double2* tw3, int ncols, cudaStream_t s) {
-  constexpr int TX = z_tile(N3, 16);
-  constexpr int NT = z_threads(N3, 16);
-  k_pass2_z_nfsep<N3, TX, NT><<<ncols / TX, NT, z_smem<double, N3>(), s>>>(fld, binv, tw3, ncols,
-                                                                         1.0 / ((double)ncols * N3));
-  return cudaGetLastError();
-}
-
-template <int N3>
-cudaError_t fields_n3(const double2* fld, const double2* binv, const double2* tw3, const double2* bloch, int n1,
-                      int ncols, double2* X, cudaStream_t s) {
-  constexpr int TX = z_tile(N3, 16);
-  constexpr int NT = z_threads(N3, 16);
-  k_fields_z_nfsep<N3, TX, NT><<<ncols / TX, NT, z_smem<double, N3>(), s>>>(
-      fld, binv, tw3, n1, ncols, bloch, 1.0 / std::sqrt((double)ncols * N3), X);
-  return cudaGetLastError();
-}
-
 }  // namespace
 
 cudaError_t nfsep_prescale(const double2* y, double2* t, const double2* lam, int n1, int n2, int n3,
@@ -404,33 +336,31 @@ cudaError_t nfsep_post(const double2* a, double2* out, const double2* lam, int n
   return cudaGetLastError();
 }
 
-cudaError_t nfsep_prepare(int n3) {
-  switch (n3) {
-#define NFS_CASE(N) case N: return prep_n3<N>();
-    NFS_FOR_EACH_SIZE(NFS_CASE)
-#undef NFS_CASE
-  }
-  return cudaErrorInvalidValue;
+cudaError_t nfsep_prepare(int n1, int n3) {
+  const cudaError_t e = columns_prepare<double, NfsepStep>(n1, n3);
+  return e != cudaSuccess ? e : columns_prepare<double, NfsepFieldsStep>(n1, n3);
 }
 
-cudaError_t nfsep_pass2(double2* fld, const double2* binv, const double2* tw3, int n1, int n2, int n3,
-                        cudaStream_t s) {
-  switch (n3) {
-#define NFS_CASE(N) case N: return pass2_n3<N>(fld, binv, tw3, n1 * n2, s);
-    NFS_FOR_EACH_SIZE(NFS_CASE)
-#undef NFS_CASE
-  }
-  return cudaErrorInvalidValue;
+cudaError_t nfsep_columns(void* fld, const double2* binv, const double2* tw1, const double2* tw3, int n1, int n3,
+                          cudaStream_t s) {
+  const long long n = (long long)n1 * n1 * n3;
+  NfsepStep step;
+  step.binv = binv;
+  step.n = n;
+  step.scale = 1.0 / (double)n;
+  return columns_launch<double>(fld, step, tw1, tw3, n1, n3, 1, nullptr, nullptr, BatchStrides{}, s);
 }
 
-cudaError_t nfsep_fields(const double2* fld, const double2* binv, const double2* tw3, const double2* bloch,
-                         int n1, int n2, int n3, double2* X, cudaStream_t s) {
-  switch (n3) {
-#define NFS_CASE(N) case N: return fields_n3<N>(fld, binv, tw3, bloch, n1, n1 * n2, X, s);
-    NFS_FOR_EACH_SIZE(NFS_CASE)
-#undef NFS_CASE
-  }
-  return cudaErrorInvalidValue;
+cudaError_t nfsep_fields(void* fld, const double2* binv, const double2* tw1, const double2* tw3, const double2* bloch,
+                         int n1, int n3, double2* X, cudaStream_t s) {
+  const long long n = (long long)n1 * n1 * n3;
+  NfsepFieldsStep step;
+  step.binv = binv;
+  step.n = n;
+  step.scale = 1.0 / std::sqrt((double)n);
+  step.bloch = bloch;
+  step.X = X;
+  return columns_launch<double>(fld, step, tw1, tw3, n1, n3, 1, nullptr, nullptr, BatchStrides{}, s);
 }
 
 cudaError_t zaxpy_basis(double2* w, const double2* V, long long N, const double* c, int m, double sign,

@@ -122,7 +122,7 @@ extern "C" int nfs_matvec_noalloc(const int grid[3], const double k[3], int kind
   if (!edge_ok(n1) || !edge_ok(n2) || !edge_ok(n3) || n1 != n2) return NFS_EUNSUPPORTED;
   const long long n = (long long)n1 * n2 * n3;
   if (n > kMaxVoxels) return NFS_EUNSUPPORTED;  // the static workspace holds 32^3 voxels at most
-  if (!nfs::matvec_supported<double>(n1, n2, n3)) return NFS_EUNSUPPORTED;
+  if (!nfs::matvec_supported(n1, n2, n3)) return NFS_EUNSUPPORTED;
   if (kind != NFS_MEDIUM_CHIRAL && kind != NFS_MEDIUM_PSEUDOCHIRAL) return NFS_EINVAL;
   if (kind == NFS_MEDIUM_PSEUDOCHIRAL &&
       (axis_a < 0 || axis_a > 2 || axis_b < 0 || axis_b > 2 || axis_a == axis_b))
@@ -170,7 +170,7 @@ extern "C" int nfs_matvec_noalloc(const int grid[3], const double k[3], int kind
     }
     base = g_scratch_addr[dev];
     // opt the kernels for this grid in to their shared memory (allocates nothing)
-    e = nfs::matvec_prepare<double>(n1, n2, n3);
+    e = nfs::matvec_prepare<double>(n1, n3);
     if (e != cudaSuccess) return NFS_ECUDA;
   }
   unsigned char* b = static_cast<unsigned char*>(base);
@@ -193,10 +193,9 @@ extern "C" int nfs_matvec_noalloc(const int grid[3], const double k[3], int kind
   nfs::MatvecArgs<double> a{};
   a.u = static_cast<const double2*>(u);
   a.Au = static_cast<double2*>(Au);
-  a.fld = reinterpret_cast<double2*>(b + kOffFld);
+  a.fld = b + kOffFld;
   a.lam = t.lam;
   a.tw1 = t.tw;
-  a.tw2 = t.tw + kMaxEdge;
   a.tw3 = t.tw + 2 * kMaxEdge;
   a.inv_phi = t.inv_phi;
   a.gam = t.gam;
@@ -205,7 +204,6 @@ extern "C" int nfs_matvec_noalloc(const int grid[3], const double k[3], int kind
   a.ax_a = kind == NFS_MEDIUM_CHIRAL ? 0 : axis_a;
   a.ax_b = kind == NFS_MEDIUM_CHIRAL ? 1 : axis_b;
   a.n1 = n1;
-  a.n2 = n2;
   a.n3 = n3;
   a.alpha = alpha;
   a.beta = beta;
