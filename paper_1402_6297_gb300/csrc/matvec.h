@@ -67,6 +67,7 @@ struct MatvecArgs {
   // (spectral order); nullptr: evaluated from the Lambda tables in the kernels
   const cplx<R>* basis;
   cudaStream_t stream;
+  bool serial;            // no overlap between kernels: the tables are being written on the stream
   CgFuse<R> cg;           // optional: one CG step (u and Au are then unused)
   // batching: P problems of this grid in one launch (P = 1 for one problem)
   int P;

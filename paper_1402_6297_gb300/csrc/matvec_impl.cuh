@@ -66,6 +66,36 @@ static cudaError_t allow_smem(K* kernel, size_t bytes) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+// Launch with programmatic stream serialisation (see depend_wait), unless the
+// tables were written on the stream a moment ago (`serial`) or it does not pay:
+// CTAs that start early are placed on the SMs that happen to be free, which is
+// harmless while the kernels are short (complex64 products on GB300, us: 8^3
+// 7.0 -> 5.5, 32^3 10.2 -> 8.7, 64^3 22.7 -> 21.3, 96^3 65.6 -> 63.1; but 128^3
+// 173.6 -> 177.4) and costly where every SM's share of the FP64 work counts
+// (complex128 8^3 15.0 -> 13.3, but 32^3 66 -> 73, 48x48x32 134 -> 191), so the
+// scalar types overlap only products with at most one CTA per SM.
+template <typename R>
+static bool overlap(int n1, int n3, int P) {
+  if (ElemOf<R>::NF == 1) return n1 < 128;
+  const int N2 = n1 < 24 ? 4 : 8, X = n1 < 24 ? 1 : NFS_X;
+  return std::max(2 * N2 * n3, 3 * (n1 / N2) * (n1 / X)) * P <= 152;
+}
+template <typename... P, typename... A>
+static cudaError_t launch_dependent(bool serial, void (*kernel)(P...), dim3 grid, int threads, size_t smem,
+                                    cudaStream_t s, A... a) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = serial ? 0 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(a)...);
+}
+
 // f(tag) with the column tile of plane edge n1: tag::N2, tag::X, tag::XL
 template <int N2_, int X_, int XL_>
 struct ColumnTile {
@@ -96,18 +126,17 @@ static cudaError_t columns_prepare(int n1, int n3) {
 
 template <typename R, class Step>
 static cudaError_t columns_launch(void* fld, const Step& step, const cplx<R>* tw1, const cplx<R>* tw3, int n1, int n3,
-                                  int P, const int* skip, CGState* st, const BatchStrides& bs, cudaStream_t s) {
+                                  int P, const int* skip, CGState* st, const BatchStrides& bs, cudaStream_t s,
+                                  bool serial = false) {
   return with_column_tile<R>(n1, [&](auto tag) -> cudaError_t {
     using T = decltype(tag);
     const dim3 grid(n1 / T::X, n1 / T::N2, 3 * P);
     auto* f = static_cast<typename ElemOf<R>::E*>(fld);
     switch (n3) {
-#define NFS_CASE(N)                                                                                              \
-  case N:                                                                                                        \
-    columns_kernel<R, T, N, Step>()<<<grid, ColumnsConfig<R, T::N2, T::X, N>::NT,                      \
-                                                columns_smem<R, T::N2, T::X, N>(), s>>>(f, step, tw1, tw3, skip, \
-                                                                                        st, bs);                 \
-    return cudaGetLastError();
+#define NFS_CASE(N)                                                                              \
+  case N:                                                                                        \
+    return launch_dependent(serial || !overlap<R>(n1, n3, P), columns_kernel<R, T, N, Step>(), grid, ColumnsConfig<R, T::N2, T::X, N>::NT, \
+                            columns_smem<R, T::N2, T::X, N>(), s, f, step, tw1, tw3, skip, st, bs);
       NFS_FOR_EACH_SIZE(NFS_CASE)
 #undef NFS_CASE
     }
@@ -126,13 +155,12 @@ static cudaError_t rows_launch_n(const MatvecArgs<R>& a, bool in) {
   const dim3 grid(PlaneSplit<R, N>::N2 * ElemOf<R>::NF, a.n3, a.P > 0 ? a.P : 1);
   auto* f = static_cast<typename ElemOf<R>::E*>(a.fld);
   constexpr int NT = RowsConfig<R, N>::NT;
+  const bool serial = a.serial || !overlap<R>(N, a.n3, a.P > 0 ? a.P : 1);
   if (in)
-    rows_in_kernel<R, N>()<<<grid, NT, rows_smem<R, N>(), a.stream>>>(a.u, f, a.lam, a.tw1, a.alpha, a.beta, a.kind,
-                                                                     a.ax_a, a.ax_b, a.skip, a.basis, a.bs, a.cg);
-  else
-    rows_out_kernel<R, N>()<<<grid, NT, rows_smem<R, N>(), a.stream>>>(f, a.Au, a.lam, a.tw1, a.alpha, a.beta, a.kind,
-                                                                      a.ax_a, a.ax_b, a.skip, a.basis, a.bs, a.cg);
-  return cudaGetLastError();
+    return launch_dependent(serial, rows_in_kernel<R, N>(), grid, NT, rows_smem<R, N>(), a.stream, a.u, f, a.lam, a.tw1,
+                            a.alpha, a.beta, a.kind, a.ax_a, a.ax_b, a.skip, a.basis, a.bs, a.cg);
+  return launch_dependent(serial, rows_out_kernel<R, N>(), grid, NT, rows_smem<R, N>(), a.stream, f, a.Au, a.lam, a.tw1,
+                          a.alpha, a.beta, a.kind, a.ax_a, a.ax_b, a.skip, a.basis, a.bs, a.cg);
 }
 
 template <typename R>
@@ -165,7 +193,8 @@ cudaError_t product_columns_launch(const MatvecArgs<R>& a) {
   const long long n = (long long)a.n1 * a.n1 * a.n3;
   const ProductStep<R> step{{a.inv_phi, a.gam, a.inv_mu, a.pmat, a.pmu, a.kind, a.ax_a, a.ax_b, n},
                             (R)(1.0 / (double)n), a.bs.smat};
-  return columns_launch<R>(a.fld, step, a.tw1, a.tw3, a.n1, a.n3, a.P > 0 ? a.P : 1, a.skip, a.cg.st, a.bs, a.stream);
+  return columns_launch<R>(a.fld, step, a.tw1, a.tw3, a.n1, a.n3, a.P > 0 ? a.P : 1, a.skip, a.cg.st, a.bs, a.stream,
+                           a.serial);
 }
 
 template <typename R>

@@ -92,7 +92,14 @@ struct MatView {
   long long n;
 };
 
-__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+// Programmatic dependent launch (the kernels of a product are launched so that
+// the next one may start while the last CTAs of the one before still run):
+// depend_begin() lets the next kernel of the stream start, depend_wait() waits
+// for the one before to end with its writes visible.  Every CTA waits before it
+// touches anything but constant tables, and before it returns: a kernel that
+// ended earlier would let its successor run ahead of its predecessor.
+__device__ __forceinline__ void depend_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void depend_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Partner axis of pair j: s(j).
 __host__ __device__ __forceinline__ int pair_axis(int kind, int ax_a, int ax_b, int j) {
@@ -369,6 +376,8 @@ k_rows_in(const vecc<R>* u, typename ElemOf<R>::E* __restrict__ fld, const cplx<
   E* buf = reinterpret_cast<E*>(smem_raw);
   E* tw = buf + LINES * PITCH;
   const int b = blockIdx.x % N2, fsel = blockIdx.x / N2, i3 = blockIdx.y, prob = blockIdx.z, n3 = gridDim.y;
+  for (int i = threadIdx.x; i < N; i += NT) tw[i] = tw_entry(twx[i]);
+  depend_wait();
   if (skip != nullptr && skip[(long long)prob * bs.sskip]) return;
   constexpr bool CGT = !std::is_same<R, df>::value;  // (the double-single product never runs CG)
   CGState* st = (CGT && cg.st != nullptr) ? cg.st + prob : nullptr;
@@ -382,9 +391,8 @@ k_rows_in(const vecc<R>* u, typename ElemOf<R>::E* __restrict__ fld, const cplx<
   // the quarters of u that this CTA needs: all, or the two of its field
   constexpr int NQ = 4 / NF;
   const int q0 = NF == 1 ? 0 : 2 * fsel;
-  // the first voxel's inputs are on their way while the tables are staged and
-  // (in CG) the partials of r^* r are summed; each later voxel's while the one
-  // before it is assembled
+  // the first voxel's inputs are on their way while (in CG) the partials of
+  // r^* r are summed; each later voxel's while the one before it is assembled
   constexpr int NV = N1 * N;
   vecc<R> v[NQ], g[NQ];
   auto fetch = [&](int vi) {
@@ -399,7 +407,6 @@ k_rows_in(const vecc<R>* u, typename ElemOf<R>::E* __restrict__ fld, const cplx<
     }
   };
   fetch(threadIdx.x);
-  for (int i = threadIdx.x; i < N; i += NT) tw[i] = tw_entry(twx[i]);
   R bt = (R)0;
   if constexpr (CGT) {
     if (st != nullptr) {
@@ -467,6 +474,7 @@ k_rows_in(const vecc<R>* u, typename ElemOf<R>::E* __restrict__ fld, const cplx<
   __syncthreads();
   stage_group<false, N1, N2, LINES, NT, PITCH, 1>(buf, tw);
   __syncthreads();
+  depend_begin();
   // stage A along y over the rows, results to the workspace
 #pragma unroll 1
   for (int it = threadIdx.x; it < 3 * N; it += NT) {
@@ -595,10 +603,11 @@ k_columns(typename ElemOf<R>::E* __restrict__ fld, Step step, const cplx<R>* __r
   E* tz = buf + N3 * PITCH;
   E* ty = tz + N3;  // w_N^{a b}, b < N2
   const int xt = blockIdx.x, a = blockIdx.y, j = blockIdx.z % 3, prob = blockIdx.z / 3;
-  if (skip != nullptr && skip[(long long)prob * bs.sskip]) return;
-  const int stop = st != nullptr ? st[prob].stop : 0;
   for (int i = threadIdx.x; i < N3; i += NT) tz[i] = tw_entry(twz[i]);
   if (threadIdx.x < N2) ty[threadIdx.x] = tw_entry(twy[a * threadIdx.x]);
+  depend_wait();
+  if (skip != nullptr && skip[(long long)prob * bs.sskip]) return;
+  const int stop = st != nullptr ? st[prob].stop : 0;
   const int N1 = gridDim.y, N = N1 * N2;
   const long long n = (long long)N * N * N3;
   static_assert(XL % X == 0, "a column tile lies within one run of the workspace");
@@ -721,6 +730,7 @@ k_columns(typename ElemOf<R>::E* __restrict__ fld, Step step, const cplx<R>* __r
       stage_group<true, Z1, Z2, LINES, NT, 1, PITCH>(buf, tz);
       __syncthreads();
     }
+    depend_begin();
     // forward stage B' along z, results to the workspace
     constexpr int ITEMS = LINES * Z2;
 #pragma unroll 1
@@ -758,6 +768,8 @@ k_rows_out(const typename ElemOf<R>::E* __restrict__ fld, vecc<R>* __restrict__ 
   E* buf = reinterpret_cast<E*>(smem_raw);
   E* tw = buf + LINES * PITCH;
   const int b = blockIdx.x % N2, fsel = blockIdx.x / N2, i3 = blockIdx.y, prob = blockIdx.z, n3 = gridDim.y;
+  for (int i = threadIdx.x; i < N; i += NT) tw[i] = tw_entry(twx[i]);
+  depend_wait();
   if (skip != nullptr && skip[(long long)prob * bs.sskip]) return;
   constexpr bool CGT = !std::is_same<R, df>::value;  // (the double-single product never runs CG)
   CGState* st = (CGT && cg.st != nullptr) ? cg.st + prob : nullptr;
@@ -773,17 +785,6 @@ k_rows_out(const typename ElemOf<R>::E* __restrict__ fld, vecc<R>* __restrict__ 
       cg.x += prob * bs.su + q0 * n;
       cg.r += prob * bs.su + q0 * n;
       cg.p += prob * bs.su + q0 * n;
-      // the CG vectors of this CTA's rows do not all stay in L2 between two
-      // steps at 96^3: fetch them there while the transforms run
-      constexpr int LINE = 128 / (int)sizeof(C);  // elements of a cache line
-      constexpr int PER = (N + LINE - 1) / LINE;  // lines of a row
-      for (int i = threadIdx.x; i < NQ * N1 * PER; i += NT) {
-        const int q = i / (N1 * PER), row = i / PER % N1, l = i % PER;
-        const long long e = q * n + ((long long)i3 * N + b + N2 * row) * N + l * LINE;
-        prefetch_l2(cg.p + e);
-        prefetch_l2(cg.r + e);
-        prefetch_l2(cg.x + e);
-      }
       const auto* pa = reinterpret_cast<const typename RedAccFor<R>::partial*>(st->part_a);
 #pragma unroll 2
       for (int i = threadIdx.x; i < 3 * N1 * (N / X); i += NT) pap_acc.add_partial(pa[i]);
@@ -793,7 +794,6 @@ k_rows_out(const typename ElemOf<R>::E* __restrict__ fld, vecc<R>* __restrict__ 
   Au += prob * bs.su;
   lam += (long long)prob * bs.slam;
   if (basis != nullptr) basis += prob * bs.sbasis;
-  for (int i = threadIdx.x; i < N; i += NT) tw[i] = tw_entry(twx[i]);
   // stage B' along y from the workspace: row k of the CTA is y = b + N2 k
 #pragma unroll 1
   for (int it = threadIdx.x; it < 3 * N; it += NT) {
@@ -835,6 +835,7 @@ k_rows_out(const typename ElemOf<R>::E* __restrict__ fld, vecc<R>* __restrict__ 
     }
   }
   __syncthreads();
+  depend_begin();
   RedAccFor<R> rr_acc;
   const C a3 = lam[2 * N + i3];
 #pragma unroll 1

@@ -209,6 +209,7 @@ extern "C" int nfs_matvec_noalloc(const int grid[3], const double k[3], int kind
   a.beta = beta;
   a.skip = nullptr;
   a.stream = s;
+  a.serial = true;  // k_noalloc_prep writes the tables
   e = nfs::matvec_launch<double>(a);
   if (e != cudaSuccess) return NFS_ECUDA;
   int status = 0;
