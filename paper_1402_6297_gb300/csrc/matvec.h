@@ -44,6 +44,24 @@ struct CgFuse {
   CGState* st = nullptr;  // per problem: st + prob; nullptr: a plain product
 };
 
+// What the row kernels do besides when they form S Q_r^* e | S P_r^* h - sigma v of
+// the NFSEP (nfsep.h; complex128, one problem), S = Sigma_r^{1/2}, and the ends of
+// a GMRES step around it: k_rows_in scales its input by S; with `tmp` the input
+// is u - sum_g tmp_g (the end of the Gram-Schmidt update), stored into v, with
+// one partial of its squared norm per CTA.  k_rows_out exchanges the halves of
+// the result, scales by S and subtracts sigma v; with nnrm partials of |v|^2 it
+// also normalises: v and the result times 1 / |v| (0 for a zero v).
+struct KrylovFuse {
+  const double* root = nullptr;  // Lambda_q^{1/4} per voxel; nullptr: a plain product
+  const double2* tmp = nullptr;  // [groups][4n]
+  int groups = 0;
+  double2* v = nullptr;          // nullptr: no sigma v
+  double* nrm_out = nullptr;     // k_rows_in's partials
+  const double* nrm = nullptr;   // k_rows_out: partials to normalise by
+  int nnrm = 0;
+  double2 sigma = {0.0, 0.0};
+};
+
 template <typename R>
 struct MatvecArgs {
   const vecc<R>* u;       // 4n, spectral
@@ -68,6 +86,7 @@ struct MatvecArgs {
   const cplx<R>* basis;
   cudaStream_t stream;
   bool serial;            // no overlap between kernels: the tables are being written on the stream
+  KrylovFuse kr;          // optional (complex128)
   CgFuse<R> cg;           // optional: one CG step (u and Au are then unused)
   // batching: P problems of this grid in one launch (P = 1 for one problem)
   int P;

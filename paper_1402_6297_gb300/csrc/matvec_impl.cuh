@@ -150,17 +150,21 @@ static cudaError_t rows_prepare_n() {
   return e != cudaSuccess ? e : allow_smem(rows_out_kernel<R, N>(), rows_smem<R, N>());
 }
 
+static inline NoKrylov krylov_of(const KrylovFuse&, NoKrylov) { return {}; }
+static inline KrylovFuse krylov_of(const KrylovFuse& k, KrylovFuse) { return k; }
+
 template <typename R, int N>
 static cudaError_t rows_launch_n(const MatvecArgs<R>& a, bool in) {
   const dim3 grid(PlaneSplit<R, N>::N2 * ElemOf<R>::NF, a.n3, a.P > 0 ? a.P : 1);
   auto* f = static_cast<typename ElemOf<R>::E*>(a.fld);
   constexpr int NT = RowsConfig<R, N>::NT;
+  const auto kr = krylov_of(a.kr, typename KrylovOf<R>::type{});
   const bool serial = a.serial || !overlap<R>(N, a.n3, a.P > 0 ? a.P : 1);
   if (in)
     return launch_dependent(serial, rows_in_kernel<R, N>(), grid, NT, rows_smem<R, N>(), a.stream, a.u, f, a.lam, a.tw1,
-                            a.alpha, a.beta, a.kind, a.ax_a, a.ax_b, a.skip, a.basis, a.bs, a.cg);
+                            a.alpha, a.beta, a.kind, a.ax_a, a.ax_b, a.skip, a.basis, a.bs, a.cg, kr);
   return launch_dependent(serial, rows_out_kernel<R, N>(), grid, NT, rows_smem<R, N>(), a.stream, f, a.Au, a.lam, a.tw1,
-                          a.alpha, a.beta, a.kind, a.ax_a, a.ax_b, a.skip, a.basis, a.bs, a.cg);
+                          a.alpha, a.beta, a.kind, a.ax_a, a.ax_b, a.skip, a.basis, a.bs, a.cg, kr);
 }
 
 template <typename R>

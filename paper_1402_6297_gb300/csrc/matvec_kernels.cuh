@@ -356,6 +356,25 @@ __device__ __forceinline__ void stage_group(E* buf, const E* tw) {
 // k_rows_in: grid (N2 NF, n3, P); scalar elements: a CTA takes one field of
 // each pair (P_r u1 or Q_r u2)
 // ---------------------------------------------------------------------------
+// a - sum_{g < G} tmp[g stride], eight loads in flight at a time
+__device__ __forceinline__ double2 minus_groups(double2 a, const double2* tmp, long long stride, int G) {
+  for (int g0 = 0; g0 < G; g0 += 8) {
+    double2 x[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t)
+      if (g0 + t < G) x[t] = tmp[(g0 + t) * stride];
+#pragma unroll
+    for (int t = 0; t < 8; ++t)
+      if (g0 + t < G) a = csub(a, x[t]);
+  }
+  return a;
+}
+
+// (only complex128 kernels carry the Krylov pieces)
+struct NoKrylov {};
+template <typename R> struct KrylovOf { using type = NoKrylov; };
+template <> struct KrylovOf<double> { using type = KrylovFuse; };
+
 template <typename R, int N>
 constexpr size_t rows_smem() {
   return (size_t)(3 * PlaneSplit<R, N>::N1 * (N + 1) + N) * 16;
@@ -365,7 +384,7 @@ template <typename R, int N, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
 k_rows_in(const vecc<R>* u, typename ElemOf<R>::E* __restrict__ fld, const cplx<R>* __restrict__ lam,
           const cplx<R>* __restrict__ twx, R alpha, R beta, int kind, int ax_a, int ax_b, const int* __restrict__ skip,
-          const cplx<R>* __restrict__ basis, BatchStrides bs, CgFuse<R> cg) {
+          const cplx<R>* __restrict__ basis, BatchStrides bs, CgFuse<R> cg, typename KrylovOf<R>::type kr) {
   using C = cplx<R>;
   using E = typename ElemOf<R>::E;
   using S = PlaneSplit<R, N>;
@@ -424,6 +443,7 @@ k_rows_in(const vecc<R>* u, typename ElemOf<R>::E* __restrict__ fld, const cplx<
     }
   }
   const C a3 = lam[2 * N + i3];
+  RedAccFor<R> nrm_acc;
 #pragma unroll 1
   for (int vi = threadIdx.x; vi < NV; vi += NT) {
     const int row = vi / N, x = vi % N, y = row * N2 + b;
@@ -442,6 +462,21 @@ k_rows_in(const vecc<R>* u, typename ElemOf<R>::E* __restrict__ fld, const cplx<
       }
     }
     fetch(vi + NT);
+    if constexpr (std::is_same<R, double>::value) {
+      if (kr.root != nullptr) {
+        const double s = kr.root[e];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+          const long long at = (q0 + q) * n + e;
+          if (kr.tmp != nullptr) {
+            w[q] = minus_groups(w[q], kr.tmp + at, 4 * n, kr.groups);
+            kr.v[at] = w[q];
+            nrm_acc.add(cabs2(w[q]));
+          }
+          w[q] = cscale(w[q], s);
+        }
+      }
+    }
     Basis<R> B;
     voxel_basis<R>(basis, n, e, lam[x], lam[N + y], a3, alpha, beta, B);
     E* cell = buf + row * PITCH + x;
@@ -467,6 +502,12 @@ k_rows_in(const vecc<R>* u, typename ElemOf<R>::E* __restrict__ fld, const cplx<
       }
 #pragma unroll
       for (int j = 0; j < 3; ++j) cell[j * N1 * PITCH] = o[j];
+    }
+  }
+  if constexpr (std::is_same<R, double>::value) {
+    if (kr.tmp != nullptr) {
+      const double part = nrm_acc.template block_total<NT>();
+      if (threadIdx.x == 0) kr.nrm_out[i3 * gridDim.x + blockIdx.x] = part;
     }
   }
   __syncthreads();
@@ -755,7 +796,8 @@ template <typename R, int N, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
 k_rows_out(const typename ElemOf<R>::E* __restrict__ fld, vecc<R>* __restrict__ Au, const cplx<R>* __restrict__ lam,
            const cplx<R>* __restrict__ twx, R alpha, R beta, int kind, int ax_a, int ax_b,
-           const int* __restrict__ skip, const cplx<R>* __restrict__ basis, BatchStrides bs, CgFuse<R> cg) {
+           const int* __restrict__ skip, const cplx<R>* __restrict__ basis, BatchStrides bs, CgFuse<R> cg,
+           typename KrylovOf<R>::type kr) {
   using C = cplx<R>;
   using E = typename ElemOf<R>::E;
   using S = PlaneSplit<R, N>;
@@ -788,6 +830,15 @@ k_rows_out(const typename ElemOf<R>::E* __restrict__ fld, vecc<R>* __restrict__ 
       const auto* pa = reinterpret_cast<const typename RedAccFor<R>::partial*>(st->part_a);
 #pragma unroll 2
       for (int i = threadIdx.x; i < 3 * N1 * (N / X); i += NT) pap_acc.add_partial(pa[i]);
+    }
+  }
+  double inv_h = 1.0;
+  if constexpr (std::is_same<R, double>::value) {
+    if (kr.nnrm > 0) {
+      RedAcc<double> acc;
+      for (int i = threadIdx.x; i < kr.nnrm; i += NT) acc.add(kr.nrm[i]);
+      const double ss = acc.template block_total<NT>();
+      inv_h = ss > 0.0 ? ::rsqrt(ss) : 0.0;  // (a zero vector stays zero)
     }
   }
   fld += prob * bs.sfld;
@@ -888,10 +939,30 @@ k_rows_out(const typename ElemOf<R>::E* __restrict__ fld, vecc<R>* __restrict__ 
         }
         rr_acc.add(s);
       }
-    } else {
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) Au[(q0 + q) * n + e] = to_vec<R>(o[q]);
+      continue;
     }
+    if constexpr (std::is_same<R, double>::value) {
+      if (kr.root != nullptr) {
+        const double s = kr.root[e] * inv_h;
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+          const long long at = ((q0 + q + 2) & 3) * n + e;
+          double2 out = cscale(o[q], s);
+          if (kr.v != nullptr) {
+            double2 vv = kr.v[at];
+            if (kr.nnrm > 0) {
+              vv = cscale(vv, inv_h);
+              kr.v[at] = vv;
+            }
+            out = csub(out, cmul(kr.sigma, vv));
+          }
+          Au[at] = out;
+        }
+        continue;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) Au[(q0 + q) * n + e] = to_vec<R>(o[q]);
   }
   if constexpr (CGT) {
     if (st != nullptr) {

@@ -67,6 +67,7 @@ struct nfs_ctx {
   cudaStream_t stream = nullptr;  // caller's stream
   cudaStream_t work = nullptr;    // the library's own stream (CG and Lanczos; graph capture)
   cudaEvent_t ev = nullptr;
+  cudaEvent_t ev_batch[2] = {nullptr, nullptr};  // GMRES batches whose columns are on the host
   int kind = 0, ax_a = 0, ax_b = 1;
   bool has_mu = false;
   long long gam_len = 0, mat_len = 0;
@@ -88,6 +89,7 @@ struct nfs_ctx {
   // component as 2 x 2 blocks [4 * 3][n]; the Arnoldi and GMRES bases and the
   // device copy of rotation coefficients of the NFSEP eigensolve
   double2* binv64 = nullptr;
+  double* root64 = nullptr;  // diagonal of Sigma_r^{1/2} per voxel
   double2* zv = nullptr;
   double2* gv = nullptr;
   double* zY = nullptr;
@@ -1332,7 +1334,7 @@ void free_ctx(nfs_ctx* c) {
                   c->mat64, c->pmat, c->pmu, c->basis64, c->bloch64, c->lamdf, c->twdf[0], c->twdf[1], c->twdf[2], c->matdf,
                   c->basisdf, c->fld, c->x64, c->r64, c->p64, c->Ap64, c->t64, c->t64b, c->x32, c->r32,
                   c->p32, c->Ap32, c->st, c->d_small, c->d_flags, c->dscratch, c->V, c->MV, c->V32, c->MV32,
-                  c->MV32lo, c->dY, c->binv64, c->zv, c->gv, c->zY};
+                  c->MV32lo, c->dY, c->binv64, c->root64, c->zv, c->gv, c->zY};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->st_host) cudaFreeHost(c->st_host);
@@ -1341,6 +1343,8 @@ void free_ctx(nfs_ctx* c) {
   if (c->hscratch) cudaFreeHost(c->hscratch);
   if (c->work) cudaStreamDestroy(c->work);
   if (c->ev) cudaEventDestroy(c->ev);
+  for (cudaEvent_t e : c->ev_batch)
+    if (e) cudaEventDestroy(e);
   delete c;
 }
 
@@ -1939,26 +1943,40 @@ extern "C" int nfs_gep_residual(nfs_ctx* c, int m, const double* omega, const vo
 
 namespace {
 
-// M y (- sigma v) on the given stream: Sigma^{1/2}, k_rows_in, the column kernel
-// with B^{-1}, k_rows_out, halves exchanged and Sigma^{1/2} (t64 and Ap64 are its temporaries)
-int nfsep_apply(nfs_ctx* c, cudaStream_t s, const double2* y, double2* out, const double2* v, double2 sigma) {
-  cudaError_t e = nfs::nfsep_prescale(y, c->t64, c->lam64, c->n1, c->n2, c->n3, s);
-  if (e != cudaSuccess) return cuda_fail(e, "nfsep prescale");
-  nfs::MatvecArgs<double> a = margs<double>(c, c->t64, c->Ap64, nullptr);
+// M y (- sigma v) on the given stream, with the pieces of a GMRES step in kr
+int nfsep_apply(nfs_ctx* c, cudaStream_t s, const double2* y, double2* out, nfs::KrylovFuse kr) {
+  nfs::MatvecArgs<double> a = margs<double>(c, y, out, nullptr);
   a.stream = s;
-  e = nfs::matvec_launch_mask<double>(a, 1);
+  a.kr = kr;
+  a.kr.root = c->root64;
+  cudaError_t e = nfs::matvec_launch_mask<double>(a, 1);
   if (e != cudaSuccess) return cuda_fail(e, "nfsep rows");
   e = nfs::nfsep_columns(c->fld, c->binv64, c->tw64[0], c->tw64[2], c->n1, c->n3, s);
   if (e != cudaSuccess) return cuda_fail(e, "nfsep columns");
   e = nfs::matvec_launch_mask<double>(a, 4);
   if (e != cudaSuccess) return cuda_fail(e, "nfsep rows out");
-  e = nfs::nfsep_post(c->Ap64, out, c->lam64, c->n1, c->n2, c->n3, v, sigma, s);
-  if (e != cudaSuccess) return cuda_fail(e, "nfsep post");
-  c->launches += 2 + nfs::kProductKernels;
+  c->launches += nfs::kProductKernels;
   return NFS_OK;
 }
 
 using nfs::host::cplxd;
+
+// steps enqueued between two host reads of the Hessenberg columns
+constexpr int kGmresBatch = 10;
+// Scratch of the device GMRES (offsets in doubles into dscratch): the partials
+// of the two Gram-Schmidt passes and of the norm of every step of a batch, the
+// norm partials of a batch's last vector, the least-squares solution, the
+// Hessenberg columns, then the updates' partial sums.
+constexpr size_t kGsPartLen = (size_t)64 * nfs::kGmresMax * 2;
+constexpr size_t kGsNrmLen = 8 * 2 * 128;  // CTAs of k_rows_in
+constexpr size_t kGsNrmOff = 2 * kGmresBatch * kGsPartLen;
+constexpr size_t kGsLastOff = kGsNrmOff + kGmresBatch * kGsNrmLen;
+constexpr size_t kGsYOff = kGsLastOff + 152 * 16 + 128;
+constexpr size_t kGsStateOff = kGsYOff + 2 * nfs::kGmresMax;
+constexpr size_t kGsTmpOff = kGsStateOff + (sizeof(nfs::GmresDev) + 15) / 16 * 2;
+static_assert(kGsYOff % 2 == 0 && kGsStateOff % 2 == 0 && kGsTmpOff % 2 == 0, "16-byte alignment");
+size_t gs_scratch_len(long long N) { return kGsTmpOff + 2 * (size_t)nfs::gs_tmp_len(N); }
+double2* gs_tmp(nfs_ctx* c) { return reinterpret_cast<double2*>(c->dscratch + kGsTmpOff); }
 
 // Long-vector operations of the Krylov drivers on device vectors (P = 1):
 // basis V (vector j at V + j N) and work vector w, on the context's stream.
@@ -1993,8 +2011,13 @@ struct DevBasis : virtual nfs::host::KrylovOps {
   int axpy(int m, const std::vector<cplxd>& cf) override {
     double* dc = c->dscratch;
     TRY(put_coef(cf, dc));
-    CK(nfs::zaxpy_basis(w, V, N, dc, m, 1.0, s));
-    c->launches += 1;
+    auto* tmp = gs_tmp(c);
+    for (int j0 = 0; j0 < m; j0 += nfs::kGmresMax) {
+      int G = 0;
+      CK(nfs::gs_update(V + (long long)j0 * N, std::min(m - j0, nfs::kGmresMax), N, dc + 2 * j0, 1, tmp, &G, s));
+      CK(nfs::gs_finish(w, tmp, G, w, N, nullptr, s));
+      c->launches += 2;
+    }
     CK(cudaStreamSynchronize(s));  // the pinned staging buffer is reused next
     return NFS_OK;
   }
@@ -2049,44 +2072,48 @@ struct DevBasis : virtual nfs::host::KrylovOps {
   }
 };
 
-// Scratch of the device GMRES (offsets in doubles into dscratch): the two
-// Gram-Schmidt passes' partials, the norm partials, the least-squares
-// solution, the GmresDev state, then gs_axpy's partial sums.
-constexpr size_t kGsPartLen = (size_t)64 * nfs::kGmresMax * 2;
-constexpr size_t kGsNrmLen = 152 * 16 + 128;
-constexpr size_t kGsYOff = 2 * kGsPartLen + kGsNrmLen;
-constexpr size_t kGsStateOff = kGsYOff + 2 * nfs::kGmresMax;
-constexpr size_t kGsTmpOff = kGsStateOff + (sizeof(nfs::GmresDev) + 15) / 16 * 2;
-static_assert(kGsYOff % 2 == 0 && kGsStateOff % 2 == 0 && kGsTmpOff % 2 == 0, "16-byte alignment");
-size_t gs_scratch_len(long long N) { return kGsTmpOff + 2 * (size_t)nfs::gs_axpy_tmp_len(N); }
-// steps enqueued between two host reads of the Hessenberg columns
-constexpr int kGmresBatch = 10;
-
-// Steps j0 .. j0 + nsteps - 1 of a GMRES cycle of length m on stream s:
-// w = (M - sigma I) V_j, two classical Gram-Schmidt passes, column j of H,
-// V_{j+1} = w / h_{j+1,j}.
-int enqueue_gmres_steps(nfs_ctx* c, cudaStream_t s, double2 sigma, double2* V, double2* w, int m, int j0, int nsteps) {
+// Steps j0 .. j0 + nsteps - 1 of a GMRES cycle on stream s: w = (M - sigma I)
+// V_j, two classical Gram-Schmidt passes, V_{j+1} = w / h_{j+1,j}; then the
+// batch's columns of H.  V_{j+1} is formed by the next step's product (its last
+// one, not yet normalised, by gs_finish: the next batch's first product
+// normalises it).
+int enqueue_gmres_steps(nfs_ctx* c, cudaStream_t s, double2 sigma, double2* V, double2* w, int j0, int nsteps) {
   const long long N = c->N;
-  double* part1 = c->dscratch;
-  double* part2 = c->dscratch + kGsPartLen;
-  double* nrm = c->dscratch + 2 * kGsPartLen;
+  double* part = c->dscratch;
+  double* nrm = c->dscratch + kGsNrmOff;
+  double* last = c->dscratch + kGsLastOff;
   auto* st = reinterpret_cast<nfs::GmresDev*>(c->dscratch + kGsStateOff);
-  auto* tmp = reinterpret_cast<double2*>(c->dscratch + kGsTmpOff);
-  const int S = nfs::gs_chunks(N), nb = nfs::gs_norm_blocks(N);
-  for (int j = j0; j < j0 + nsteps; ++j) {
-    const double2* vj = V + (long long)j * N;
-    TRY(nfsep_apply(c, s, vj, w, vj, sigma));
-    CK(nfs::gs_dots(V, j + 1, w, N, part1, s));
-    CK(nfs::gs_axpy(w, V, N, j + 1, part1, nullptr, tmp, s));
-    CK(nfs::gs_dots(V, j + 1, w, N, part2, s));
-    CK(nfs::gs_axpy(w, V, N, j + 1, part2, nrm, tmp, s));
-    CK(nfs::gmres_column(j, part1, part2, S, nrm, nb, st, s));
-    c->launches += 3 + 2 * nfs::gs_axpy_kernels(N);
-    if (j + 1 < m) {
-      CK(nfs::gmres_store(w, V + (long long)(j + 1) * N, st, N, s));
-      c->launches += 1;
+  double2* tmp = gs_tmp(c);
+  double2* w2 = c->t64;
+  const int S = nfs::gs_chunks(N), nlast = nfs::gs_norm_blocks(N), nnrm = nfs::cg_partials<double>(c->n1, c->n3);
+  int G = 0;
+  for (int t = 0; t < nsteps; ++t) {
+    const int j = j0 + t;
+    double2* vj = V + (long long)j * N;
+    nfs::KrylovFuse kr;
+    kr.v = vj;
+    kr.sigma = sigma;
+    if (t > 0) {
+      kr.tmp = tmp;
+      kr.groups = G;
+      kr.nrm_out = nrm + (t - 1) * kGsNrmLen;
+      kr.nrm = kr.nrm_out;
+      kr.nnrm = nnrm;
+    } else if (j > 0) {
+      kr.nrm = last;
+      kr.nnrm = nlast;
     }
+    TRY(nfsep_apply(c, s, t > 0 ? w2 : vj, w, kr));
+    double* p1 = part + 2 * t * kGsPartLen;
+    CK(nfs::gs_dots(V, j + 1, w, nullptr, 0, nullptr, N, p1, s));
+    CK(nfs::gs_update(V, j + 1, N, p1, S, tmp, &G, s));
+    CK(nfs::gs_dots(V, j + 1, w, tmp, G, w2, N, p1 + kGsPartLen, s));
+    CK(nfs::gs_update(V, j + 1, N, p1 + kGsPartLen, S, tmp, &G, s));
+    c->launches += 4;
   }
+  CK(nfs::gs_finish(w2, tmp, G, V + (long long)(j0 + nsteps) * N, N, last, s));
+  CK(nfs::gmres_columns(j0, nsteps, part, kGsPartLen, S, nrm, kGsNrmLen, nnrm, last, nlast, st, s));
+  c->launches += 2;
   return NFS_OK;
 }
 
@@ -2098,7 +2125,7 @@ int enqueue_gmres_steps(nfs_ctx* c, cudaStream_t s, double2 sigma, double2* V, d
 #define NFS_GMRES_GRAPH 1
 #endif
 int gmres_steps(nfs_ctx* c, cudaStream_t s, double2 sigma, double2* V, double2* w, int m, int j0, int nsteps) {
-  if (!NFS_GMRES_GRAPH) return enqueue_gmres_steps(c, s, sigma, V, w, m, j0, nsteps);
+  if (!NFS_GMRES_GRAPH) return enqueue_gmres_steps(c, s, sigma, V, w, j0, nsteps);
   // one set of batches is kept: a new shift or buffer replaces it
   if (!c->gm_graphs.empty()) {
     const GmresGraph& f = c->gm_graphs.front();
@@ -2117,7 +2144,7 @@ int gmres_steps(nfs_ctx* c, cudaStream_t s, double2 sigma, double2* V, double2* 
   const long long l0 = c->launches;
   cudaGraph_t graph = nullptr;
   CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-  const int rc = enqueue_gmres_steps(c, s, sigma, V, w, m, j0, nsteps);
+  const int rc = enqueue_gmres_steps(c, s, sigma, V, w, j0, nsteps);
   cudaError_t e2 = cudaStreamEndCapture(s, &graph);
   const long long kernels = c->launches - l0;
   c->launches = l0;
@@ -2149,7 +2176,7 @@ int dev_gmres(nfs_ctx* c, const double2* b, double2* x, double2 sigma, double2* 
   if (!(bnorm > 0.0)) return NFS_OK;
   cudaStream_t s = c->work;
   const long long N = c->N;
-  double* nrm = c->dscratch + 2 * kGsPartLen;
+  double* nrm = c->dscratch + kGsLastOff;
   double* yd = c->dscratch + kGsYOff;
   auto* st = reinterpret_cast<nfs::GmresDev*>(c->dscratch + kGsStateOff);
   const int nb = nfs::gs_norm_blocks(N);
@@ -2159,7 +2186,10 @@ int dev_gmres(nfs_ctx* c, const double2* b, double2* x, double2 sigma, double2* 
   std::vector<nfs::host::cplxd> col(kCol), y;
   for (;;) {
     // r = b - (M - sigma I) x; V_0 = r / ||r||
-    TRY(nfsep_apply(c, s, x, w, x, sigma));
+    nfs::KrylovFuse kr;
+    kr.v = x;
+    kr.sigma = sigma;
+    TRY(nfsep_apply(c, s, x, w, kr));
     CK(nfs::gmres_residual(b, w, N, nrm, s));
     c->launches += 1;
     CK(cudaMemcpyAsync(c->hscratch, nrm, nb * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -2173,40 +2203,53 @@ int dev_gmres(nfs_ctx* c, const double2* b, double2* x, double2 sigma, double2* 
       out.status = NFS_ENOCONV;
       return NFS_OK;
     }
-    CK(cudaMemsetAsync(st, 0, 2 * sizeof(double2), s));  // done, inv_h
     CK(nfs::zscale_copy(w, V, 1.0 / beta, N, s));
     c->launches += 1;
     ls.reset(m, beta);
-    int j = 0;
+    // the host reads a batch's columns while the next batch runs; a batch that
+    // was enqueued past the converged column is thrown away (and not counted)
+    int queued = 0, steps_of[2] = {0, 0};
     bool done = false;
-    while (j < m && out.iterations < maxit && !done) {
-      const int steps = std::min({kGmresBatch, m - j, maxit - out.iterations});
-      TRY(gmres_steps(c, s, sigma, V, w, m, j, steps));
+    auto enqueue = [&](int slot) -> int {
+      const int steps = std::min({kGmresBatch, m - queued, maxit - out.iterations - (queued - ls.columns())});
+      steps_of[slot] = std::max(steps, 0);
+      if (steps <= 0) return NFS_OK;
+      TRY(gmres_steps(c, s, sigma, V, w, m, queued, steps));
       const auto* hc_dev = reinterpret_cast<const double2*>(reinterpret_cast<const char*>(st) +
                                                              offsetof(nfs::GmresDev, Hc));
-      CK(cudaMemcpyAsync(c->hscratch, hc_dev + (size_t)j * kCol, (size_t)steps * kCol * sizeof(double2),
-                         cudaMemcpyDeviceToHost, s));
-      CK(cudaStreamSynchronize(s));
+      CK(cudaMemcpyAsync(c->hscratch + (size_t)slot * kGmresBatch * kCol * 2, hc_dev + (size_t)queued * kCol,
+                         (size_t)steps * kCol * sizeof(double2), cudaMemcpyDeviceToHost, s));
+      CK(cudaEventRecord(c->ev_batch[slot], s));
+      queued += steps;
+      return NFS_OK;
+    };
+    TRY(enqueue(0));
+    for (int slot = 0; steps_of[slot] > 0 && !done; slot ^= 1) {
+      const int steps = steps_of[slot], j = ls.columns();
+      TRY(enqueue(slot ^ 1));
+      CK(cudaEventSynchronize(c->ev_batch[slot]));
       for (int t = 0; t < steps && !done; ++t) {
-        const double* hc = c->hscratch + (size_t)t * kCol * 2;
+        const double* hc = c->hscratch + ((size_t)slot * kGmresBatch + t) * kCol * 2;
         const int jj = j + t;
         for (int i = 0; i <= jj; ++i) col[i] = nfs::host::cplxd(hc[2 * i], hc[2 * i + 1]);
         const double h = hc[2 * (jj + 1)];
         const double res = ls.add_column(col.data(), h);
         done = res <= tolb || h == 0.0;
       }
-      j += steps;
       out.iterations += steps;
     }
+    CK(cudaStreamSynchronize(s));  // (a batch thrown away still writes the staging buffer)
     // y = R^{-1} g over the cycle's columns, x += V y
     if (!ls.solve(y)) return NFS_EBREAKDOWN;
     for (size_t i = 0; i < y.size(); ++i) {
-      c->hscratch[2 * i] = y[i].real();
-      c->hscratch[2 * i + 1] = y[i].imag();
+      c->hscratch[2 * i] = -y[i].real();
+      c->hscratch[2 * i + 1] = -y[i].imag();
     }
     CK(cudaMemcpyAsync(yd, c->hscratch, y.size() * sizeof(double2), cudaMemcpyHostToDevice, s));
-    CK(nfs::zaxpy_basis(x, V, N, yd, ls.columns(), -1.0, s));
-    c->launches += 1;
+    int G = 0;
+    CK(nfs::gs_update(V, ls.columns(), N, yd, 1, gs_tmp(c), &G, s));
+    CK(nfs::gs_finish(x, gs_tmp(c), G, x, N, nullptr, s));
+    c->launches += 2;
     CK(cudaStreamSynchronize(s));  // the pinned staging buffer is reused next
     ++out.restarts;
   }
@@ -2324,7 +2367,11 @@ extern "C" int nfs_setup_biiso(nfs_ctx** out, const int grid[3], const double* l
   const int rc = [&]() -> int {
     TRY(dalloc(c, &c->binv64, binv.size()));
     CK(cudaMemcpy(c->binv64, binv.data(), binv.size() * sizeof(double2), cudaMemcpyHostToDevice));
+    TRY(dalloc(c, &c->root64, (size_t)n));
+    CK(nfs::nfsep_root(c->lam64, c->n1, c->n2, c->n3, c->root64, 0));
     CK(nfs::nfsep_prepare(c->n1, c->n3));
+    for (cudaEvent_t& e : c->ev_batch) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    CK(cudaDeviceSynchronize());
     return NFS_OK;
   }();
   if (rc != NFS_OK) {
@@ -2339,7 +2386,7 @@ extern "C" int nfs_nfsep_matvec(nfs_ctx* c, const void* y, void* My) {
   if (!c || !y || !My || y == My) return NFS_EINVAL;
   if (!c->binv64) return NFS_EUNSUPPORTED;
   if (((uintptr_t)y | (uintptr_t)My) & 15) return NFS_EINVAL;
-  return nfsep_apply(c, c->stream, (const double2*)y, (double2*)My, nullptr, make_double2(0.0, 0.0));
+  return nfsep_apply(c, c->stream, (const double2*)y, (double2*)My, nfs::KrylovFuse{});
 }
 
 extern "C" int nfs_nfsep_eigs(nfs_ctx* c, int nev, const double sigma[2], double* omega, void* Y,
@@ -2400,16 +2447,14 @@ extern "C" int nfs_nfsep_fields(nfs_ctx* c, int m, const void* Yv, void* Xv) {
   const long long n = c->n, N = c->N;
   for (int j = 0; j < m; ++j) {
     // Algorithm 1, second branch: y <- Sigma^{1/2} y, x = B^{-1} diag(P_r, Q_r) y
-    cudaError_t e = nfs::nfsep_prescale((const double2*)Yv + (long long)j * N, c->t64, c->lam64, c->n1, c->n2,
-                                        c->n3, c->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "nfsep fields prescale");
-    nfs::MatvecArgs<double> a = margs<double>(c, c->t64, nullptr, nullptr);
-    e = nfs::matvec_launch_mask<double>(a, 1);
+    nfs::MatvecArgs<double> a = margs<double>(c, (const double2*)Yv + (long long)j * N, nullptr, nullptr);
+    a.kr.root = c->root64;
+    cudaError_t e = nfs::matvec_launch_mask<double>(a, 1);
     if (e != cudaSuccess) return cuda_fail(e, "nfsep fields rows");
     e = nfs::nfsep_fields(c->fld, c->binv64, c->tw64[0], c->tw64[2], c->bloch64, c->n1, c->n3,
                           (double2*)Xv + (long long)j * 6 * n, c->stream);
     if (e != cudaSuccess) return cuda_fail(e, "nfsep fields");
-    c->launches += 3;
+    c->launches += 2;
   }
   return NFS_OK;
 }

@@ -12,29 +12,13 @@ namespace nfs {
 
 namespace {
 
-__device__ __forceinline__ double quarter_root_lq(const double2* lam, int n1, int n2, long long e) {
-  const int i1 = (int)(e % n1);
-  const int i2 = (int)((e / n1) % n2);
-  const int i3 = (int)(e / ((long long)n1 * n2));
-  const double lq = cabs2(lam[i1]) + cabs2(lam[n1 + i2]) + cabs2(lam[n1 + n2 + i3]);
-  return sqrt(sqrt(lq));
-}
-
-__global__ void k_nfsep_prescale(const double2* __restrict__ y, double2* __restrict__ t,
-                                 const double2* __restrict__ lam, int n1, int n2, long long n) {
-  for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < 4 * n; g += (long long)gridDim.x * blockDim.x) {
-    const long long e = g % n;
-    t[g] = cscale(y[g], quarter_root_lq(lam, n1, n2, e));
-  }
-}
-
-__global__ void k_nfsep_post(const double2* __restrict__ a, double2* __restrict__ out, const double2* __restrict__ lam,
-                             int n1, int n2, long long n, const double2* __restrict__ v, double2 sigma) {
-  for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < 4 * n; g += (long long)gridDim.x * blockDim.x) {
-    const long long q = g / n, e = g % n;
-    double2 r = cscale(a[((q + 2) & 3) * n + e], quarter_root_lq(lam, n1, n2, e));
-    if (v != nullptr) r = csub(r, cmul(sigma, v[g]));
-    out[g] = r;
+__global__ void k_nfsep_root(const double2* __restrict__ lam, int n1, int n2, long long n, double* __restrict__ root) {
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
+    const int i1 = (int)(e % n1);
+    const int i2 = (int)((e / n1) % n2);
+    const int i3 = (int)(e / ((long long)n1 * n2));
+    const double lq = cabs2(lam[i1]) + cabs2(lam[n1 + i2]) + cabs2(lam[n1 + n2 + i3]);
+    root[e] = sqrt(sqrt(lq));
   }
 }
 
@@ -83,19 +67,6 @@ struct NfsepFieldsStep : BinvStep {
   }
 };
 
-__global__ void k_zaxpy_basis(double2* __restrict__ w, const double2* __restrict__ V, long long N,
-                              const double* __restrict__ c, int m, double sign) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  double2* cs = reinterpret_cast<double2*>(smem_raw);
-  for (int j = threadIdx.x; j < m; j += blockDim.x) cs[j] = make_double2(sign * c[2 * j], sign * c[2 * j + 1]);
-  __syncthreads();
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    double2 a = w[i];
-    for (int j = 0; j < m; ++j) a = csub(a, cmul(cs[j], V[(long long)j * N + i]));
-    w[i] = a;
-  }
-}
-
 __global__ void k_zscale_copy(const double2* __restrict__ src, double2* __restrict__ dst, double scale, long long N) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x)
     dst[i] = cscale(src[i], scale);
@@ -129,210 +100,231 @@ __global__ void k_zrotate(double2* __restrict__ V, int m, const double* __restri
 }
 
 // --- device-resident GMRES -------------------------------------------------
+//
+// A step is seven kernels: the three of the product (which also end the
+// Gram-Schmidt update of the step before and normalise its vector, KrylovFuse)
+// and dots, update, dots, update.  At 8^3 (2048 elements, up to 101 basis
+// vectors) every one is a chain of latencies and FP64 instructions, so the work
+// is spread over as many SMs as the vectors allow: the dots over element tiles
+// and groups of 8 vectors, the updates over elements and groups of vectors,
+// whose partial sums the next kernel adds up (w - sum_g tmp_g).  One GB300, a
+// step at 8^3: 62 us with fourteen kernels (separate scalings, sums over the
+// groups, norm column and store), 38 us now.
 
-constexpr int kGsChunk = 512;   // elements of one dot-product chunk
-constexpr int kGsMaxChunks = 64;
 constexpr int kGsThreads = 256;
+constexpr int kGsTile = 128;      // elements of w that a block of k_gs_dots holds
+constexpr int kGsMaxChunks = 64;
+constexpr int kGsPerWarp = 2;     // vectors per warp (4: the FP64 work of a block takes 3 us instead of 1.9)
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
+// (The kernels fetch what they need of the older basis vectors before they wait
+// for the kernel before them: those vectors were complete when that kernel
+// passed its own wait, which is before it let this one start.)
 
-// sum over the block (blockDim.x = kGsThreads); the result in every thread
-__device__ __forceinline__ double gs_block_sum(double v, double* red) {
-  v = warp_sum(v);
-  const int wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) red[wi] = v;
-  __syncthreads();
-  double t = 0.0;
-#pragma unroll
-  for (int i = 0; i < kGsThreads / 32; ++i) t += red[i];
-  return t;
-}
-
-// grid (S, ceil(m / 8)): warp wi of block (s, b) forms chunk s of V_j^* w, j = 8 b + wi
-__global__ void __launch_bounds__(kGsThreads)
-k_gs_dots(const double2* __restrict__ V, int m, const double2* __restrict__ w, long long N, long long chunk,
-          double* __restrict__ part) {
-  const int j = blockIdx.y * (kGsThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (j >= m) return;  // whole warps
+// grid (S, ceil(m / 8)): part[(s m + j) 2 + {0, 1}] = chunk s's share of
+// V_j^* w', w' = w - sum_{g < G} tmp_g (written to w2 when G > 0)
+__global__ void __launch_bounds__(kGsTile)
+k_gs_dots(const double2* __restrict__ V, int m, const double2* w, const double2* tmp, int G, double2* w2, long long N,
+          long long chunk, double* __restrict__ part) {
+  constexpr int PER = kGsTile / 32;  // elements of a tile per lane
+  __shared__ double2 ws[kGsTile];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int j0 = (blockIdx.y * (kGsTile / 32) + warp) * kGsPerWarp;
   const int s = blockIdx.x;
   const long long i0 = (long long)s * chunk, i1 = min(N, i0 + chunk);
-  const double2* v = V + (long long)j * N;
-  double re = 0.0, im = 0.0;
-#pragma unroll 4
-  for (long long i = i0 + lane; i < i1; i += 32) {
-    const double2 a = v[i], b = w[i];
-    re += a.x * b.x + a.y * b.y;
-    im += a.x * b.y - a.y * b.x;
+  double2 x[kGsPerWarp][PER];
+  auto fetch = [&](long long base, int from, int to) {
+#pragma unroll
+    for (int t = 0; t < kGsPerWarp; ++t)
+      if (j0 + t >= from && j0 + t < to)
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+          const long long i = base + k * 32 + lane;
+          x[t][k] = i < i1 ? V[(long long)(j0 + t) * N + i] : make_double2(0.0, 0.0);
+        }
+  };
+  fetch(i0, 0, m - 1);  // (the newest vector may still be being normalised)
+  depend_wait();
+  fetch(i0, m - 1, m);
+  double acc[2 * kGsPerWarp];
+#pragma unroll
+  for (int t = 0; t < 2 * kGsPerWarp; ++t) acc[t] = 0.0;
+  for (long long base = i0; base < i1; base += kGsTile) {
+    const long long i = base + threadIdx.x;
+    double2 a = make_double2(0.0, 0.0);
+    if (i < i1) {
+      a = minus_groups(w[i], tmp + i, N, G);
+      if (G > 0 && blockIdx.y == 0) w2[i] = a;
+    }
+    if (base > i0) {
+      fetch(base, 0, m);
+      __syncthreads();  // the tile before has been read
+    }
+    ws[threadIdx.x] = a;
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < kGsPerWarp; ++t)
+      if (j0 + t < m)
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+          const double2 v = x[t][k], y = ws[k * 32 + lane];
+          acc[2 * t] += v.x * y.x + v.y * y.y;
+          acc[2 * t + 1] += v.x * y.y - v.y * y.x;
+        }
   }
-  re = warp_sum(re);
-  im = warp_sum(im);
-  if (lane == 0) {
-    part[((long long)s * m + j) * 2] = re;
-    part[((long long)s * m + j) * 2 + 1] = im;
+  depend_begin();
+  // the four sums over the 32 lanes at once: two halving exchanges leave each
+  // eight lanes with one of the four values, three more steps complete it (six
+  // FP64 additions instead of twenty)
+#pragma unroll
+  for (int h = kGsPerWarp, o = 16; h >= 1; h >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int t = 0; t < h; ++t) {
+      const double keep = up ? acc[t + h] : acc[t], give = up ? acc[t] : acc[t + h];
+      acc[t] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
   }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+  static_assert(kGsPerWarp == 2, "two exchanges");
+  const int which = ((lane >> 4) & 1) * 2 + ((lane >> 3) & 1);
+  if ((lane & 7) == 0 && j0 + which / 2 < m) part[((long long)s * m + j0) * 2 + which] = acc[0];
 }
 
-__global__ void __launch_bounds__(kGsThreads)
-k_gs_axpy(double2* __restrict__ w, const double2* __restrict__ V, long long N, int m, const double* __restrict__ part,
-          int S, double* __restrict__ nrm_part) {
+// grid (ceil(N / NT), G): tmp[g N + i] = sum over the g-th group of VB basis
+// vectors of c_j V_j[i], c_j = sum over the S chunks' partials
+template <int NT>
+__global__ void __launch_bounds__(NT)
+k_gs_update(const double2* __restrict__ V, long long N, int m, int VB, const double* part, int S, double2* tmp) {
+  constexpr int AHEAD = 12;  // vectors fetched before the wait
   __shared__ double2 cs[kGmresMax];
-  __shared__ double red[kGsThreads / 32];
-  for (int j = threadIdx.x; j < m; j += kGsThreads) {
+  const int j0 = blockIdx.y * VB, nj = min(VB, m - j0);
+  const long long i = (long long)blockIdx.x * NT + threadIdx.x;
+  const double2* v = V + (long long)j0 * N + (i < N ? i : 0);
+  double2 x[AHEAD];
+#pragma unroll
+  for (int t = 0; t < AHEAD; ++t)
+    if (t < nj) x[t] = v[(long long)t * N];
+  depend_wait();
+  // four threads add up one coefficient
+  for (int t = threadIdx.x; t < (nj + NT / 4 - 1) / (NT / 4) * NT; t += NT) {
+    const int j = t / 4;
     double re = 0.0, im = 0.0;
-    for (int q = 0; q < S; ++q) {
-      re += part[((long long)q * m + j) * 2];
-      im += part[((long long)q * m + j) * 2 + 1];
-    }
-    cs[j] = make_double2(re, im);
-  }
-  __syncthreads();
-  double nr = 0.0;
-  for (long long i = (long long)blockIdx.x * kGsThreads + threadIdx.x; i < N; i += (long long)gridDim.x * kGsThreads) {
-    // eight basis loads in flight per round, two accumulators
-    double2 a0 = w[i], a1 = make_double2(0.0, 0.0);
-    int j = 0;
-    for (; j + 8 <= m; j += 8) {
-      double2 v[8];
-#pragma unroll
-      for (int t = 0; t < 8; ++t) v[t] = V[(long long)(j + t) * N + i];
-#pragma unroll
-      for (int t = 0; t < 8; t += 2) {
-        a0 = csub(a0, cmul(cs[j + t], v[t]));
-        a1 = csub(a1, cmul(cs[j + t + 1], v[t + 1]));
+    if (j < nj) {
+      const double2* p = reinterpret_cast<const double2*>(part) + j0 + j;
+#pragma unroll 4
+      for (int q = t % 4; q < S; q += 4) {
+        const double2 y = p[(long long)q * m];
+        re += y.x;
+        im += y.y;
       }
     }
-    for (; j < m; ++j) a0 = csub(a0, cmul(cs[j], V[(long long)j * N + i]));
-    const double2 a = cadd(a0, a1);
-    w[i] = a;
-    nr += cabs2(a);
-  }
-  if (nrm_part) {
-    nr = gs_block_sum(nr, red);
-    if (threadIdx.x == 0) nrm_part[blockIdx.x] = nr;
-  }
-}
-
-// Short vectors: grid (ceil(N / kGsThreads), chunks of kGsAxpyChunk basis
-// vectors); tmp[jc N + i] = sum over chunk jc of c_j V_j[i]
-constexpr int kGsAxpyChunk = 16;
-__global__ void __launch_bounds__(kGsThreads)
-k_gs_axpy_part(const double2* __restrict__ V, long long N, int m, const double* __restrict__ part, int S,
-               double2* __restrict__ tmp) {
-  __shared__ double2 cs[kGsAxpyChunk];
-  const int j0 = blockIdx.y * kGsAxpyChunk;
-  const int nj = min(kGsAxpyChunk, m - j0);
-  if (threadIdx.x < nj) {
-    double re = 0.0, im = 0.0;
-    for (int q = 0; q < S; ++q) {
-      re += part[((long long)q * m + j0 + threadIdx.x) * 2];
-      im += part[((long long)q * m + j0 + threadIdx.x) * 2 + 1];
+#pragma unroll
+    for (int o = 2; o > 0; o >>= 1) {
+      re += __shfl_xor_sync(0xffffffffu, re, o);
+      im += __shfl_xor_sync(0xffffffffu, im, o);
     }
-    cs[threadIdx.x] = make_double2(re, im);
+    if (t % 4 == 0 && j < nj) cs[j] = make_double2(re, im);
   }
   __syncthreads();
-  const long long i = (long long)blockIdx.x * kGsThreads + threadIdx.x;
+  depend_begin();
   if (i >= N) return;
-  double2 v[kGsAxpyChunk];
+  double2 a0 = make_double2(0.0, 0.0), a1 = a0;
 #pragma unroll
-  for (int t = 0; t < kGsAxpyChunk; ++t) v[t] = t < nj ? V[(long long)(j0 + t) * N + i] : make_double2(0.0, 0.0);
-  double2 a0 = make_double2(0.0, 0.0), a1 = make_double2(0.0, 0.0);
-#pragma unroll
-  for (int t = 0; t < kGsAxpyChunk; t += 2) {
-    if (t < nj) a0 = cadd(a0, cmul(cs[t], v[t]));
-    if (t + 1 < nj) a1 = cadd(a1, cmul(cs[t + 1], v[t + 1]));
+  for (int t = 0; t < AHEAD; t += 2) {
+    if (t < nj) a0 = cadd(a0, cmul(cs[t], x[t]));
+    if (t + 1 < nj) a1 = cadd(a1, cmul(cs[t + 1], x[t + 1]));
   }
+  int j = AHEAD;
+  for (; j + 8 <= nj; j += 8) {
+    double2 y[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) y[t] = v[(long long)(j + t) * N];
+#pragma unroll
+    for (int t = 0; t < 8; t += 2) {
+      a0 = cadd(a0, cmul(cs[j + t], y[t]));
+      a1 = cadd(a1, cmul(cs[j + t + 1], y[t + 1]));
+    }
+  }
+  for (; j < nj; ++j) a0 = cadd(a0, cmul(cs[j], v[(long long)j * N]));
   tmp[(long long)blockIdx.y * N + i] = cadd(a0, a1);
 }
 
-// w -= sum over the JC partial sums in tmp, and the partials of ||w||^2
+// sum over the block (blockDim.x = kGsThreads); the result in every thread
+__device__ __forceinline__ double gs_block_sum(double v) {
+  RedAcc<double> a;
+  a.v = v;
+  return a.block_total<kGsThreads>();
+}
+
+// dst = w - sum_g tmp_g, and (nrm_part != nullptr) the partials of |dst|^2
 __global__ void __launch_bounds__(kGsThreads)
-k_gs_axpy_sum(double2* __restrict__ w, long long N, const double2* __restrict__ tmp, int JC,
-              double* __restrict__ nrm_part) {
-  __shared__ double red[kGsThreads / 32];
+k_gs_finish(const double2* w, const double2* __restrict__ tmp, int G, double2* dst, long long N,
+            double* __restrict__ nrm_part) {
+  depend_wait();
   double nr = 0.0;
   for (long long i = (long long)blockIdx.x * kGsThreads + threadIdx.x; i < N; i += (long long)gridDim.x * kGsThreads) {
-    double2 a = w[i];
-    for (int jc = 0; jc < JC; ++jc) a = csub(a, tmp[(long long)jc * N + i]);
-    w[i] = a;
+    const double2 a = minus_groups(w[i], tmp + i, N, G);
+    dst[i] = a;
     nr += cabs2(a);
   }
+  depend_begin();
   if (nrm_part) {
-    nr = gs_block_sum(nr, red);
+    nr = gs_block_sum(nr);
     if (threadIdx.x == 0) nrm_part[blockIdx.x] = nr;
   }
 }
 
 __global__ void __launch_bounds__(kGsThreads)
 k_gmres_residual(const double2* __restrict__ b, double2* __restrict__ w, long long N, double* __restrict__ nrm_part) {
-  __shared__ double red[kGsThreads / 32];
   double nr = 0.0;
   for (long long i = (long long)blockIdx.x * kGsThreads + threadIdx.x; i < N; i += (long long)gridDim.x * kGsThreads) {
     const double2 a = csub(b[i], w[i]);
     w[i] = a;
     nr += cabs2(a);
   }
-  nr = gs_block_sum(nr, red);
+  nr = gs_block_sum(nr);
   if (threadIdx.x == 0) nrm_part[blockIdx.x] = nr;
 }
 
-__device__ __forceinline__ double gs_sum_partials(const double* part, int nb, double* red) {
-  double t = 0.0;
-  for (int b = threadIdx.x; b < nb; b += kGsThreads) t += part[b];
-  return gs_block_sum(t, red);
-}
-
+// Columns j0 .. j0 + gridDim.x - 1 of H from their steps' partials: step t's
+// two passes at part + 2 t plen (and + plen), its norm partials at nrm + t nlen
+// (nnrm of them; the last step's at nrm_last, nlast of them).
 __global__ void __launch_bounds__(kGsThreads)
-k_gmres_column(int j, const double* __restrict__ part1, const double* __restrict__ part2, int S,
-               const double* __restrict__ nrm_part, int nb, GmresDev* st) {
-  __shared__ double red[kGsThreads / 32];
-  if (st->done) {  // the same value in every thread: nothing below writes it before this point
-    if (threadIdx.x == 0) st->inv_h = 0.0;
-    return;
-  }
-  const int m = j + 1;  // vectors the two passes ran over
+k_gmres_columns(int j0, const double* __restrict__ part, long long plen, int S, const double* __restrict__ nrm,
+                long long nlen, int nnrm, const double* __restrict__ nrm_last, int nlast, GmresDev* st) {
+  depend_wait();
+  depend_begin();
+  const int t = blockIdx.x, j = j0 + t, m = j + 1;
+  const double* p1 = part + 2 * t * plen;
+  const double* p2 = p1 + plen;
   double2* col = st->Hc + (long long)j * (kGmresMax + 1);
   for (int i = threadIdx.x; i < m; i += kGsThreads) {
     double re = 0.0, im = 0.0;
+#pragma unroll 4
     for (int q = 0; q < S; ++q) {
-      re += part1[((long long)q * m + i) * 2] + part2[((long long)q * m + i) * 2];
-      im += part1[((long long)q * m + i) * 2 + 1] + part2[((long long)q * m + i) * 2 + 1];
+      const double2 x = reinterpret_cast<const double2*>(p1)[(long long)q * m + i];
+      const double2 y = reinterpret_cast<const double2*>(p2)[(long long)q * m + i];
+      re += x.x + y.x;
+      im += x.y + y.y;
     }
     col[i] = make_double2(re, im);
   }
-  const double h = sqrt(fmax(gs_sum_partials(nrm_part, nb, red), 0.0));
-  if (threadIdx.x == 0) {
-    col[j + 1] = make_double2(h, 0.0);
-    st->done = h == 0.0 ? 1 : 0;
-    st->inv_h = h > 0.0 ? 1.0 / h : 0.0;
-  }
-}
-
-__global__ void k_gmres_store(const double2* __restrict__ w, double2* __restrict__ dst, const GmresDev* st, long long N) {
-  const double sc = st->inv_h;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x)
-    dst[i] = cscale(w[i], sc);
+  const bool last = t == (int)gridDim.x - 1;
+  const double* np = last ? nrm_last : nrm + t * nlen;
+  double h = 0.0;
+  for (int i = threadIdx.x; i < (last ? nlast : nnrm); i += kGsThreads) h += np[i];
+  h = sqrt(fmax(gs_block_sum(h), 0.0));
+  if (threadIdx.x == 0) col[j + 1] = make_double2(h, 0.0);
 }
 
 int blocks_for(long long work) { return (int)std::max<long long>(1, std::min<long long>((work + 255) / 256, 152LL * 16)); }
 
 }  // namespace
 
-cudaError_t nfsep_prescale(const double2* y, double2* t, const double2* lam, int n1, int n2, int n3,
-                           cudaStream_t s) {
+cudaError_t nfsep_root(const double2* lam, int n1, int n2, int n3, double* root, cudaStream_t s) {
   const long long n = (long long)n1 * n2 * n3;
-  k_nfsep_prescale<<<blocks_for(4 * n), 256, 0, s>>>(y, t, lam, n1, n2, n);
-  return cudaGetLastError();
-}
-
-cudaError_t nfsep_post(const double2* a, double2* out, const double2* lam, int n1, int n2, int n3,
-                       const double2* v, double2 sigma, cudaStream_t s) {
-  const long long n = (long long)n1 * n2 * n3;
-  k_nfsep_post<<<blocks_for(4 * n), 256, 0, s>>>(a, out, lam, n1, n2, n, v, sigma);
+  k_nfsep_root<<<blocks_for(n), 256, 0, s>>>(lam, n1, n2, n, root);
   return cudaGetLastError();
 }
 
@@ -363,13 +355,6 @@ cudaError_t nfsep_fields(void* fld, const double2* binv, const double2* tw1, con
   return columns_launch<double>(fld, step, tw1, tw3, n1, n3, 1, nullptr, nullptr, BatchStrides{}, s);
 }
 
-cudaError_t zaxpy_basis(double2* w, const double2* V, long long N, const double* c, int m, double sign,
-                        cudaStream_t s) {
-  if (m <= 0) return cudaSuccess;
-  k_zaxpy_basis<<<blocks_for(N), 256, (size_t)m * sizeof(double2), s>>>(w, V, N, c, m, sign);
-  return cudaGetLastError();
-}
-
 cudaError_t zscale_copy(const double2* src, double2* dst, double scale, long long N, cudaStream_t s) {
   k_zscale_copy<<<blocks_for(N), 256, 0, s>>>(src, dst, scale, N);
   return cudaGetLastError();
@@ -386,59 +371,58 @@ cudaError_t zrotate(double2* V, int m, const double* Y, int k, long long N, cuda
 }
 
 int gs_chunks(long long N) {
-  return (int)std::min<long long>(kGsMaxChunks, std::max<long long>(1, (N + kGsChunk - 1) / kGsChunk));
+  return (int)std::min<long long>(kGsMaxChunks, (N + kGsTile - 1) / kGsTile);
 }
-
 int gs_norm_blocks(long long N) { return blocks_for(N); }
 
-// vectors shorter than this split the basis sum of gs_axpy across blocks
-constexpr long long kGsSplitN = 152LL * 2 * kGsThreads;
-
-long long gs_axpy_tmp_len(long long N) {
-  return N < kGsSplitN ? (long long)((kGmresMax + kGsAxpyChunk - 1) / kGsAxpyChunk) * N : 0;
+// Vector groups of the update: enough that the GPU has about four warps per SM
+// (grids up to 24^3 or so), one for longer vectors
+static int gs_groups(long long N, int m) {
+  const long long warps = (N + 31) / 32;
+  return (int)std::max<long long>(1, std::min<long long>((m + 7) / 8, 152 * 4 / warps));
 }
+long long gs_tmp_len(long long N) { return (long long)gs_groups(N, kGmresMax) * N; }
+// kernels of vectors this short overlap (see depend_wait)
+static bool gs_serial(long long N) { return N >= 152LL * 256; }
 
-cudaError_t gs_dots(const double2* V, int m, const double2* w, long long N, double* part, cudaStream_t s) {
+cudaError_t gs_dots(const double2* V, int m, const double2* w, const double2* tmp, int G, double2* w2, long long N,
+                    double* part, cudaStream_t s) {
   if (m <= 0 || m > kGmresMax) return cudaErrorInvalidValue;
   const int S = gs_chunks(N);
-  const long long chunk = (N + S - 1) / S;
-  const dim3 grid(S, (m + kGsThreads / 32 - 1) / (kGsThreads / 32));
-  k_gs_dots<<<grid, kGsThreads, 0, s>>>(V, m, w, N, chunk, part);
-  return cudaGetLastError();
+  const long long chunk = ((N + S - 1) / S + kGsTile - 1) / kGsTile * kGsTile;
+  return launch_dependent(gs_serial(N), k_gs_dots, dim3(S, (m + 7) / 8), kGsTile, 0, s, V, m, w, tmp, G, w2, N,
+                          chunk, part);
 }
 
-cudaError_t gs_axpy(double2* w, const double2* V, long long N, int m, const double* part, double* nrm_part,
-                    double2* tmp, cudaStream_t s) {
+cudaError_t gs_update(const double2* V, int m, long long N, const double* part, int S, double2* tmp, int* groups,
+                      cudaStream_t s) {
   if (m <= 0 || m > kGmresMax) return cudaErrorInvalidValue;
-  if (N < kGsSplitN) {
-    if (tmp == nullptr) return cudaErrorInvalidValue;
-    const int JC = (m + kGsAxpyChunk - 1) / kGsAxpyChunk;
-    k_gs_axpy_part<<<dim3((unsigned)((N + kGsThreads - 1) / kGsThreads), JC), kGsThreads, 0, s>>>(V, N, m, part,
-                                                                                                gs_chunks(N), tmp);
-    k_gs_axpy_sum<<<gs_norm_blocks(N), kGsThreads, 0, s>>>(w, N, tmp, JC, nrm_part);
-  } else {
-    k_gs_axpy<<<gs_norm_blocks(N), kGsThreads, 0, s>>>(w, V, N, m, part, gs_chunks(N), nrm_part);
-  }
-  return cudaGetLastError();
+  const int VB = (m + gs_groups(N, m) - 1) / gs_groups(N, m);
+  const int G = (m + VB - 1) / VB;
+  *groups = G;
+  if (gs_serial(N))
+    return launch_dependent(true, k_gs_update<256>, dim3((unsigned)((N + 255) / 256), G), 256, 0, s, V, N, m, VB, part,
+                            S, tmp);
+  return launch_dependent(false, k_gs_update<64>, dim3((unsigned)((N + 63) / 64), G), 64, 0, s, V, N, m, VB, part, S,
+                          tmp);
 }
 
-int gs_axpy_kernels(long long N) { return N < kGsSplitN ? 2 : 1; }
+cudaError_t gs_finish(const double2* w, const double2* tmp, int G, double2* dst, long long N, double* nrm_part,
+                      cudaStream_t s) {
+  return launch_dependent(gs_serial(N), k_gs_finish, dim3(gs_norm_blocks(N)), kGsThreads, 0, s, w, tmp, G, dst, N,
+                          nrm_part);
+}
 
 cudaError_t gmres_residual(const double2* b, double2* w, long long N, double* nrm_part, cudaStream_t s) {
   k_gmres_residual<<<gs_norm_blocks(N), kGsThreads, 0, s>>>(b, w, N, nrm_part);
   return cudaGetLastError();
 }
 
-cudaError_t gmres_column(int j, const double* part1, const double* part2, int S, const double* nrm_part, int nb,
-                         GmresDev* st, cudaStream_t s) {
-  if (j < 0 || j >= kGmresMax) return cudaErrorInvalidValue;
-  k_gmres_column<<<1, kGsThreads, 0, s>>>(j, part1, part2, S, nrm_part, nb, st);
-  return cudaGetLastError();
-}
-
-cudaError_t gmres_store(const double2* w, double2* dst, const GmresDev* st, long long N, cudaStream_t s) {
-  k_gmres_store<<<blocks_for(N), 256, 0, s>>>(w, dst, st, N);
-  return cudaGetLastError();
+cudaError_t gmres_columns(int j0, int nsteps, const double* part, long long plen, int S, const double* nrm,
+                          long long nlen, int nnrm, const double* nrm_last, int nlast, GmresDev* st, cudaStream_t s) {
+  if (j0 < 0 || j0 + nsteps > kGmresMax) return cudaErrorInvalidValue;
+  return launch_dependent(false, k_gmres_columns, dim3(nsteps), kGsThreads, 0, s, j0, part, plen, S, nrm, nlen, nnrm,
+                          nrm_last, nlast, st);
 }
 
 }  // namespace nfs
