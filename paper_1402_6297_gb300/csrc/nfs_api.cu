@@ -885,6 +885,39 @@ int zrotate_basis(nfs_ctx* c, int p, int q, int k, const std::vector<double>& z,
   return NFS_OK;
 }
 
+// A_r V of the basis vectors [0, n) of the masked problems, from fresh products.
+// The recurrence carries A_r V along (A_r w = B_r v_j - r, less the same
+// combinations that are taken from w), and the rounding E_j = MV_j - A_r V_j in
+// it obeys the recurrence of the Lanczos polynomials at 0, which lies in the
+// gap in the middle of the spectrum of A_r^-1 B_r: E grows exponentially, from
+// 1e-16 to about 1e-9 over a basis of 96 and, were it carried over a restart,
+// to 1e-3 within three, where the re-orthogonalisation works in a wrong inner
+// product (a homogeneous 16^3 grid at the tight tolerances lost an eigenvalue's
+// accuracy, or broke down, for 6 of 16 start vectors).  n products once per
+// restart cost a few per cent of the solves between two restarts.
+int refresh_products(nfs_ctx* c, int n, const std::vector<int>& mask) {
+  const long long N = c->N, vstride = (long long)c->vcap * N;
+  std::vector<int> skip(c->P);
+  for (int p = 0; p < c->P; ++p) skip[p] = !mask[p];
+  TRY(put_flags(c, c->work, 2 * c->P, skip));
+  const int* d_skip = c->d_flags + 2 * c->P;
+  for (int i = 0; i < n; ++i) {
+    for (int p = 0; p < c->P; ++p)
+      if (mask[p])
+        CK(cudaMemcpyAsync(c->t64 + p * N, c->V + p * vstride + i * N, N * sizeof(double2), cudaMemcpyDeviceToDevice,
+                           c->work));
+    if (c->lamdf)
+      TRY(matvec<nfs::df>(c, c->work, c->t64, c->t64b, d_skip, 1));
+    else
+      TRY(matvec<double>(c, c->work, c->t64, c->t64b, d_skip, 1));
+    for (int p = 0; p < c->P; ++p)
+      if (mask[p])
+        CK(cudaMemcpyAsync(c->MV + p * vstride + i * N, c->t64b + p * N, N * sizeof(double2), cudaMemcpyDeviceToDevice,
+                           c->work));
+  }
+  return NFS_OK;
+}
+
 // Largest loss of A_r-orthogonality removed with the FP32 shadow update; a
 // larger one is removed in FP64 (the shadow update's rounding, ~6e-8 of the
 // coefficients, would otherwise reappear above orth_tol).
@@ -1161,6 +1194,7 @@ int eigs_core(nfs_ctx* c, int nev, double* omega, double2* Y, nfs_eigs_info* inf
       }
       ++restarts_p[p];
     }
+    TRY(refresh_products(c, keep + 1, active));
     TRY(refresh_shadows(c, 0, keep + 1));
     jstart = keep;
     local_lo = 0;
@@ -1207,6 +1241,7 @@ int eigs_core(nfs_ctx* c, int nev, double* omega, double2* Y, nfs_eigs_info* inf
     }
     active = part;
     TRY(put_flags(c, s, 0, active));
+    TRY(refresh_products(c, nev, part));
     TRY(refresh_shadows(c, 0, nev));
     // the new start vector, A_r-orthogonalised twice against the locked ones
     nfs::k_random_fill<<<nb, 256, 0, s>>>(c->V + (long long)nev * N, N, vstride, P,
