@@ -83,22 +83,22 @@ k_residual_parts(const double2* __restrict__ Ay, const double2* __restrict__ By,
   }
 }
 
-// CG start, one block per problem: r^* r = the sum of the nred partials of
-// k_dot_re in part_a becomes the only partial of the nb in part_b.
+// CG start, one block per problem: r^* r = the sum of the nred partials in
+// part_a (k_dot_re, k_inner_start) becomes the only partial of the nb in part_b.
 template <typename R>
 __global__ void __launch_bounds__(kRedThreads)
 k_cg_init(CGState* st, const double* __restrict__ tol2, int maxit, int nred, int nb) {
   using P = typename RedAccFor<R>::partial;
   st += blockIdx.x;
-  const double rr = sum_partials(st->part_a, nred);
+  const P rr = sum_partials_all<R, kRedThreads>(st->part_a, nred);
   P* pb = reinterpret_cast<P*>(st->part_b);
   for (int i = threadIdx.x; i < nb; i += kRedThreads) {
-    P v;
-    scalar_from(i == 0 ? rr : 0.0, v);  // (thread 0 holds the sum)
+    P v = rr;
+    if (i > 0) scalar_from(0.0, v);
     pb[i] = v;
   }
   if (threadIdx.x == 0) {
-    st->rr = rr;
+    st->rr = scalar_double(rr);
     st->it = 0;
     st->maxit = maxit;
     st->done = st->status = 0;
@@ -163,14 +163,32 @@ __global__ void k_refine_residual(double2* __restrict__ r, const double2* __rest
   }
 }
 
-// complex64 <- complex128 * s[problem]
-__global__ void k_demote(const double2* __restrict__ a, const double* __restrict__ s, float2* __restrict__ y,
-                         long long N, long long total) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const double2 v = a[i];
-    const double f = s[i / N];
-    y[i] = make_float2((float)(v.x * f), (float)(v.y * f));
+// Start of an inner solve: r32 = s[problem] r64 rounded to complex64, zero iterate
+// and direction, and the partials of r32^* r32 (part_a; grid (blocks, P)).  One
+// kernel instead of the conversion, two memsets and a dot product: 30 instead of
+// 66 us at 96^3, bound by the FP64 pipe (two products and two conversions per
+// element).
+__global__ void __launch_bounds__(kRedThreads)
+k_inner_start(const double2* __restrict__ r64, const double* __restrict__ s, float2* __restrict__ r32,
+              float2* __restrict__ x32, float2* __restrict__ p32, long long N, CGState* st) {
+  const int p = blockIdx.y;
+  const double f = s[p];
+  const double2* a = r64 + (long long)p * N;
+  float4* r = reinterpret_cast<float4*>(r32 + (long long)p * N);
+  float4* x = reinterpret_cast<float4*>(x32 + (long long)p * N);
+  float4* d = reinterpret_cast<float4*>(p32 + (long long)p * N);
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  RedAcc<float> acc;
+  for (long long i = (long long)blockIdx.x * kRedThreads + threadIdx.x; i < N / 2; i += (long long)gridDim.x * kRedThreads) {
+    const double2 v0 = a[2 * i], v1 = a[2 * i + 1];
+    const float4 o = make_float4((float)(v0.x * f), (float)(v0.y * f), (float)(v1.x * f), (float)(v1.y * f));
+    r[i] = o;
+    x[i] = zero;
+    d[i] = zero;
+    acc.add(o.x * o.x + o.y * o.y + o.z * o.z + o.w * o.w);
   }
+  const float2 t = acc.block_total<kRedThreads>();
+  if (threadIdx.x == 0) reinterpret_cast<float2*>(st[p].part_a)[blockIdx.x] = t;
 }
 
 // x += s[problem] * complex128(d)
@@ -477,35 +495,56 @@ k_dots_finish(const double* __restrict__ part, int m, int nb, double* __restrict
   }
 }
 
-// part[(((p * m + j) * gridDim.x) + b) * 2 + {0, 1}] = block b's share of
-// conj(S_pj)^T w_p (S = Shi + Slo, w = whi + wlo) for the G vectors
-// j = blockIdx.y * G + g < m; grid (blocks, ceil(m / G), P).
-template <int G>
+// part[(((p * m + j) * gridDim.y) + b) * 2 + {0, 1}] = block b's share of
+// conj(S_pj)^T w_p (S = Shi + Slo, w = whi + wlo) for the two vectors
+// j = 2 blockIdx.x, 2 blockIdx.x + 1 < m; grid (ceil(m / 2), blocks, P).  A thread
+// takes two neighbouring elements at a time (N is even): six 16-byte loads in
+// flight.  Bound by memory, 16 bytes per element and vector: all pairs of one
+// range of elements run together (their w is read from L2) and few blocks per
+// pair, whose FP64 ends (a pair sum per value, then the block's) would otherwise
+// show.  One GB300, 96^3, 52 vectors on average: 738 us with 304 blocks per pair,
+// 8-byte loads and a full block sum per value, 693 with this body but all blocks
+// of one pair together (w from memory again for every pair), 649 now (430 us at
+// the copy rate); 16 problems of 32^3: 378, 364, 339 us.
 __global__ void __launch_bounds__(kRedThreads)
 k_exact_dots(const float2* __restrict__ Shi, const float2* __restrict__ Slo, long long sstride, int m,
              const float2* __restrict__ whi, const float2* __restrict__ wlo, long long N, double* __restrict__ part,
              const int* __restrict__ active) {
+  constexpr int G = 2;
   const int p = blockIdx.z;
   if (active && !active[p]) return;
-  Shi += (long long)p * sstride;
-  Slo += (long long)p * sstride;
-  whi += (long long)p * N;
-  wlo += (long long)p * N;
-  const int j0 = blockIdx.y * G;
+  const int j0 = blockIdx.x * G;
+  const int j1 = min(j0 + 1, m - 1);  // (an odd last vector is done twice and stored once)
+  const float4* wh4 = reinterpret_cast<const float4*>(whi + (long long)p * N);
+  const float4* wl4 = reinterpret_cast<const float4*>(wlo + (long long)p * N);
+  const float4* sh4[G] = {reinterpret_cast<const float4*>(Shi + p * sstride + j0 * N),
+                          reinterpret_cast<const float4*>(Shi + p * sstride + j1 * N)};
+  const float4* sl4[G] = {reinterpret_cast<const float4*>(Slo + p * sstride + j0 * N),
+                          reinterpret_cast<const float4*>(Slo + p * sstride + j1 * N)};
   // per vector: the exact sum of the hi x hi products (real, imaginary) and
   // an ordinary sum of their rounding errors and the hi x lo, lo x hi terms
   DSAccX2 acc[G];
   float2 small[G];
 #pragma unroll
   for (int g = 0; g < G; ++g) small[g] = make_float2(0.f, 0.f);
-  for (long long i = (long long)blockIdx.x * kRedThreads + threadIdx.x; i < N; i += (long long)gridDim.x * kRedThreads) {
-    const float2 bh = whi[i], bl = wlo[i];
-    // conj(a) b = (ar br + ai bi, ar bi - ai br) = ar (br, bi) + ai (bi, -br)
-    const float2 bh2 = make_float2(bh.y, -bh.x), bl2 = make_float2(bl.y, -bl.x);
+  for (long long i = (long long)blockIdx.y * kRedThreads + threadIdx.x; i < N / 2; i += (long long)gridDim.y * kRedThreads) {
+    const float4 bh4 = wh4[i], bl4 = wl4[i];
+    float4 ah4[G], al4[G];
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-      if (j0 + g < m) {
-        const float2 ah = Shi[(long long)(j0 + g) * N + i], al = Slo[(long long)(j0 + g) * N + i];
+      ah4[g] = __ldcs(sh4[g] + i);
+      al4[g] = __ldcs(sl4[g] + i);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float2 bh = h == 0 ? make_float2(bh4.x, bh4.y) : make_float2(bh4.z, bh4.w);
+      const float2 bl = h == 0 ? make_float2(bl4.x, bl4.y) : make_float2(bl4.z, bl4.w);
+      // conj(a) b = (ar br + ai bi, ar bi - ai br) = ar (br, bi) + ai (bi, -br)
+      const float2 bh2 = make_float2(bh.y, -bh.x), bl2 = make_float2(bl.y, -bl.x);
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const float2 ah = h == 0 ? make_float2(ah4[g].x, ah4[g].y) : make_float2(ah4[g].z, ah4[g].w);
+        const float2 al = h == 0 ? make_float2(al4[g].x, al4[g].y) : make_float2(al4[g].z, al4[g].w);
         const float2 ax = make_float2(ah.x, ah.x), ay = make_float2(ah.y, ah.y);
         float2 p1, e1, p2, e2;
         two_prod_x2(ax, bh, p1, e1);
@@ -521,19 +560,37 @@ k_exact_dots(const float2* __restrict__ Shi, const float2* __restrict__ Slo, lon
       }
     }
   }
-  // block sums in FP64.  (Double-single sums on the FP32 units would free
-  // the FP64 pipe, which these sums keep ~70% busy at small sizes, but they
-  // lost the accuracy the monitor needs on homogeneous media at symmetric
-  // k-points: spurious losses of 1e-6 and wrong degenerate eigenvalues.)
+  // block sums in FP64.  (Double-single sums on the FP32 units lost the
+  // accuracy the monitor needs on homogeneous media at symmetric k-points:
+  // spurious losses of 1e-6 and wrong degenerate eigenvalues.)  The four values
+  // of a warp at once: two halving exchanges leave each eight lanes with one of
+  // them, three more steps complete it (six FP64 additions instead of twenty).
+  double v[2 * G];
 #pragma unroll
   for (int g = 0; g < G; ++g) {
-    const double sr = block_sum<kRedThreads>((double)acc[g].hi.x + (double)acc[g].lo.x + (double)small[g].x);
-    const double si = block_sum<kRedThreads>((double)acc[g].hi.y + (double)acc[g].lo.y + (double)small[g].y);
-    if (threadIdx.x == 0 && j0 + g < m) {
-      const long long o = (((long long)p * m + j0 + g) * gridDim.x + blockIdx.x) * 2;
-      part[o] = sr;
-      part[o + 1] = si;
+    v[2 * g] = (double)acc[g].hi.x + (double)acc[g].lo.x + (double)small[g].x;
+    v[2 * g + 1] = (double)acc[g].hi.y + (double)acc[g].lo.y + (double)small[g].y;
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int h = G, o = 16; h >= 1; h >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int t = 0; t < h; ++t) {
+      const double keep = up ? v[t + h] : v[t], give = up ? v[t] : v[t + h];
+      v[t] = keep + __shfl_xor_sync(0xffffffffu, give, o);
     }
+  }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  __shared__ double sh[kRedThreads / 32][2 * G];
+  if ((lane & 7) == 0) sh[warp][((lane >> 4) & 1) * 2 + ((lane >> 3) & 1)] = v[0];
+  __syncthreads();
+  if (threadIdx.x < 2 * G && j0 + (int)threadIdx.x / 2 < m) {
+    double t = sh[0][threadIdx.x];
+#pragma unroll
+    for (int w = 1; w < kRedThreads / 32; ++w) t += sh[w][threadIdx.x];
+    part[(((long long)p * m + j0 + threadIdx.x / 2) * gridDim.y + blockIdx.y) * 2 + threadIdx.x % 2] = t;
   }
 }
 

@@ -35,7 +35,7 @@ struct CGState {
   double rr_now;    // r^* r of this step's residual (k_rows_in; a `partial`)
   double rr_last;   // of the step before (k_rows_out; infinite at the start: beta = 0)
   double tol2;      // stop when r^* r <= tol2 (a `partial`)
-  double part_a[kMaxPartials];  // p^* A p, one per CTA of k_columns (at the start: r^* r from k_dot_re, doubles)
+  double part_a[kMaxPartials];  // p^* A p, one per CTA of k_columns (at the start: of r^* r)
   double part_b[kMaxPartials];  // r^* r, one per CTA of k_rows_out
 };
 constexpr long long kStateDoubles = sizeof(CGState) / sizeof(double);

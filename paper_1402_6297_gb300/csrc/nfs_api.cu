@@ -413,16 +413,23 @@ int cg_chunk_graph(nfs_ctx* c, nfs::cplx<R>* x, nfs::cplx<R>* r, nfs::cplx<R>* p
 // Iterations run in graph-replayed chunks; every kernel returns at once after
 // its problem's device `done` flag is set, and the host reads the flags
 // between chunks.
+// r64, scale_off (complex64 runs): r is first formed as r64 times the per-problem
+// scale at d_small + scale_off, and x set to zero.
 template <typename R>
 int cg_run(nfs_ctx* c, nfs::cplx<R>* x, nfs::cplx<R>* r, nfs::cplx<R>* p, const std::vector<double>& tol2, int maxit,
-           std::vector<int>& iters, std::vector<int>& status) {
+           std::vector<int>& iters, std::vector<int>& status, const double2* r64 = nullptr, int scale_off = 0) {
   using C = nfs::cplx<R>;
   cudaStream_t s = c->work;
   CK(cudaStreamSynchronize(s));  // earlier work is not the loop's
   const double t0 = now_s();
-  CK(cudaMemsetAsync(p, 0, c->P * c->N * sizeof(C), s));  // with beta = 0 the first pass 1 sets p = r
+  // (p = 0: with beta = 0 the first step sets p = r)
   const int nb = red_blocks(c->N, c->P);
-  nfs::k_dot_re<C><<<dim3(nb, c->P), kRedThreads, 0, s>>>(r, r, c->N, c->st->part_a, nfs::kStateDoubles);
+  if constexpr (std::is_same<R, float>::value) {
+    nfs::k_inner_start<<<dim3(nb, c->P), kRedThreads, 0, s>>>(r64, c->d_small + scale_off, r, x, p, c->N, c->st);
+  } else {
+    CK(cudaMemsetAsync(p, 0, c->P * c->N * sizeof(C), s));
+    nfs::k_dot_re<C><<<dim3(nb, c->P), kRedThreads, 0, s>>>(r, r, c->N, c->st->part_a, nfs::kStateDoubles);
+  }
   TRY(put_small(c, s, 0, tol2));
   nfs::k_cg_init<R><<<c->P, kRedThreads, 0, s>>>(c->st, c->d_small, maxit, nb, nfs::cg_partials<R>(c->n1, c->n3));
   CK(cudaGetLastError());
@@ -541,12 +548,8 @@ int solve(nfs_ctx* c, const double2* b, double2* x, bool x_zero, const std::vect
     }
     if (!any) break;
     TRY(put_small(c, s, P, inv));
-    nfs::k_demote<<<nb, 256, 0, s>>>(c->r64, c->d_small + P, c->r32, c->N, tot);
-    CK(cudaGetLastError());
-    c->launches += 1;
-    CK(cudaMemsetAsync(c->x32, 0, tot * sizeof(float2), s));
     std::vector<int> it, st;
-    TRY(cg_run<float>(c, c->x32, c->r32, c->p32, itol2, c->opt.cg_maxit, it, st));
+    TRY(cg_run<float>(c, c->x32, c->r32, c->p32, itol2, c->opt.cg_maxit, it, st, c->r64, P));
     TRY(put_small(c, s, 2 * P, nrm));
     nfs::k_axpy_promote<<<nb, 256, 0, s>>>(x, c->d_small + 2 * P, c->x32, c->N, tot);
     CK(cudaGetLastError());
@@ -624,23 +627,16 @@ int multi_axpy(nfs_ctx* c, double2* w, double2* Mw, int j0, int m, const std::ve
 int exact_dots(nfs_ctx* c, int m, const double2* w, std::vector<double>& out, const int* d_active) {
   cudaStream_t s = c->work;
   const long long vstride = (long long)c->vcap * c->N;
-  // basis vectors per block: each block streams its slice of w once per G
-  // vectors, so a larger G re-reads w less often, but each vector costs a
-  // thread six accumulator registers; measured on GB300 at 96^3 (headline
-  // orthogonalisation time): G = 2 0.309 s, 4 0.343 s, 8 0.53 s, 16 0.91 s
-#ifndef NFS_EXACT_G
-#define NFS_EXACT_G 2
-#endif
-  constexpr int G = NFS_EXACT_G;
   double* part = c->dscratch;
   double* fin = c->dscratch + off_fin(c);
   // w split once into floats (the CG work vectors x32 / r32 are free here)
   float2* whi = c->x32 ? c->x32 : reinterpret_cast<float2*>(c->Ap64);
   float2* wlo = c->x32 ? c->r32 : reinterpret_cast<float2*>(c->Ap64) + c->P * c->N;
   nfs::k_split_hi_lo<<<grid_blocks(c->P * c->N, 256), 256, 0, s>>>(w, whi, wlo, c->P * c->N);
-  const int nb = red_blocks(c->N, c->P);
-  nfs::k_exact_dots<G><<<dim3(nb, (m + G - 1) / G, c->P), kRedThreads, 0, s>>>(c->MV32, c->MV32lo, vstride, m,
-                                                                                       whi, wlo, c->N, part, d_active);
+  // with many vectors one block per SM and pair: fewer FP64 ends of blocks
+  const int nb = m < 16 ? red_blocks(c->N, c->P) : std::min(red_blocks(c->N, c->P), (kRedBlocks / 2 + c->P - 1) / c->P);
+  nfs::k_exact_dots<<<dim3((m + 1) / 2, nb, c->P), kRedThreads, 0, s>>>(c->MV32, c->MV32lo, vstride, m, whi, wlo, c->N,
+                                                                        part, d_active);
   nfs::k_dots_finish<<<dim3(m, c->P), kRedThreads, 0, s>>>(part, m, nb, fin, d_active);
   CK(cudaGetLastError());
   c->launches += 3;
@@ -757,7 +753,7 @@ int default_ncv(nfs_ctx* c, int nev) {
   return wanted_ncv(nev);
 }
 
-// Rayleigh-Ritz over the nev Ritz vectors of problem p (basis positions
+// Rayleigh-Ritz over the nev Ritz vectors of a problem (basis positions
 // 0..nev-1 after a rotation): the pencil H z = theta G z with
 // H = Y^* B_r Y and G = Y^* A_r Y (A_r Y from fresh products), formed with
 // FP64 inner products and solved on the host (Cholesky of G, Schur form of the
@@ -765,35 +761,63 @@ int default_ncv(nfs_ctx* c, int nev) {
 // deflation checks were each converged against locked vectors that are only
 // accurate to eig_tol, so their eigenvalues carry a first-order error; the
 // Rayleigh quotients on the span of all nev vectors are accurate to second
-// order.  theta: ascending order of omega = 1/theta on return; z: the
-// row-major nev x nev complex coefficients (interleaved re, im), columns in
-// that order.  flags: a device mask with problem p alone set.
-int final_rayleigh_ritz(nfs_ctx* c, int p, int nev, const int* flags, std::vector<double>& theta,
-                        std::vector<double>& z, int kout = -1) {
+// order.
+
+using RitzMatrix = std::vector<std::complex<double>>;
+
+// H and G of every problem with a nonzero mask, all problems in the same
+// launches (one problem after the other, each in launches of its own, took 100
+// of 590 ms for 16 k-points at 32^3).
+int ritz_matrices(nfs_ctx* c, int nev, const std::vector<int>& mask, std::vector<RitzMatrix>& H,
+                  std::vector<RitzMatrix>& G) {
   using cplxd = std::complex<double>;
   const long long N = c->N, vstride = (long long)c->vcap * N;
-  if (kout < 0) kout = nev;
-  std::vector<cplxd> H((size_t)nev * nev), G((size_t)nev * nev);
+  const int P = c->P;
+  H.assign(P, RitzMatrix());
+  G.assign(P, RitzMatrix());
+  std::vector<int> skip(P);
+  for (int p = 0; p < P; ++p) {
+    skip[p] = !mask[p];
+    if (mask[p]) {
+      H[p].resize((size_t)nev * nev);
+      G[p].resize((size_t)nev * nev);
+    }
+  }
   std::vector<double> d;
-  // A_r y_i from fresh products (complex128, or double-single in mixed
-  // contexts) of problem p alone
-  std::vector<int> skip(c->P, 1);
-  skip[p] = 0;
-  TRY(put_flags(c, c->work, 2 * c->P, skip));
-  const int* d_skip = c->d_flags + 2 * c->P;
+  TRY(put_flags(c, c->work, P, mask));
+  TRY(put_flags(c, c->work, 2 * P, skip));
+  const int *d_mask = c->d_flags + P, *d_skip = c->d_flags + 2 * P;
+  auto column = [&](std::vector<RitzMatrix>& A, int i) {
+    for (int p = 0; p < P; ++p)
+      if (mask[p])
+        for (int j = 0; j < nev; ++j)
+          A[p][(size_t)j * nev + i] = cplxd(d[(size_t)p * 2 * nev + 2 * j], d[(size_t)p * 2 * nev + 2 * j + 1]);
+  };
   for (int i = 0; i < nev; ++i) {
-    TRY(apply_Br_basis(c, i, c->t64));  // B_r y_i (every problem; p's is used)
-    TRY(multi_dot(c, c->V, 0, nev, c->t64, d, flags));
-    for (int j = 0; j < nev; ++j) H[(size_t)j * nev + i] = cplxd(d[(size_t)p * 2 * nev + 2 * j], d[(size_t)p * 2 * nev + 2 * j + 1]);
-    CK(cudaMemcpyAsync(c->t64 + (long long)p * N, c->V + p * vstride + (long long)i * N, N * sizeof(double2),
-                       cudaMemcpyDeviceToDevice, c->work));
+    TRY(apply_Br_basis(c, i, c->t64));  // B_r y_i
+    TRY(multi_dot(c, c->V, 0, nev, c->t64, d, d_mask));
+    column(H, i);
+    // A_r y_i from fresh products (complex128, or double-single in mixed contexts)
+    for (int p = 0; p < P; ++p)
+      if (mask[p])
+        CK(cudaMemcpyAsync(c->t64 + (long long)p * N, c->V + p * vstride + (long long)i * N, N * sizeof(double2),
+                           cudaMemcpyDeviceToDevice, c->work));
     if (c->lamdf)
       TRY(matvec<nfs::df>(c, c->work, c->t64, c->t64b, d_skip, 1));
     else
       TRY(matvec<double>(c, c->work, c->t64, c->t64b, d_skip, 1));
-    TRY(multi_dot(c, c->V, 0, nev, c->t64b, d, flags));
-    for (int j = 0; j < nev; ++j) G[(size_t)j * nev + i] = cplxd(d[(size_t)p * 2 * nev + 2 * j], d[(size_t)p * 2 * nev + 2 * j + 1]);
+    TRY(multi_dot(c, c->V, 0, nev, c->t64b, d, d_mask));
+    column(G, i);
   }
+  return NFS_OK;
+}
+
+// theta: descending (ascending order of omega = 1/theta); z: the row-major
+// nev x nev complex coefficients (interleaved re, im), columns in that order.
+// H and G are overwritten.
+int ritz_solve(int p, int nev, RitzMatrix& H, RitzMatrix& G, std::vector<double>& theta, std::vector<double>& z) {
+  using cplxd = std::complex<double>;
+  const int kout = nev;
   // symmetrise (the inner products are exact only to rounding)
   for (int i = 0; i < nev; ++i)
     for (int j = 0; j <= i; ++j) {
@@ -1284,47 +1308,46 @@ int eigs_core(nfs_ctx* c, int nev, double* omega, double2* Y, nfs_eigs_info* inf
   // results from each problem's leading jm x jm block: omega ascending = theta descending
   const double tv0 = now_s();
   int worst = NFS_OK;
+  std::vector<int> ok(P);
+  std::vector<double> maxres(P, 0.0);
+  bool any_ok = false;
   for (int p = 0; p < P; ++p) {
     const int k = jm[p];
     if (!nfs::host::sym_eig(k, leading(p, k), theta, Z)) return NFS_EBREAKDOWN;
-    double maxres = 0.0;
     for (int i = 0; i < nev; ++i) {
       const int cc = k - 1 - i;
       omega[(size_t)p * nev + i] = 1.0 / theta[cc];
-      maxres = std::max(maxres, std::fabs(beta_last[p] * Z[(size_t)(k - 1) * k + cc]) / std::fabs(theta[cc]));
+      maxres[p] = std::max(maxres[p], std::fabs(beta_last[p] * Z[(size_t)(k - 1) * k + cc]) / std::fabs(theta[cc]));
     }
-    if (status[p] == NFS_OK) {
-      // a Rayleigh-Ritz on the span of the nev Ritz vectors with the true
-      // inner products: second-order accurate eigenvalues for copies found by
-      // deflation checks, and values that stay inside the spectrum even where
-      // the basis has lost A_r-orthogonality
-      std::vector<double> Ycm((size_t)P * k * nev, 0.0);
-      for (int i = 0; i < nev; ++i)
-        for (int r = 0; r < k; ++r) Ycm[(size_t)p * k * nev + (size_t)i * k + r] = Z[(size_t)r * k + (k - 1 - i)];
-      std::fill(one.begin(), one.end(), 0);
-      one[p] = 1;
-      TRY(put_flags(c, s, P, one));
-      TRY(rotate(c, c->V, k, Ycm, nev, c->d_flags + P));
+    ok[p] = status[p] == NFS_OK;
+    any_ok = any_ok || ok[p];
+    if (!ok[p] && !Y) continue;
+    // the Ritz vectors of problem p: rotate its basis (only p flagged)
+    std::vector<double> Ycm((size_t)P * k * nev, 0.0);
+    for (int i = 0; i < nev; ++i)
+      for (int r = 0; r < k; ++r) Ycm[(size_t)p * k * nev + (size_t)i * k + r] = Z[(size_t)r * k + (k - 1 - i)];
+    std::fill(one.begin(), one.end(), 0);
+    one[p] = 1;
+    TRY(put_flags(c, s, P, one));
+    TRY(rotate(c, c->V, k, Ycm, nev, c->d_flags + P));
+  }
+  // a Rayleigh-Ritz on the span of the nev Ritz vectors with the true inner
+  // products: second-order accurate eigenvalues for copies found by deflation
+  // checks, and values that stay inside the spectrum even where the basis has
+  // lost A_r-orthogonality
+  std::vector<RitzMatrix> RH, RG;
+  if (any_ok) TRY(ritz_matrices(c, nev, ok, RH, RG));
+  for (int p = 0; p < P; ++p) {
+    if (ok[p]) {
       std::vector<double> th2, zc;
-      TRY(final_rayleigh_ritz(c, p, nev, c->d_flags + P, th2, zc));
+      TRY(ritz_solve(p, nev, RH[p], RG[p], th2, zc));
       for (int i = 0; i < nev; ++i) omega[(size_t)p * nev + i] = 1.0 / th2[i];
-      TRY(zrotate_basis(c, p, nev, nev, zc, false));
-      if (Y) {
-        CK(cudaMemcpyAsync(Y + (long long)p * nev * N, col(c->V, p, 0), (size_t)nev * N * sizeof(double2),
-                           cudaMemcpyDeviceToDevice, s));
-        CK(cudaStreamSynchronize(s));
-      }
-    } else if (Y) {
-      // Ritz vectors of problem p: rotate its basis (only p flagged), then copy
-      std::vector<double> Ycm((size_t)P * k * nev, 0.0);
-      for (int i = 0; i < nev; ++i)
-        for (int r = 0; r < k; ++r) Ycm[(size_t)p * k * nev + (size_t)i * k + r] = Z[(size_t)r * k + (k - 1 - i)];
-      std::fill(one.begin(), one.end(), 0);
-      one[p] = 1;
-      TRY(put_flags(c, s, P, one));
-      TRY(rotate(c, c->V, k, Ycm, nev, c->d_flags + P));
+      if (Y) TRY(zrotate_basis(c, p, nev, nev, zc, false));
+    }
+    if (Y) {
       CK(cudaMemcpyAsync(Y + (long long)p * nev * N, col(c->V, p, 0), (size_t)nev * N * sizeof(double2),
                          cudaMemcpyDeviceToDevice, s));
+      CK(cudaStreamSynchronize(s));
     }
     if (infos) {
       nfs_eigs_info& in = infos[p];
@@ -1334,7 +1357,7 @@ int eigs_core(nfs_ctx* c, int nev, double* omega, double2* Y, nfs_eigs_info* inf
       in.matvecs_c64 = (c->mv32 - mv32_0) / P;
       in.matvecs_c128 = (c->mv64 - mv64_0) / P;
       in.nconv = status[p] == NFS_OK ? nev : nconv[p];
-      in.max_ritz_residual = maxres;
+      in.max_ritz_residual = maxres[p];
       in.status = status[p];
       in.kernel_launches = c->launches - launches_0;
       in.seconds_total = now_s() - t_begin;
