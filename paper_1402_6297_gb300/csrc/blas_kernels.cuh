@@ -84,10 +84,12 @@ k_residual_parts(const double2* __restrict__ Ay, const double2* __restrict__ By,
 }
 
 // CG start, one block per problem: r^* r = the sum of the nred partials in
-// part_a (k_dot_re, k_inner_start) becomes the only partial of the nb in part_b.
+// part_a (k_dot_re, k_inner_start, k_solve_start) becomes the only partial of the
+// nb in part_b; tol2 is the threshold, or (relative) its ratio to r^* r.  An
+// infinite one, or an r^* r that is not positive, means nothing to solve.
 template <typename R>
 __global__ void __launch_bounds__(kRedThreads)
-k_cg_init(CGState* st, const double* __restrict__ tol2, int maxit, int nred, int nb) {
+k_cg_init(CGState* st, const double* __restrict__ tol2, bool relative, int maxit, int nred, int nb) {
   using P = typename RedAccFor<R>::partial;
   st += blockIdx.x;
   const P rr = sum_partials_all<R, kRedThreads>(st->part_a, nred);
@@ -98,13 +100,16 @@ k_cg_init(CGState* st, const double* __restrict__ tol2, int maxit, int nred, int
     pb[i] = v;
   }
   if (threadIdx.x == 0) {
-    st->rr = scalar_double(rr);
+    const double r2 = scalar_double(rr);
+    double tol = tol2[blockIdx.x];
+    if (relative) tol = r2 > 0.0 && tol < (double)INFINITY ? tol * r2 : (double)INFINITY;
+    st->rr = st->rr0 = r2;
     st->it = 0;
     st->maxit = maxit;
     st->done = st->status = 0;
     st->stop = st->halt = st->broken = 0;
     scalar_from((double)INFINITY, *reinterpret_cast<P*>(&st->rr_last));
-    scalar_from(tol2[blockIdx.x], *reinterpret_cast<P*>(&st->tol2));
+    scalar_from(tol, *reinterpret_cast<P*>(&st->tol2));
   }
 }
 
@@ -189,6 +194,24 @@ k_inner_start(const double2* __restrict__ r64, const double* __restrict__ s, flo
   }
   const float2 t = acc.block_total<kRedThreads>();
   if (threadIdx.x == 0) reinterpret_cast<float2*>(st[p].part_a)[blockIdx.x] = t;
+}
+
+// Likewise of a complex128 solve from x = 0: r = b.
+__global__ void __launch_bounds__(kRedThreads)
+k_solve_start(const double2* __restrict__ b, double2* __restrict__ r, double2* __restrict__ x, double2* __restrict__ d,
+              long long N, CGState* st) {
+  const long long off = (long long)blockIdx.y * N;
+  const double2 zero = make_double2(0.0, 0.0);
+  RedAcc<double> acc;
+  for (long long i = (long long)blockIdx.x * kRedThreads + threadIdx.x; i < N; i += (long long)gridDim.x * kRedThreads) {
+    const double2 v = b[off + i];
+    r[off + i] = v;
+    x[off + i] = zero;
+    d[off + i] = zero;
+    acc.add(v.x * v.x + v.y * v.y);
+  }
+  const double t = acc.block_total<kRedThreads>();
+  if (threadIdx.x == 0) st[blockIdx.y].part_a[blockIdx.x] = t;
 }
 
 // x += s[problem] * complex128(d)

@@ -27,6 +27,7 @@ constexpr int kMaxPartials = 3072;  // >= kRedBlocks and the CTAs of one problem
 struct CGState {
   // what the host reads (set by k_cg_check at the end of a chunk)
   double rr;        // r^* r of the current residual
+  double rr0;       // and of the one at the start (set by k_cg_init)
   int it, maxit;    // steps taken, and how many are allowed
   int done;         // 1: converged, broken down or out of iterations
   int status;       // 0, -6 (no convergence) or -7 (breakdown)

@@ -13,6 +13,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 #include <chrono>
 #include <cmath>
@@ -128,6 +129,8 @@ struct nfs_ctx {
   size_t dY_len = 0;
   std::vector<GraphEntry> graphs;
   std::vector<GmresGraph> gm_graphs;  // NFSEP inner-solve step batches
+  // chunks that the last CG run took, per precision and refinement round
+  int cg_chunks[2][4] = {{1, 1, 1, 1}, {1, 1, 1, 1}};
   long long bytes = 0;
   long long mv32 = 0, mv64 = 0;
   long long launches = 0;  // kernels this context has launched (graph nodes included)
@@ -312,21 +315,31 @@ int red_blocks(long long N, int P) {
   return (int)std::max<long long>(1, nb);
 }
 
-// Re(x_p^* y_p) for every problem, on the host
+// Re(x_p^* y_p) for every problem, on the host: the launch and the copy of the
+// partials to hscratch + off, and their sums once the stream has got there
 template <typename C>
-int dots_re(nfs_ctx* c, cudaStream_t s, const C* x, const C* y, std::vector<double>& out) {
+int dots_re_start(nfs_ctx* c, cudaStream_t s, const C* x, const C* y, size_t off) {
   const int nb = red_blocks(c->N, c->P);
   nfs::k_dot_re<C><<<dim3(nb, c->P), kRedThreads, 0, s>>>(x, y, c->N, c->dscratch, nb);
   CK(cudaGetLastError());
   c->launches += 1;
-  CK(cudaMemcpyAsync(c->hscratch, c->dscratch, (size_t)nb * c->P * sizeof(double), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
+  CK(cudaMemcpyAsync(c->hscratch + off, c->dscratch, (size_t)nb * c->P * sizeof(double), cudaMemcpyDeviceToHost, s));
+  return NFS_OK;
+}
+void dots_re_finish(const nfs_ctx* c, size_t off, std::vector<double>& out) {
+  const int nb = red_blocks(c->N, c->P);
   out.assign(c->P, 0.0);
   for (int p = 0; p < c->P; ++p) {
     double t = 0.0;
-    for (int i = 0; i < nb; ++i) t += c->hscratch[(size_t)p * nb + i];
+    for (int i = 0; i < nb; ++i) t += c->hscratch[off + (size_t)p * nb + i];
     out[p] = t;
   }
+}
+template <typename C>
+int dots_re(nfs_ctx* c, cudaStream_t s, const C* x, const C* y, std::vector<double>& out) {
+  TRY(dots_re_start(c, s, x, y, 0));
+  CK(cudaStreamSynchronize(s));
+  dots_re_finish(c, 0, out);
   return NFS_OK;
 }
 
@@ -411,40 +424,54 @@ int cg_chunk_graph(nfs_ctx* c, nfs::cplx<R>* x, nfs::cplx<R>* r, nfs::cplx<R>* p
 // CG from the state r = b - A x (already formed) for every problem, on the
 // work stream; tol2 the absolute thresholds on r^* r (+inf skips a problem).
 // Iterations run in graph-replayed chunks; every kernel returns at once after
-// its problem's device `done` flag is set, and the host reads the flags
-// between chunks.
-// r64, scale_off (complex64 runs): r is first formed as r64 times the per-problem
-// scale at d_small + scale_off, and x set to zero.
+// its problem's device `done` flag is set.  The host first reads the flags after
+// as many chunks as the last run of the same kind took (the solves of an
+// eigensolve differ by an iteration or two), then after each: every round trip
+// leaves the GPU idle for about 20 us (8^3 complex128 eigensolves spent 9 of 86
+// ms on them).
+// r64 given: r is first formed from it (complex64: times the per-problem scale
+// at d_small + scale_off), and x set to zero.  relative: tol2 is a factor of the
+// starting r^* r.
 template <typename R>
 int cg_run(nfs_ctx* c, nfs::cplx<R>* x, nfs::cplx<R>* r, nfs::cplx<R>* p, const std::vector<double>& tol2, int maxit,
-           std::vector<int>& iters, std::vector<int>& status, const double2* r64 = nullptr, int scale_off = 0) {
+           std::vector<int>& iters, std::vector<int>& status, const double2* r64 = nullptr, int scale_off = 0,
+           int round = 0, bool relative = false) {
   using C = nfs::cplx<R>;
   cudaStream_t s = c->work;
-  CK(cudaStreamSynchronize(s));  // earlier work is not the loop's
   const double t0 = now_s();
   // (p = 0: with beta = 0 the first step sets p = r)
   const int nb = red_blocks(c->N, c->P);
   if constexpr (std::is_same<R, float>::value) {
     nfs::k_inner_start<<<dim3(nb, c->P), kRedThreads, 0, s>>>(r64, c->d_small + scale_off, r, x, p, c->N, c->st);
+  } else if (r64 != nullptr) {
+    nfs::k_solve_start<<<dim3(nb, c->P), kRedThreads, 0, s>>>(r64, r, x, p, c->N, c->st);
   } else {
     CK(cudaMemsetAsync(p, 0, c->P * c->N * sizeof(C), s));
     nfs::k_dot_re<C><<<dim3(nb, c->P), kRedThreads, 0, s>>>(r, r, c->N, c->st->part_a, nfs::kStateDoubles);
   }
   TRY(put_small(c, s, 0, tol2));
-  nfs::k_cg_init<R><<<c->P, kRedThreads, 0, s>>>(c->st, c->d_small, maxit, nb, nfs::cg_partials<R>(c->n1, c->n3));
+  nfs::k_cg_init<R><<<c->P, kRedThreads, 0, s>>>(c->st, c->d_small, relative, maxit, nb,
+                                                 nfs::cg_partials<R>(c->n1, c->n3));
   CK(cudaGetLastError());
   c->launches += 2;
   cudaGraphExec_t exec = nullptr;
   TRY(cg_chunk_graph<R>(c, x, r, p, &exec));
   const size_t head = offsetof(CGState, part_a);
-  for (;;) {
-    CK(cudaGraphLaunch(exec, s));
-    c->launches += nfs::kProductKernels * kCgChunk + 1;
+  int& last = c->cg_chunks[sizeof(R) == 4][std::min(round, 3)];
+  for (int ahead = std::max(1, std::min(last, maxit / kCgChunk)), ran = 0;; ahead = 1) {
+    for (int i = 0; i < ahead; ++i) CK(cudaGraphLaunch(exec, s));
+    c->launches += (nfs::kProductKernels * kCgChunk + 1) * ahead;
+    ran += ahead;
     CK(cudaMemcpy2DAsync(c->st_host, sizeof(CGState), c->st, sizeof(CGState), head, c->P, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     bool all = true;
     for (int q = 0; q < c->P; ++q) all = all && c->st_host[q].done;
-    if (all) break;
+    if (all) {
+      int it = 1;
+      for (int q = 0; q < c->P; ++q) it = std::max(it, c->st_host[q].it);
+      last = std::min(ran, (it + kCgChunk - 1) / kCgChunk);
+      break;
+    }
   }
   iters.resize(c->P);
   status.resize(c->P);
@@ -479,12 +506,28 @@ int solve(nfs_ctx* c, const double2* b, double2* x, bool x_zero, const std::vect
   cudaStream_t s = c->work;
   const int P = c->P;
   const long long tot = P * c->N;
-  std::vector<double> bb;
-  TRY(dots_re(c, s, b, b, bb));
+  const double tol = c->opt.cg_tol;
   so.iters.assign(P, 0);
   so.refines.assign(P, 0);
   so.status.assign(P, NFS_OK);
   so.relres.assign(P, 0.0);
+  if (x_zero && c->opt.precision != NFS_PREC_MIXED) {
+    // r = b: the threshold is formed on the device, without waiting for |b|
+    std::vector<double> tol2(P);
+    for (int q = 0; q < P; ++q) tol2[q] = active[q] ? tol * tol : INFINITY;
+    std::vector<int> it, st;
+    TRY(cg_run<double>(c, x, c->r64, c->p64, tol2, c->opt.cg_maxit, it, st, b, 0, 0, true));
+    for (int q = 0; q < P; ++q) {
+      const double bb = c->st_host[q].rr0;
+      if (!active[q] || !(bb > 0.0)) continue;
+      so.iters[q] = it[q];
+      so.status[q] = st[q];
+      so.relres[q] = std::sqrt(std::max(c->st_host[q].rr, 0.0) / bb);
+    }
+    return NFS_OK;
+  }
+  std::vector<double> bb;
+  TRY(dots_re(c, s, b, b, bb));
   if (x_zero) {
     CK(cudaMemsetAsync(x, 0, tot * sizeof(double2), s));
     CK(cudaMemcpyAsync(c->r64, b, tot * sizeof(double2), cudaMemcpyDeviceToDevice, s));
@@ -492,7 +535,6 @@ int solve(nfs_ctx* c, const double2* b, double2* x, bool x_zero, const std::vect
     TRY(matvec<double>(c, s, x, c->Ap64));
     TRY(sub64(c, s, b, c->Ap64, c->r64));
   }
-  const double tol = c->opt.cg_tol;
   std::vector<int> need(P);
   for (int q = 0; q < P; ++q) need[q] = active[q] && bb[q] > 0.0;
   if (c->opt.precision != NFS_PREC_MIXED) {
@@ -520,8 +562,11 @@ int solve(nfs_ctx* c, const double2* b, double2* x, bool x_zero, const std::vect
   const int nb = grid_blocks(tot, 256);
   std::vector<double> rr;
   std::vector<int> live(need);
-  for (;;) {
-    TRY(dots_re(c, s, c->r64, c->r64, rr));
+  for (int round = 0;; ++round) {
+    if (round == 0 && x_zero)
+      rr = bb;  // r = b
+    else
+      TRY(dots_re(c, s, c->r64, c->r64, rr));
     bool any = false, any64 = false, any32 = false;
     std::vector<double> inv(P, 0.0), nrm(P, 0.0), itol2(P, INFINITY);
     std::vector<int> skip(P, 1), skip64(P, 1), skip32(P, 1);
@@ -549,7 +594,7 @@ int solve(nfs_ctx* c, const double2* b, double2* x, bool x_zero, const std::vect
     if (!any) break;
     TRY(put_small(c, s, P, inv));
     std::vector<int> it, st;
-    TRY(cg_run<float>(c, c->x32, c->r32, c->p32, itol2, c->opt.cg_maxit, it, st, c->r64, P));
+    TRY(cg_run<float>(c, c->x32, c->r32, c->p32, itol2, c->opt.cg_maxit, it, st, c->r64, P, round));
     TRY(put_small(c, s, 2 * P, nrm));
     nfs::k_axpy_promote<<<nb, 256, 0, s>>>(x, c->d_small + 2 * P, c->x32, c->N, tot);
     CK(cudaGetLastError());
@@ -583,13 +628,15 @@ size_t lanczos_scratch_len(int P, int mcap) {
   return (size_t)P * kRedBlocks * 2 * mcap + 4 * (size_t)P * mcap + 64;
 }
 size_t off_fin(const nfs_ctx* c) { return (size_t)c->P * kRedBlocks * 2 * c->vcap; }
-size_t off_coef(const nfs_ctx* c) { return off_fin(c) + (size_t)2 * c->P * c->vcap; }
+// and in hscratch while a Lanczos step is in flight: the coefficients of the
+// recurrence at 0, then the partials of w^* A_r w, then the exact products
+size_t off_host_dots(const nfs_ctx* c) { return (size_t)2 * c->P * c->vcap; }
+size_t off_host_exact(const nfs_ctx* c) { return off_host_dots(c) + (size_t)c->P * kRedBlocks; }
 
 // Per-problem complex inner products of w_p with basis vectors [j0, j0 + m) of
 // Vbase (V or MV, FP64) -> out[p * 2m + 2i + {0,1}] on the host; problems with
 // a zero flag in d_active are skipped.
-int multi_dot(nfs_ctx* c, const double2* Vbase, int j0, int m, const double2* w, std::vector<double>& out,
-              const int* d_active) {
+int multi_dot_start(nfs_ctx* c, const double2* Vbase, int j0, int m, const double2* w, const int* d_active) {
   cudaStream_t s = c->work;
   const long long vstride = (long long)c->vcap * c->N;
   double* part = c->dscratch;
@@ -601,30 +648,33 @@ int multi_dot(nfs_ctx* c, const double2* Vbase, int j0, int m, const double2* w,
   CK(cudaGetLastError());
   c->launches += 2;
   CK(cudaMemcpyAsync(c->hscratch, fin, (size_t)c->P * m * 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
+  return NFS_OK;
+}
+// (the first half leaves the products on the device too, at off_fin)
+int multi_dot(nfs_ctx* c, const double2* Vbase, int j0, int m, const double2* w, std::vector<double>& out,
+              const int* d_active) {
+  TRY(multi_dot_start(c, Vbase, j0, m, w, d_active));
+  CK(cudaStreamSynchronize(c->work));
   out.assign(c->hscratch, c->hscratch + (size_t)c->P * 2 * m);
   return NFS_OK;
 }
 
-// w_p -= V_p[j0 : j0 + m] coef_p ; Mw_p -= MV_p[j0 : j0 + m] coef_p
-int multi_axpy(nfs_ctx* c, double2* w, double2* Mw, int j0, int m, const std::vector<double>& coef,
-               const int* d_active) {
-  cudaStream_t s = c->work;
+// w_p -= V_p[j0 : j0 + m] coef_p ; Mw_p -= MV_p[j0 : j0 + m] coef_p with the
+// coefficients where multi_dot leaves them on the device
+int multi_axpy(nfs_ctx* c, double2* w, double2* Mw, int j0, int m, const int* d_active) {
   const long long vstride = (long long)c->vcap * c->N;
-  double* dcoef = c->dscratch + off_coef(c);
-  std::memcpy(c->hscratch, coef.data(), coef.size() * sizeof(double));
-  CK(cudaMemcpyAsync(dcoef, c->hscratch, coef.size() * sizeof(double), cudaMemcpyHostToDevice, s));
-  nfs::k_multi_axpy<<<dim3(grid_blocks(c->N, 256), c->P), 256, 0, s>>>(
-      w, Mw, c->V + (long long)j0 * c->N, c->MV + (long long)j0 * c->N, vstride, dcoef, m, c->N, d_active);
+  nfs::k_multi_axpy<<<dim3(grid_blocks(c->N, 256), c->P), 256, 0, c->work>>>(
+      w, Mw, c->V + (long long)j0 * c->N, c->MV + (long long)j0 * c->N, vstride, c->dscratch + off_fin(c), m, c->N,
+      d_active);
   CK(cudaGetLastError());
   c->launches += 1;
-  CK(cudaStreamSynchronize(s));  // the pinned staging buffer is reused next
   return NFS_OK;
 }
 
 // d_p = MV_p[0:m]^* w_p, exact to ~1e-14 of the terms, from the split FP32
-// shadows of MV on the FP32 units (orthogonality monitor and coefficients)
-int exact_dots(nfs_ctx* c, int m, const double2* w, std::vector<double>& out, const int* d_active) {
+// shadows of MV on the FP32 units (orthogonality monitor and coefficients), at
+// hscratch + off once the stream has got there
+int exact_dots_start(nfs_ctx* c, int m, const double2* w, const int* d_active, size_t off) {
   cudaStream_t s = c->work;
   const long long vstride = (long long)c->vcap * c->N;
   double* part = c->dscratch;
@@ -640,9 +690,7 @@ int exact_dots(nfs_ctx* c, int m, const double2* w, std::vector<double>& out, co
   nfs::k_dots_finish<<<dim3(m, c->P), kRedThreads, 0, s>>>(part, m, nb, fin, d_active);
   CK(cudaGetLastError());
   c->launches += 3;
-  CK(cudaMemcpyAsync(c->hscratch, fin, (size_t)c->P * m * 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
-  out.assign(c->hscratch, c->hscratch + (size_t)c->P * 2 * m);
+  CK(cudaMemcpyAsync(c->hscratch + off, fin, (size_t)c->P * m * 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
   return NFS_OK;
 }
 
@@ -942,6 +990,33 @@ int refresh_products(nfs_ctx* c, int n, const std::vector<int>& mask) {
   return NFS_OK;
 }
 
+// f(p) for p < P on up to eight host threads (the projected eigenproblems of a
+// batch: 16 of size 130 take 1.4 ms one after the other, with the GPU idle
+// meanwhile).  f reports through what it writes; false if it threw.
+template <typename F>
+bool for_problems(int P, F f) {
+  std::atomic<int> next{0};
+  std::atomic<bool> ok{true};
+  auto work = [&] {
+    try {
+      for (int p; (p = next.fetch_add(1)) < P;) f(p);
+    } catch (...) {
+      ok = false;
+    }
+  };
+  std::thread helpers[7];
+  const int want = std::min(P - 1, 7);
+  int started = 0;
+  try {
+    for (; started < want; ++started) helpers[started] = std::thread(work);
+  } catch (...) {
+    // fewer threads, then
+  }
+  work();
+  for (int t = 0; t < started; ++t) helpers[t].join();
+  return ok;
+}
+
 // Largest loss of A_r-orthogonality removed with the FP32 shadow update; a
 // larger one is removed in FP64 (the shadow update's rounding, ~6e-8 of the
 // coefficients, would otherwise reappear above orth_tol).
@@ -1040,10 +1115,8 @@ int eigs_core(nfs_ctx* c, int nev, double* omega, double2* Y, nfs_eigs_info* inf
       // w = A_r^{-1} B_r v_j (CG); A_r w = B_r v_j
       TRY(apply_Br_basis(c, j, Mw));
       SolveOut so;
-      CK(cudaStreamSynchronize(s));
       const double ts = now_s();
-      TRY(solve(c, Mw, w, true, active, so));
-      CK(cudaStreamSynchronize(s));
+      TRY(solve(c, Mw, w, true, active, so));  // (ends with the stream idle)
       c->sec_solve += now_s() - ts;
       // A_r w = B_r v_j - r with r the solve's final residual (the refined
       // FP64 residual in mixed contexts): the right-hand side alone would
@@ -1067,8 +1140,15 @@ int eigs_core(nfs_ctx* c, int nev, double* omega, double2* Y, nfs_eigs_info* inf
       // vectors) in the A_r inner product
       const int nl = j - local_lo + 1;
       const double tr0 = now_s();
-      TRY(multi_dot(c, c->MV, local_lo, nl, w, coef, d_active));
-      TRY(multi_axpy(c, w, Mw, local_lo, nl, coef, d_active));
+      TRY(multi_dot_start(c, c->MV, local_lo, nl, w, d_active));
+      TRY(multi_axpy(c, w, Mw, local_lo, nl, d_active));
+      TRY(dots_re_start(c, s, w, Mw, off_host_dots(c)));
+      CK(cudaEventRecord(c->ev, s));
+      // (the orthogonality monitor of the step follows without a gap)
+      if (local_lo > 0) TRY(exact_dots_start(c, local_lo, w, d_active, off_host_exact(c)));
+      CK(cudaEventSynchronize(c->ev));
+      coef.assign(c->hscratch, c->hscratch + (size_t)P * 2 * nl);
+      dots_re_finish(c, off_host_dots(c), bb);
       std::vector<double> alpha(P);
       for (int p = 0; p < P; ++p) {
         alpha[p] = coef[(size_t)p * 2 * nl + 2 * (j - local_lo)];
@@ -1084,7 +1164,6 @@ int eigs_core(nfs_ctx* c, int nev, double* omega, double2* Y, nfs_eigs_info* inf
           for (int i = 0; i < j; ++i)
             H[p][(size_t)i * m + j] = H[p][(size_t)j * m + i] = coef[(size_t)p * 2 * nl + 2 * i];
       }
-      TRY(dots_re(c, s, w, Mw, bb));
       const std::vector<double> bb_recur = bb;
       std::vector<double> loss_first(P, 0.0);
       const double tr1 = now_s();
@@ -1100,7 +1179,9 @@ int eigs_core(nfs_ctx* c, int nev, double* omega, double2* Y, nfs_eigs_info* inf
       if (local_lo > 0) {
         std::vector<int> reorth(P, 0);
         for (int pass = 0; pass < 3; ++pass) {
-          TRY(exact_dots(c, local_lo, w, d, d_active));
+          if (pass > 0) TRY(exact_dots_start(c, local_lo, w, d_active, off_host_exact(c)));
+          CK(cudaStreamSynchronize(s));
+          d.assign(c->hscratch + off_host_exact(c), c->hscratch + off_host_exact(c) + (size_t)P * 2 * local_lo);
           bool any_re = false, big = false, big_loss = false;
           for (int p = 0; p < P; ++p) {
             reorth[p] = 0;
@@ -1123,7 +1204,7 @@ int eigs_core(nfs_ctx* c, int nev, double* omega, double2* Y, nfs_eigs_info* inf
             // rounding is ~6e-8 of the coefficients): remove the components
             // in FP64, with coefficients v_i^* A_r w from the stored A_r V
             TRY(multi_dot(c, c->MV, 0, local_lo, w, coef2, c->d_flags + P));
-            TRY(multi_axpy(c, w, Mw, 0, local_lo, coef2, c->d_flags + P));
+            TRY(multi_axpy(c, w, Mw, 0, local_lo, c->d_flags + P));
             for (int p = 0; p < P; ++p)
               if (reorth[p]) ++full_reorths[p];
           } else {
@@ -1162,17 +1243,21 @@ int eigs_core(nfs_ctx* c, int nev, double* omega, double2* Y, nfs_eigs_info* inf
       const int k = j + 1;
       if (k >= nwant + 1 && ((k - jstart) % check_every == 0 || j == m - 1)) {
         bool changed = false;
+        std::vector<std::vector<double>> th(P), zl(P);
+        std::vector<char> good(P, 1);
+        const double th0 = now_s();
+        const bool ran = for_problems(P, [&](int p) {
+          if (active[p]) good[p] = nfs::host::sym_eig(k, leading(p, k), th[p], zl[p], true);
+        });
+        c->sec_ritz += now_s() - th0;
+        if (!ran) return NFS_ENOMEM;
         for (int p = 0; p < P; ++p) {
           if (!active[p]) continue;
-          std::vector<double> zl;
-          const double th0 = now_s();
-          const bool ok = nfs::host::sym_eig(k, leading(p, k), theta, zl, true);
-          c->sec_ritz += now_s() - th0;
-          if (!ok) return NFS_EBREAKDOWN;
+          if (!good[p]) return NFS_EBREAKDOWN;
           int nc = 0;
           for (int i = 0; i < nwant; ++i) {
             const int cc = k - 1 - i;  // largest theta first
-            if (std::fabs(beta_last[p] * zl[cc]) <= c->opt.eig_tol * std::fabs(theta[cc])) ++nc;
+            if (std::fabs(beta_last[p] * zl[p][cc]) <= c->opt.eig_tol * std::fabs(th[p][cc])) ++nc;
           }
           nconv[p] = std::min(nc, nev);
           if (nc == nwant) {
@@ -1277,7 +1362,7 @@ int eigs_core(nfs_ctx* c, int nev, double* omega, double2* Y, nfs_eigs_info* inf
     TRY(matvec<double>(c, s, w, Mw));
     for (int pass = 0; pass < 2; ++pass) {
       TRY(multi_dot(c, c->MV, 0, nev, w, coef, d_active));
-      TRY(multi_axpy(c, w, Mw, 0, nev, coef, d_active));
+      TRY(multi_axpy(c, w, Mw, 0, nev, d_active));
     }
     TRY(dots_re(c, s, w, Mw, bb));
     for (int p = 0; p < P; ++p) {
@@ -1311,23 +1396,36 @@ int eigs_core(nfs_ctx* c, int nev, double* omega, double2* Y, nfs_eigs_info* inf
   std::vector<int> ok(P);
   std::vector<double> maxres(P, 0.0);
   bool any_ok = false;
+  std::vector<std::vector<double>> thp(P), Zp(P);
+  std::vector<char> good(P, 1);
+  if (!for_problems(P, [&](int p) { good[p] = nfs::host::sym_eig(jm[p], leading(p, jm[p]), thp[p], Zp[p]); }))
+    return NFS_ENOMEM;
+  std::vector<int> todo(P, 0);
   for (int p = 0; p < P; ++p) {
     const int k = jm[p];
-    if (!nfs::host::sym_eig(k, leading(p, k), theta, Z)) return NFS_EBREAKDOWN;
+    if (!good[p]) return NFS_EBREAKDOWN;
     for (int i = 0; i < nev; ++i) {
       const int cc = k - 1 - i;
-      omega[(size_t)p * nev + i] = 1.0 / theta[cc];
-      maxres[p] = std::max(maxres[p], std::fabs(beta_last[p] * Z[(size_t)(k - 1) * k + cc]) / std::fabs(theta[cc]));
+      omega[(size_t)p * nev + i] = 1.0 / thp[p][cc];
+      maxres[p] = std::max(maxres[p], std::fabs(beta_last[p] * Zp[p][(size_t)(k - 1) * k + cc]) / std::fabs(thp[p][cc]));
     }
     ok[p] = status[p] == NFS_OK;
     any_ok = any_ok || ok[p];
-    if (!ok[p] && !Y) continue;
-    // the Ritz vectors of problem p: rotate its basis (only p flagged)
+    todo[p] = ok[p] || Y;
+  }
+  // the Ritz vectors: rotate the bases, those of one size in one launch
+  for (int p0 = 0; p0 < P; ++p0) {
+    if (!todo[p0]) continue;
+    const int k = jm[p0];
     std::vector<double> Ycm((size_t)P * k * nev, 0.0);
-    for (int i = 0; i < nev; ++i)
-      for (int r = 0; r < k; ++r) Ycm[(size_t)p * k * nev + (size_t)i * k + r] = Z[(size_t)r * k + (k - 1 - i)];
     std::fill(one.begin(), one.end(), 0);
-    one[p] = 1;
+    for (int p = p0; p < P; ++p) {
+      if (!todo[p] || jm[p] != k) continue;
+      for (int i = 0; i < nev; ++i)
+        for (int r = 0; r < k; ++r) Ycm[(size_t)p * k * nev + (size_t)i * k + r] = Zp[p][(size_t)r * k + (k - 1 - i)];
+      one[p] = 1;
+      todo[p] = 0;
+    }
     TRY(put_flags(c, s, P, one));
     TRY(rotate(c, c->V, k, Ycm, nev, c->d_flags + P));
   }
