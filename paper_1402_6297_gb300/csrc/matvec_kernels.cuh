@@ -370,6 +370,19 @@ __device__ __forceinline__ double2 minus_groups(double2 a, const double2* tmp, l
   return a;
 }
 
+// Whether a thread of the scalar types' kernels fetches all that its items read
+// (nv of them, nt threads, `per` items per thread at most) when the kernel
+// starts.  The grids this holds for are bound by the chain of latencies from
+// one kernel to the next, not by the FP64 pipe: an item's operands fetched where
+// they are used add an L2 round trip behind each barrier.  CG iterations in
+// complex128 on GB300: 8^3 20.1 -> 19.4 us, 16^3 22.2 -> 21.5.  (On larger grids
+// a thread has several items, whose operands would not fit in its registers,
+// and other CTAs of the SM fill the gap.)
+template <typename R>
+__host__ __device__ constexpr bool kAhead(int nv, int nt, int per = 1) {
+  return sizeof(cplx<R>) == 16 && nv <= per * nt;
+}
+
 // (only complex128 kernels carry the Krylov pieces)
 struct NoKrylov {};
 template <typename R> struct KrylovOf { using type = NoKrylov; };
@@ -426,12 +439,21 @@ k_rows_in(const vecc<R>* u, typename ElemOf<R>::E* __restrict__ fld, const cplx<
     }
   };
   fetch(threadIdx.x);
+  // (one voxel per thread: its basis too; see kAhead)
+  constexpr bool AHEAD = kAhead<R>(NV, NT);
+  Basis<R> B;
+  if constexpr (AHEAD) {
+    if (threadIdx.x < NV) {
+      const int x = threadIdx.x % N, y = threadIdx.x / N * N2 + b;
+      voxel_basis<R>(basis, n, ((long long)i3 * N + y) * N + x, lam[x], lam[N + y], lam[2 * N + i3], alpha, beta, B);
+    }
+  }
   R bt = (R)0;
   if constexpr (CGT) {
     if (st != nullptr) {
       using P = typename RedAccFor<R>::partial;
       const P tol2 = *reinterpret_cast<const P*>(&st->tol2), last = *reinterpret_cast<const P*>(&st->rr_last);
-      const bool over = st->halt || st->it >= st->maxit;
+      const bool over = (st->halt != 0) | (st->it >= st->maxit);
       const P rr = sum_partials_all<R, NT>(st->part_b, gridDim.x * n3);
       const bool stop = over || scalar_nan(rr) || scalar_le(rr, tol2);
       if (blockIdx.x == 0 && i3 == 0 && threadIdx.x == 0) {
@@ -477,8 +499,7 @@ k_rows_in(const vecc<R>* u, typename ElemOf<R>::E* __restrict__ fld, const cplx<
         }
       }
     }
-    Basis<R> B;
-    voxel_basis<R>(basis, n, e, lam[x], lam[N + y], a3, alpha, beta, B);
+    if constexpr (!AHEAD) voxel_basis<R>(basis, n, e, lam[x], lam[N + y], a3, alpha, beta, B);
     E* cell = buf + row * PITCH + x;
     if constexpr (NF == 1) {
       C p[3], q[3];
@@ -655,6 +676,19 @@ k_columns(typename ElemOf<R>::E* __restrict__ fld, Step step, const cplx<R>* __r
   E* tile = fld + prob * bs.sfld + (long long)j * NF * n + ((long long)a * N + xt * X / XL * XL) * (N3 * N2) + xt * X % XL;
   auto gaddr = [&](int l, int z) { return tile + (l / L) * n + z * (N2 * XL) + l % L / X * XL + l % X; };
   if (stop) return;
+  auto position = [&](int xi, int zs) {
+    return ColumnPos{j,  a, xt * X + xi, zs, prob, slot_index<N2>(xt * X + xi, N1), slot_index<Z2>(zs, Z1), N, N1, N3};
+  };
+  constexpr int VITEMS = L * N3;
+  constexpr bool AHEAD = NF == 2 && kAhead<R>(VITEMS, NT, 2);
+  typename Step::template Vals<1> ahead[2];
+  if constexpr (AHEAD) {
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const int it = threadIdx.x + t * NT;
+      if (it < VITEMS) step.template load<1>(position(it / N3 % X, it % N3), it / N3 / X, ahead[t]);
+    }
+  }
   __syncthreads();  // twiddles
   // inverse stage A along z from the workspace
   {
@@ -679,9 +713,6 @@ k_columns(typename ElemOf<R>::E* __restrict__ fld, Step step, const cplx<R>* __r
   }
   // stage B along y, the material step, stage A' along y
   RedAccFor<R> dot;
-  auto position = [&](int xi, int zs) {
-    return ColumnPos{j,  a, xt * X + xi, zs, prob, slot_index<N2>(xt * X + xi, N1), slot_index<Z2>(zs, Z1), N, N1, N3};
-  };
   if constexpr (NF == 1) {
     // all in registers: items (x slot, z slot), the z slot fastest across
     // threads (odd pitch)
@@ -728,19 +759,27 @@ k_columns(typename ElemOf<R>::E* __restrict__ fld, Step step, const cplx<R>* __r
       for (int k = 0; k < N2; ++k) cell[k * X] = v[k];
     }
     __syncthreads();
-    constexpr int VITEMS = L * N3;
-#pragma unroll 1
-    for (int it = threadIdx.x; it < VITEMS; it += NT) {
+    auto voxel_step = [&](int it, typename Step::template Vals<1>& mv) {
       const int zs = it % N3, l = it / N3;
       const ColumnPos pos = position(l % X, zs);
-      typename Step::template Vals<1> mv;
-      step.template load<1>(pos, l / X, mv);
+      if constexpr (!AHEAD) step.template load<1>(pos, l / X, mv);
       E* cell = buf + zs * PITCH + l;
       C p = cell[0], q = cell[L];
       const R s = step.template apply<1>(pos, l / X, mv, 0, p, q);
       if (st != nullptr) dot.add(static_cast<typename RedAccFor<R>::value_type>(s));
       cell[0] = p;
       cell[L] = q;
+    };
+    if constexpr (AHEAD) {
+#pragma unroll
+      for (int t = 0; t < 2; ++t)
+        if (threadIdx.x + t * NT < VITEMS) voxel_step(threadIdx.x + t * NT, ahead[t]);
+    } else {
+#pragma unroll 1
+      for (int it = threadIdx.x; it < VITEMS; it += NT) {
+        typename Step::template Vals<1> mv;
+        voxel_step(it, mv);
+      }
     }
     if constexpr (Step::kForward) {
       __syncthreads();
@@ -845,6 +884,27 @@ k_rows_out(const typename ElemOf<R>::E* __restrict__ fld, vecc<R>* __restrict__ 
   Au += prob * bs.su;
   lam += (long long)prob * bs.slam;
   if (basis != nullptr) basis += prob * bs.sbasis;
+  // one voxel per thread: the operands of the last step (see kAhead)
+  constexpr bool AHEAD = kAhead<R>(NV, NT);
+  Basis<R> B;
+  vecc<R> pv[NQ], xv[NQ], rv[NQ];
+  if constexpr (AHEAD) {
+    if (threadIdx.x < NV) {
+      const int x = threadIdx.x % N, y = b + N2 * (threadIdx.x / N);
+      const long long e = ((long long)i3 * N + y) * N + x;
+      if constexpr (CGT) {
+        if (st != nullptr) {
+#pragma unroll
+          for (int q = 0; q < NQ; ++q) {
+            pv[q] = cg.p[e + q * n];
+            rv[q] = cg.r[e + q * n];
+            xv[q] = cg.x[e + q * n];
+          }
+        }
+      }
+      voxel_basis<R>(basis, n, e, lam[x], lam[N + y], lam[2 * N + i3], alpha, beta, B);
+    }
+  }
   // stage B' along y from the workspace: row k of the CTA is y = b + N2 k
 #pragma unroll 1
   for (int it = threadIdx.x; it < 3 * N; it += NT) {
@@ -893,8 +953,7 @@ k_rows_out(const typename ElemOf<R>::E* __restrict__ fld, vecc<R>* __restrict__ 
   for (int vi = threadIdx.x; vi < NV; vi += NT) {
     const int row = vi / N, x = vi % N, y = b + N2 * row;
     const long long e = ((long long)i3 * N + y) * N + x;
-    vecc<R> pv[NQ], xv[NQ], rv[NQ];
-    if constexpr (CGT) {
+    if constexpr (CGT && !AHEAD) {
       if (ok) {
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
@@ -904,8 +963,7 @@ k_rows_out(const typename ElemOf<R>::E* __restrict__ fld, vecc<R>* __restrict__ 
         }
       }
     }
-    Basis<R> B;
-    voxel_basis<R>(basis, n, e, lam[x], lam[N + y], a3, alpha, beta, B);
+    if constexpr (!AHEAD) voxel_basis<R>(basis, n, e, lam[x], lam[N + y], a3, alpha, beta, B);
     // P_r^* f = [-sum conj(c) f ; sum conj(x) f],  Q_r^* w = [sum x w ; sum c w]
     const E* cell = buf + row * PITCH + x;
     C o[NQ];
