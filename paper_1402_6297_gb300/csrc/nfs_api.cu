@@ -532,7 +532,11 @@ int solve(nfs_ctx* c, const double2* b, double2* x, bool x_zero, const std::vect
     CK(cudaMemsetAsync(x, 0, tot * sizeof(double2), s));
     CK(cudaMemcpyAsync(c->r64, b, tot * sizeof(double2), cudaMemcpyDeviceToDevice, s));
   } else {
-    TRY(matvec<double>(c, s, x, c->Ap64));
+    // (mixed: by the double-single product, as the residuals that follow)
+    if (c->opt.precision == NFS_PREC_MIXED)
+      TRY(matvec<nfs::df>(c, s, x, c->Ap64));
+    else
+      TRY(matvec<double>(c, s, x, c->Ap64));
     TRY(sub64(c, s, b, c->Ap64, c->r64));
   }
   std::vector<int> need(P);
