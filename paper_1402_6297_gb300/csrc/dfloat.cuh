@@ -66,11 +66,4 @@ template <> struct CplxOf<df> { using type = dfc; };
 template <> struct RealOf<dfc> { using type = df; };
 __host__ __device__ __forceinline__ dfc mk(df a, df b) { return dfc{a, b}; }
 
-// The element type of the double-single product in memory: 16 bytes
-// (re.hi, re.lo, im.hi, im.lo), loaded and stored as one float4.
-__device__ __forceinline__ dfc ldg_c(const dfc* p) {
-  const float4 v = __ldg(reinterpret_cast<const float4*>(p));
-  return dfc{df(v.x, v.y), df(v.z, v.w)};
-}
-
 }  // namespace nfs

@@ -97,7 +97,16 @@ struct MatView {
 // depend_begin() lets the next kernel of the stream start, depend_wait() waits
 // for the one before to end with its writes visible.  Every CTA waits before it
 // touches anything but constant tables, and before it returns: a kernel that
-// ended earlier would let its successor run ahead of its predecessor.
+// ended earlier would let its successor run ahead of its predecessor.  (The
+// Gram-Schmidt kernels also read older basis vectors ahead of the wait, see
+// load_l2.)
+//
+// Such a kernel is alive while its predecessor writes, so what any kernel on the
+// stream writes is read by plain loads from plain pointers: __ldg and const
+// __restrict__ promise the compiler and the hardware that the data does not
+// change during the kernel's life (a load may then move above the wait, whose
+// "memory" clobber does not reach a __restrict__ pointer).  Only the tables of
+// set-up (lam, tw*, basis, the material) keep them.
 __device__ __forceinline__ void depend_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void depend_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -395,8 +404,8 @@ constexpr size_t rows_smem() {
 
 template <typename R, int N, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
-k_rows_in(const vecc<R>* u, typename ElemOf<R>::E* __restrict__ fld, const cplx<R>* __restrict__ lam,
-          const cplx<R>* __restrict__ twx, R alpha, R beta, int kind, int ax_a, int ax_b, const int* __restrict__ skip,
+k_rows_in(const vecc<R>* u, typename ElemOf<R>::E* fld, const cplx<R>* __restrict__ lam,
+          const cplx<R>* __restrict__ twx, R alpha, R beta, int kind, int ax_a, int ax_b, const int* skip,
           const cplx<R>* __restrict__ basis, BatchStrides bs, CgFuse<R> cg, typename KrylovOf<R>::type kr) {
   using C = cplx<R>;
   using E = typename ElemOf<R>::E;
@@ -434,7 +443,7 @@ k_rows_in(const vecc<R>* u, typename ElemOf<R>::E* __restrict__ fld, const cplx<
       for (int q = 0; q < NQ; ++q) v[q] = u[q * n + e];
       if (r_in != nullptr) {
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) g[q] = ldg_c(r_in + q * n + e);
+        for (int q = 0; q < NQ; ++q) g[q] = r_in[q * n + e];
       }
     }
   };
@@ -651,8 +660,8 @@ constexpr size_t columns_smem() {
 // The plane edge N1 N2 is a run-time value (it only sets strides).
 template <typename R, int N2, int X, int XL, int N3, int NT, int MINB, class Step>
 __global__ void __launch_bounds__(NT, MINB)
-k_columns(typename ElemOf<R>::E* __restrict__ fld, Step step, const cplx<R>* __restrict__ twy,
-          const cplx<R>* __restrict__ twz, const int* __restrict__ skip, CGState* st, BatchStrides bs) {
+k_columns(typename ElemOf<R>::E* fld, Step step, const cplx<R>* __restrict__ twy, const cplx<R>* __restrict__ twz,
+          const int* skip, CGState* st, BatchStrides bs) {
   using C = cplx<R>;
   using E = typename ElemOf<R>::E;
   using S = DepthSplit<R, N3>;
@@ -833,10 +842,9 @@ k_columns(typename ElemOf<R>::E* __restrict__ fld, Step step, const cplx<R>* __r
 // ---------------------------------------------------------------------------
 template <typename R, int N, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
-k_rows_out(const typename ElemOf<R>::E* __restrict__ fld, vecc<R>* __restrict__ Au, const cplx<R>* __restrict__ lam,
-           const cplx<R>* __restrict__ twx, R alpha, R beta, int kind, int ax_a, int ax_b,
-           const int* __restrict__ skip, const cplx<R>* __restrict__ basis, BatchStrides bs, CgFuse<R> cg,
-           typename KrylovOf<R>::type kr) {
+k_rows_out(const typename ElemOf<R>::E* fld, vecc<R>* Au, const cplx<R>* __restrict__ lam,
+           const cplx<R>* __restrict__ twx, R alpha, R beta, int kind, int ax_a, int ax_b, const int* skip,
+           const cplx<R>* __restrict__ basis, BatchStrides bs, CgFuse<R> cg, typename KrylovOf<R>::type kr) {
   using C = cplx<R>;
   using E = typename ElemOf<R>::E;
   using S = PlaneSplit<R, N>;

@@ -116,15 +116,23 @@ constexpr int kGsTile = 128;      // elements of w that a block of k_gs_dots hol
 constexpr int kGsMaxChunks = 64;
 constexpr int kGsPerWarp = 2;     // vectors per warp (4: the FP64 work of a block takes 3 us instead of 1.9)
 
-// (The kernels fetch what they need of the older basis vectors before they wait
-// for the kernel before them: those vectors were complete when that kernel
-// passed its own wait, which is before it let this one start.)
+// The kernels fetch what they need of the older basis vectors before they wait
+// for the kernel before them.  All but the newest vector were written by kernels
+// that had ended when the predecessor passed its own wait, which it did before it
+// let this one start; their writes are in the L2 by then, and the load takes
+// them from there (a line of the L1 may be older than they are).  The newest one,
+// which k_rows_out normalises, is read after the wait by a plain load.
+__device__ __forceinline__ double2 load_l2(const double2* p) {
+  double2 v;
+  asm volatile("ld.global.cg.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+  return v;
+}
 
 // grid (S, ceil(m / 8)): part[(s m + j) 2 + {0, 1}] = chunk s's share of
 // V_j^* w', w' = w - sum_{g < G} tmp_g (written to w2 when G > 0)
 __global__ void __launch_bounds__(kGsTile)
-k_gs_dots(const double2* __restrict__ V, int m, const double2* w, const double2* tmp, int G, double2* w2, long long N,
-          long long chunk, double* __restrict__ part) {
+k_gs_dots(const double2* V, int m, const double2* w, const double2* tmp, int G, double2* w2, long long N,
+          long long chunk, double* part) {
   constexpr int PER = kGsTile / 32;  // elements of a tile per lane
   __shared__ double2 ws[kGsTile];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -132,19 +140,21 @@ k_gs_dots(const double2* __restrict__ V, int m, const double2* w, const double2*
   const int s = blockIdx.x;
   const long long i0 = (long long)s * chunk, i1 = min(N, i0 + chunk);
   double2 x[kGsPerWarp][PER];
-  auto fetch = [&](long long base, int from, int to) {
+  auto fetch = [&](long long base, int from, int to, auto load) {
 #pragma unroll
     for (int t = 0; t < kGsPerWarp; ++t)
       if (j0 + t >= from && j0 + t < to)
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
           const long long i = base + k * 32 + lane;
-          x[t][k] = i < i1 ? V[(long long)(j0 + t) * N + i] : make_double2(0.0, 0.0);
+          x[t][k] = i < i1 ? load(V + (long long)(j0 + t) * N + i) : make_double2(0.0, 0.0);
         }
   };
-  fetch(i0, 0, m - 1);  // (the newest vector may still be being normalised)
+  auto plain = [](const double2* p) { return *p; };
+  auto older = [](const double2* p) { return load_l2(p); };
+  fetch(i0, 0, m - 1, older);  // (the newest vector may still be being normalised)
   depend_wait();
-  fetch(i0, m - 1, m);
+  fetch(i0, m - 1, m, plain);
   double acc[2 * kGsPerWarp];
 #pragma unroll
   for (int t = 0; t < 2 * kGsPerWarp; ++t) acc[t] = 0.0;
@@ -156,7 +166,7 @@ k_gs_dots(const double2* __restrict__ V, int m, const double2* w, const double2*
       if (G > 0 && blockIdx.y == 0) w2[i] = a;
     }
     if (base > i0) {
-      fetch(base, 0, m);
+      fetch(base, 0, m, plain);
       __syncthreads();  // the tile before has been read
     }
     ws[threadIdx.x] = a;
@@ -195,7 +205,7 @@ k_gs_dots(const double2* __restrict__ V, int m, const double2* w, const double2*
 // vectors of c_j V_j[i], c_j = sum over the S chunks' partials
 template <int NT>
 __global__ void __launch_bounds__(NT)
-k_gs_update(const double2* __restrict__ V, long long N, int m, int VB, const double* part, int S, double2* tmp) {
+k_gs_update(const double2* V, long long N, int m, int VB, const double* part, int S, double2* tmp) {
   constexpr int AHEAD = 12;  // vectors fetched before the wait
   __shared__ double2 cs[kGmresMax];
   const int j0 = blockIdx.y * VB, nj = min(VB, m - j0);
@@ -204,8 +214,11 @@ k_gs_update(const double2* __restrict__ V, long long N, int m, int VB, const dou
   double2 x[AHEAD];
 #pragma unroll
   for (int t = 0; t < AHEAD; ++t)
-    if (t < nj) x[t] = v[(long long)t * N];
+    if (t < nj && j0 + t < m - 1) x[t] = load_l2(v + (long long)t * N);
   depend_wait();
+#pragma unroll
+  for (int t = 0; t < AHEAD; ++t)
+    if (t < nj && j0 + t == m - 1) x[t] = v[(long long)t * N];
   // four threads add up one coefficient
   for (int t = threadIdx.x; t < (nj + NT / 4 - 1) / (NT / 4) * NT; t += NT) {
     const int j = t / 4;
@@ -259,8 +272,7 @@ __device__ __forceinline__ double gs_block_sum(double v) {
 
 // dst = w - sum_g tmp_g, and (nrm_part != nullptr) the partials of |dst|^2
 __global__ void __launch_bounds__(kGsThreads)
-k_gs_finish(const double2* w, const double2* __restrict__ tmp, int G, double2* dst, long long N,
-            double* __restrict__ nrm_part) {
+k_gs_finish(const double2* w, const double2* tmp, int G, double2* dst, long long N, double* nrm_part) {
   depend_wait();
   double nr = 0.0;
   for (long long i = (long long)blockIdx.x * kGsThreads + threadIdx.x; i < N; i += (long long)gridDim.x * kGsThreads) {
@@ -291,8 +303,8 @@ k_gmres_residual(const double2* __restrict__ b, double2* __restrict__ w, long lo
 // two passes at part + 2 t plen (and + plen), its norm partials at nrm + t nlen
 // (nnrm of them; the last step's at nrm_last, nlast of them).
 __global__ void __launch_bounds__(kGsThreads)
-k_gmres_columns(int j0, const double* __restrict__ part, long long plen, int S, const double* __restrict__ nrm,
-                long long nlen, int nnrm, const double* __restrict__ nrm_last, int nlast, GmresDev* st) {
+k_gmres_columns(int j0, const double* part, long long plen, int S, const double* nrm, long long nlen, int nnrm,
+                const double* nrm_last, int nlast, GmresDev* st) {
   depend_wait();
   depend_begin();
   const int t = blockIdx.x, j = j0 + t, m = j + 1;
