@@ -114,14 +114,17 @@ k_cg_init(CGState* st, const double* __restrict__ tol2, bool relative, int maxit
 }
 
 // End of a chunk of CG steps, one block per problem: the state that the host
-// reads, from the nb partials of r^* r (k_rows_in reaches the same decision from
-// the same partials when another chunk follows).
+// reads, from the nb partials of r^* r.  Where the steps have stopped, r^* r is
+// the sum that k_rows_in stopped them by: its blocks add the partials up in
+// another order, which may round to the other side of the threshold, and a state
+// that steps no more has to be done.
 template <typename R>
 __global__ void __launch_bounds__(kRedThreads) k_cg_check(CGState* st, int nb) {
   using P = typename RedAccFor<R>::partial;
   st += blockIdx.x;
-  const P rr = sum_partials_all<R, kRedThreads>(st->part_b, nb);
+  const P sum = sum_partials_all<R, kRedThreads>(st->part_b, nb);
   if (threadIdx.x == 0) {
+    const P rr = st->halt ? *reinterpret_cast<const P*>(&st->rr_now) : sum;
     st->rr = scalar_double(rr);
     const bool bad = st->broken || scalar_nan(rr);
     const bool conv = scalar_le(rr, *reinterpret_cast<const P*>(&st->tol2));

@@ -472,6 +472,8 @@ int cg_run(nfs_ctx* c, nfs::cplx<R>* x, nfs::cplx<R>* r, nfs::cplx<R>* p, const 
       last = std::min(ran, (it + kCgChunk - 1) / kCgChunk);
       break;
     }
+    // (a chunk ends a problem or takes kCgChunk of its maxit steps)
+    if (ran > maxit / kCgChunk + 1) return NFS_EBREAKDOWN;
   }
   iters.resize(c->P);
   status.resize(c->P);
