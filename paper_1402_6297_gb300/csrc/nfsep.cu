@@ -146,8 +146,9 @@ k_gs_dots(const double2* V, int m, const double2* w, const double2* tmp, int G, 
       if (j0 + t >= from && j0 + t < to)
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
-          const long long i = base + k * 32 + lane;
-          x[t][k] = i < i1 ? load(V + (long long)(j0 + t) * N + i) : make_double2(0.0, 0.0);
+          // (past the chunk: any element, which meets a zero of ws)
+          const long long i = min(base + k * 32 + lane, N - 1);
+          x[t][k] = load(V + (long long)(j0 + t) * N + i);
         }
   };
   auto plain = [](const double2* p) { return *p; };
@@ -212,13 +213,17 @@ k_gs_update(const double2* V, long long N, int m, int VB, const double* part, in
   const long long i = (long long)blockIdx.x * NT + threadIdx.x;
   const double2* v = V + (long long)j0 * N + (i < N ? i : 0);
   double2 x[AHEAD];
+  // (older vectors of the group; the newest, if it is among the AHEAD, comes
+  // after the wait and is added behind them)
+  const int older = min(nj, m - 1 - j0), fetched = min(older, AHEAD);
+  const bool newest = older < nj && older < AHEAD;
+  if (older > 0) {
 #pragma unroll
-  for (int t = 0; t < AHEAD; ++t)
-    if (t < nj && j0 + t < m - 1) x[t] = load_l2(v + (long long)t * N);
+    for (int t = 0; t < AHEAD; ++t) x[t] = load_l2(v + (long long)min(t, older - 1) * N);
+  }
   depend_wait();
-#pragma unroll
-  for (int t = 0; t < AHEAD; ++t)
-    if (t < nj && j0 + t == m - 1) x[t] = v[(long long)t * N];
+  double2 xn = make_double2(0.0, 0.0);
+  if (newest) xn = v[(long long)older * N];
   // four threads add up one coefficient
   for (int t = threadIdx.x; t < (nj + NT / 4 - 1) / (NT / 4) * NT; t += NT) {
     const int j = t / 4;
@@ -245,8 +250,13 @@ k_gs_update(const double2* V, long long N, int m, int VB, const double* part, in
   double2 a0 = make_double2(0.0, 0.0), a1 = a0;
 #pragma unroll
   for (int t = 0; t < AHEAD; t += 2) {
-    if (t < nj) a0 = cadd(a0, cmul(cs[t], x[t]));
-    if (t + 1 < nj) a1 = cadd(a1, cmul(cs[t + 1], x[t + 1]));
+    if (t < fetched) a0 = cadd(a0, cmul(cs[t], x[t]));
+    if (t + 1 < fetched) a1 = cadd(a1, cmul(cs[t + 1], x[t + 1]));
+  }
+  if (newest) {
+    const double2 y = cmul(cs[older], xn);
+    if (older % 2 == 0) a0 = cadd(a0, y);
+    else a1 = cadd(a1, y);
   }
   int j = AHEAD;
   for (; j + 8 <= nj; j += 8) {
