@@ -147,9 +147,15 @@ def main():
                 if knob in KNOB_SIZES and not (KNOB_SIZES[knob] & set(sizes)):
                     continue
                 cands = [dict(best, **{knob: v}) for v in values if v != best[knob]]
+
+                def prebuild(d):
+                    try:
+                        build_variant(d, workdir)
+                    except RuntimeError:
+                        cache[tuple(sorted(d.items()))] = None  # does not compile: no candidate
+
                 with cf.ThreadPoolExecutor(max_workers=args.jobs) as ex:
-                    list(ex.map(lambda d: build_variant(d, workdir) if tuple(sorted(d.items())) not in cache else None,
-                                cands))
+                    list(ex.map(prebuild, [d for d in cands if tuple(sorted(d.items())) not in cache]))
                 for cand in cands:
                     sc = score(cand, sizes, workdir, cache)
                     print(json.dumps({"try": {knob: cand[knob]}, "score": sc}), flush=True)

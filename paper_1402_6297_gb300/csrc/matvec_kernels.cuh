@@ -164,11 +164,17 @@ __device__ __forceinline__ double block_sum_dbl(double v) {
 #ifndef NFS_XL
 #define NFS_XL 4
 #endif
+constexpr int common_divisor(int a, int b) { return b == 0 ? a : common_divisor(b, a % b); }
 template <typename R, int N> struct PlaneSplit {
   static constexpr bool F32 = sizeof(cplx<R>) == 8;
   static constexpr int N2 = N < 24 ? 4 : (F32 && N == 48) ? NFS_N2_48 : (F32 && N == 96) ? NFS_N2_96 : 8, N1 = N / N2;
   static constexpr int X = N < 24 ? 1 : NFS_X;
-  static constexpr int XL = NFS_XL;
+  // (whole runs of whole tiles: the largest part of NFS_XL that divides the
+  // edge, but no shorter than a tile.  A run that does not divide it would share
+  // its room with the next row's, and leave the workspace at its end)
+  static constexpr int RUN = common_divisor(N, NFS_XL);
+  static constexpr int XL = RUN % X == 0 ? RUN : X;
+  static_assert(N % N2 == 0 && N % XL == 0 && XL % X == 0, "the x slots of a row come in whole runs of whole tiles");
 };
 
 // N = N1 N2 of the z transforms.  The packed elements take the shortest lengths
@@ -681,7 +687,6 @@ k_columns(typename ElemOf<R>::E* fld, Step step, const cplx<R>* __restrict__ twy
   const int stop = st != nullptr ? st[prob].stop : 0;
   const int N1 = gridDim.y, N = N1 * N2;
   const long long n = (long long)N * N * N3;
-  static_assert(XL % X == 0, "a column tile lies within one run of the workspace");
   E* tile = fld + prob * bs.sfld + (long long)j * NF * n + ((long long)a * N + xt * X / XL * XL) * (N3 * N2) + xt * X % XL;
   auto gaddr = [&](int l, int z) { return tile + (l / L) * n + z * (N2 * XL) + l % L / X * XL + l % X; };
   if (stop) return;
