@@ -143,6 +143,16 @@ __global__ void k_sub(const C* __restrict__ a, const C* __restrict__ b, C* __res
     y[i] = csub(a[i], b[i]);
 }
 
+// *mark = 1 if an entry of x is not zero (a NaN is not)
+__global__ void k_mark_nonzero(const double2* __restrict__ x, long long total, int* mark) {
+  bool any = false;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+    const double2 v = x[i];
+    any = any || !(v.x == 0.0) || !(v.y == 0.0);
+  }
+  if (any) *mark = 1;
+}
+
 __global__ void k_add(const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ y, long long n) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     y[i] = a[i] + b[i];

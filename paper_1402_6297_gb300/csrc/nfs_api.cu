@@ -495,6 +495,21 @@ int sub64(nfs_ctx* c, cudaStream_t s, const double2* a, const double2* b, double
   return NFS_OK;
 }
 
+// Whether every entry of the P vectors x is zero (mixed solves: without a start,
+// as the binding's solve without one, the first residual is b itself; its
+// product would cost as much as 20 CG iterations, 1.6 ms at 96^3).
+int is_zero(nfs_ctx* c, cudaStream_t s, const double2* x, bool& zero) {
+  const long long tot = c->P * c->N;
+  TRY(put_flags(c, s, c->P, std::vector<int>(1, 0)));
+  nfs::k_mark_nonzero<<<grid_blocks(tot, 256), 256, 0, s>>>(x, tot, c->d_flags + c->P);
+  CK(cudaGetLastError());
+  c->launches += 1;
+  CK(cudaMemcpyAsync(c->h_flags + c->P, c->d_flags + c->P, sizeof(int), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  zero = c->h_flags[c->P] == 0;
+  return NFS_OK;
+}
+
 // Solve A_r x_p = b_p for every problem p with active[p] (b, x: P x N, on the
 // work stream).  FP64 contexts run complex128 CG; MIXED contexts run complex64
 // CG inside FP64 iterative refinement (the residual r = b - A_r x with the
@@ -534,11 +549,9 @@ int solve(nfs_ctx* c, const double2* b, double2* x, bool x_zero, const std::vect
     CK(cudaMemsetAsync(x, 0, tot * sizeof(double2), s));
     CK(cudaMemcpyAsync(c->r64, b, tot * sizeof(double2), cudaMemcpyDeviceToDevice, s));
   } else {
-    // (mixed: by the double-single product, as the residuals that follow)
-    if (c->opt.precision == NFS_PREC_MIXED)
-      TRY(matvec<nfs::df>(c, s, x, c->Ap64));
-    else
-      TRY(matvec<double>(c, s, x, c->Ap64));
+    // (complex128 in mixed contexts too, whose later residuals are double-single:
+    // a start may be better than 48 bits can tell)
+    TRY(matvec<double>(c, s, x, c->Ap64));
     TRY(sub64(c, s, b, c->Ap64, c->r64));
   }
   std::vector<int> need(P);
@@ -1926,9 +1939,11 @@ extern "C" int nfs_cg_solve(nfs_ctx* c, const void* b, void* x, nfs_solve_info* 
   const size_t bytes = (size_t)c->P * c->N * sizeof(double2);
   CK(cudaMemcpyAsync(c->t64b, b, bytes, cudaMemcpyDeviceToDevice, c->work));
   CK(cudaMemcpyAsync(c->t64, x, bytes, cudaMemcpyDeviceToDevice, c->work));
+  bool x_zero = false;
+  if (c->opt.precision == NFS_PREC_MIXED) TRY(is_zero(c, c->work, c->t64, x_zero));
   SolveOut so;
   std::vector<int> active(c->P, 1);
-  TRY(solve(c, c->t64b, c->t64, false, active, so));
+  TRY(solve(c, c->t64b, c->t64, x_zero, active, so));
   CK(cudaMemcpyAsync(x, c->t64, bytes, cudaMemcpyDeviceToDevice, c->work));
   CK(cudaStreamSynchronize(c->work));
   if (info) {
