@@ -8,6 +8,7 @@
 // partial per block, and a one-block kernel sums the partials in a fixed
 // order.
 #pragma once
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 
@@ -15,6 +16,34 @@
 #include "nfs_complex.cuh"
 
 namespace nfs {
+
+// Blocks per problem of the reductions over P problems' vectors of length N.
+// Never more blocks than the vector has threads' worth of elements (empty
+// blocks add exact zeros: a single problem's sums are the same at any larger
+// count); for batches, fewer, with at least 32 elements per thread, as long
+// as all problems together still have kRedBlocks blocks.  Each block ends in
+// FP64 block sums, which GB300 retires at about one warp instruction per 17
+// SM cycles: a full grid per problem over the short vectors of a batch of
+// small grids made those epilogues, not the data, the cost of a reduction.
+inline int red_blocks(long long N, int P) {
+  long long nb = std::min<long long>(kRedBlocks, (N + kRedThreads - 1) / kRedThreads);
+  if (P > 1) {
+    const long long per32 = (N + (long long)kRedThreads * 32 - 1) / ((long long)kRedThreads * 32);
+    nb = std::min(nb, std::max<long long>(per32, (kRedBlocks + P - 1) / P));
+  }
+  return (int)std::max<long long>(1, nb);
+}
+
+// Blocks per problem and pair of k_exact_dots over m vectors: with many vectors
+// half of them, for fewer FP64 ends of blocks.  A thread's FP32 sums are then as
+// long as those of one element at a time over all the blocks, since it keeps two
+// of each.  52 vectors on one GB300, with k_dots_finish, all blocks and half of
+// them: 96^3 636 and 594 us, 64^3 271 and 217, 32^3 137 and 82, 16 problems of
+// 32^3 428 and 383.
+inline int exact_dots_blocks(long long N, int P, int m) {
+  const int nb = red_blocks(N, P);
+  return m < 16 ? nb : (nb + 1) / 2;
+}
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -538,10 +567,13 @@ k_dots_finish(const double* __restrict__ part, int m, int nb, double* __restrict
 // flight.  Bound by memory, 16 bytes per element and vector: all pairs of one
 // range of elements run together (their w is read from L2) and few blocks per
 // pair, whose FP64 ends (a pair sum per value, then the block's) would otherwise
-// show.  One GB300, 96^3, 52 vectors on average: 738 us with 304 blocks per pair,
-// 8-byte loads and a full block sum per value, 693 with this body but all blocks
-// of one pair together (w from memory again for every pair), 649 now (430 us at
-// the copy rate); 16 problems of 32^3: 378, 364, 339 us.
+// show.  One GB300, 52 vectors, with k_dots_finish: 752 us at 96^3 and 174 at 32^3
+// with 304 blocks per pair, 8-byte loads, a full block sum per value and the
+// blocks of one pair together (w from memory again for every pair), 594 and 82 now
+// (430 at 96^3 at the copy rate).  The error against 64 bits, rms of 40 products of
+// random vectors over the sum of the terms' magnitudes: 3.8e-18 then and 3.9e-18
+// now at 96^3, 7.8e-18 and 8.0e-18 at 32^3; with one FP32 sum for both elements of
+// the pair 1.2e-17 at 32^3.
 __global__ void __launch_bounds__(kRedThreads)
 k_exact_dots(const float2* __restrict__ Shi, const float2* __restrict__ Slo, long long sstride, int m,
              const float2* __restrict__ whi, const float2* __restrict__ wlo, long long N, double* __restrict__ part,
@@ -557,12 +589,14 @@ k_exact_dots(const float2* __restrict__ Shi, const float2* __restrict__ Slo, lon
                           reinterpret_cast<const float4*>(Shi + p * sstride + j1 * N)};
   const float4* sl4[G] = {reinterpret_cast<const float4*>(Slo + p * sstride + j0 * N),
                           reinterpret_cast<const float4*>(Slo + p * sstride + j1 * N)};
-  // per vector: the exact sum of the hi x hi products (real, imaginary) and
-  // an ordinary sum of their rounding errors and the hi x lo, lo x hi terms
-  DSAccX2 acc[G];
-  float2 small[G];
+  // per vector and element of the pair: the exact sum of the hi x hi products
+  // (real, imaginary) and an ordinary sum of their rounding errors and the hi x
+  // lo, lo x hi terms.  (Apart for the two elements: the error of the ordinary
+  // sums grows with their length.)
+  DSAccX2 acc[G][2];
+  float2 small[G][2];
 #pragma unroll
-  for (int g = 0; g < G; ++g) small[g] = make_float2(0.f, 0.f);
+  for (int g = 0; g < G; ++g) small[g][0] = small[g][1] = make_float2(0.f, 0.f);
   for (long long i = (long long)blockIdx.y * kRedThreads + threadIdx.x; i < N / 2; i += (long long)gridDim.y * kRedThreads) {
     const float4 bh4 = wh4[i], bl4 = wl4[i];
     float4 ah4[G], al4[G];
@@ -585,16 +619,22 @@ k_exact_dots(const float2* __restrict__ Shi, const float2* __restrict__ Slo, lon
         float2 p1, e1, p2, e2;
         two_prod_x2(ax, bh, p1, e1);
         two_prod_x2(ay, bh2, p2, e2);
-        acc[g].add(p1);
-        acc[g].add(p2);
+        acc[g][h].add(p1);
+        acc[g][h].add(p2);
         float2 t = add_x2(e1, e2);
         t = fma_x2(ax, bl, t);
         t = fma_x2(make_float2(al.x, al.x), bh, t);
         t = fma_x2(ay, bl2, t);
         t = fma_x2(make_float2(al.y, al.y), bh2, t);
-        small[g] = add_x2(small[g], t);
+        small[g][h] = add_x2(small[g][h], t);
       }
     }
+  }
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    acc[g][0].add(acc[g][1].hi);
+    acc[g][0].lo = add_x2(acc[g][0].lo, acc[g][1].lo);
+    small[g][0] = add_x2(small[g][0], small[g][1]);
   }
   // block sums in FP64.  (Double-single sums on the FP32 units lost the
   // accuracy the monitor needs on homogeneous media at symmetric k-points:
@@ -604,8 +644,8 @@ k_exact_dots(const float2* __restrict__ Shi, const float2* __restrict__ Slo, lon
   double v[2 * G];
 #pragma unroll
   for (int g = 0; g < G; ++g) {
-    v[2 * g] = (double)acc[g].hi.x + (double)acc[g].lo.x + (double)small[g].x;
-    v[2 * g + 1] = (double)acc[g].hi.y + (double)acc[g].lo.y + (double)small[g].y;
+    v[2 * g] = (double)acc[g][0].hi.x + (double)acc[g][0].lo.x + (double)small[g][0].x;
+    v[2 * g + 1] = (double)acc[g][0].hi.y + (double)acc[g][0].lo.y + (double)small[g][0].y;
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll

@@ -40,6 +40,7 @@
 using nfs::CGState;
 using nfs::kRedBlocks;
 using nfs::kRedThreads;
+using nfs::red_blocks;
 
 namespace {
 struct GraphEntry {
@@ -296,23 +297,6 @@ int ensure_scratch(nfs_ctx* c, size_t dlen) {
     c->hscratch_len = dlen;
   }
   return NFS_OK;
-}
-
-// Blocks per problem of the reductions over P problems' vectors of length N.
-// Never more blocks than the vector has threads' worth of elements (empty
-// blocks add exact zeros: a single problem's sums are the same at any larger
-// count); for batches, fewer, with at least 32 elements per thread, as long
-// as all problems together still have kRedBlocks blocks.  Each block ends in
-// FP64 block sums, which GB300 retires at about one warp instruction per 17
-// SM cycles: a full grid per problem over the short vectors of a batch of
-// small grids made those epilogues, not the data, the cost of a reduction.
-int red_blocks(long long N, int P) {
-  long long nb = std::min<long long>(kRedBlocks, (N + kRedThreads - 1) / kRedThreads);
-  if (P > 1) {
-    const long long per32 = (N + (long long)kRedThreads * 32 - 1) / ((long long)kRedThreads * 32);
-    nb = std::min(nb, std::max<long long>(per32, (kRedBlocks + P - 1) / P));
-  }
-  return (int)std::max<long long>(1, nb);
 }
 
 // Re(x_p^* y_p) for every problem, on the host: the launch and the copy of the
@@ -702,8 +686,7 @@ int exact_dots_start(nfs_ctx* c, int m, const double2* w, const int* d_active, s
   float2* whi = c->x32 ? c->x32 : reinterpret_cast<float2*>(c->Ap64);
   float2* wlo = c->x32 ? c->r32 : reinterpret_cast<float2*>(c->Ap64) + c->P * c->N;
   nfs::k_split_hi_lo<<<grid_blocks(c->P * c->N, 256), 256, 0, s>>>(w, whi, wlo, c->P * c->N);
-  // with many vectors one block per SM and pair: fewer FP64 ends of blocks
-  const int nb = m < 16 ? red_blocks(c->N, c->P) : std::min(red_blocks(c->N, c->P), (kRedBlocks / 2 + c->P - 1) / c->P);
+  const int nb = nfs::exact_dots_blocks(c->N, c->P, m);
   nfs::k_exact_dots<<<dim3((m + 1) / 2, nb, c->P), kRedThreads, 0, s>>>(c->MV32, c->MV32lo, vstride, m, whi, wlo, c->N,
                                                                         part, d_active);
   nfs::k_dots_finish<<<dim3(m, c->P), kRedThreads, 0, s>>>(part, m, nb, fin, d_active);
