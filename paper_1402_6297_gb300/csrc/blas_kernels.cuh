@@ -232,7 +232,8 @@ k_inner_start(const double2* __restrict__ r64, const double* __restrict__ s, flo
     r[i] = o;
     x[i] = zero;
     d[i] = zero;
-    acc.add(o.x * o.x + o.y * o.y + o.z * o.z + o.w * o.w);
+    acc.add(o.x * o.x + o.y * o.y);  // (one sum in FP32 for both elements would lose the smaller's low bits)
+    acc.add(o.z * o.z + o.w * o.w);
   }
   const float2 t = acc.block_total<kRedThreads>();
   if (threadIdx.x == 0) reinterpret_cast<float2*>(st[p].part_a)[blockIdx.x] = t;
