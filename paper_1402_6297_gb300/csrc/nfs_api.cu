@@ -130,8 +130,8 @@ struct nfs_ctx {
   size_t dY_len = 0;
   std::vector<GraphEntry> graphs;
   std::vector<GmresGraph> gm_graphs;  // NFSEP inner-solve step batches
-  // chunks that the last CG run took, per precision and refinement round
-  int cg_chunks[2][4] = {{1, 1, 1, 1}, {1, 1, 1, 1}};
+  // chunks that the last CG run from a zero start took, per refinement round
+  int cg_chunks[4] = {1, 1, 1, 1};
   long long bytes = 0;
   long long mv32 = 0, mv64 = 0;
   long long launches = 0;  // kernels this context has launched (graph nodes included)
@@ -408,18 +408,19 @@ int cg_chunk_graph(nfs_ctx* c, nfs::cplx<R>* x, nfs::cplx<R>* r, nfs::cplx<R>* p
 // CG from the state r = b - A x (already formed) for every problem, on the
 // work stream; tol2 the absolute thresholds on r^* r (+inf skips a problem).
 // Iterations run in graph-replayed chunks; every kernel returns at once after
-// its problem's device `done` flag is set.  The host first reads the flags after
-// as many chunks as the last run of the same kind took (the solves of an
-// eigensolve differ by an iteration or two), then after each: every round trip
-// leaves the GPU idle for about 20 us (8^3 complex128 eigensolves spent 9 of 86
-// ms on them).
+// its problem's device flags `stop` or `halt` are set (`done` is the host's, set
+// at the end of a chunk).  The host reads the state after every chunk, or, with
+// `last`, first after as many chunks as the last run of the same kind took (the
+// solves of an eigensolve differ by an iteration or two): every round trip leaves
+// the GPU idle for about 20 us (8^3 complex128 eigensolves spent 9 of 86 ms on
+// them).
 // r64 given: r is first formed from it (complex64: times the per-problem scale
 // at d_small + scale_off), and x set to zero.  relative: tol2 is a factor of the
 // starting r^* r.
 template <typename R>
 int cg_run(nfs_ctx* c, nfs::cplx<R>* x, nfs::cplx<R>* r, nfs::cplx<R>* p, const std::vector<double>& tol2, int maxit,
-           std::vector<int>& iters, std::vector<int>& status, const double2* r64 = nullptr, int scale_off = 0,
-           int round = 0, bool relative = false) {
+           std::vector<int>& iters, std::vector<int>& status, int* last, const double2* r64 = nullptr, int scale_off = 0,
+           bool relative = false) {
   using C = nfs::cplx<R>;
   cudaStream_t s = c->work;
   const double t0 = now_s();
@@ -441,8 +442,7 @@ int cg_run(nfs_ctx* c, nfs::cplx<R>* x, nfs::cplx<R>* r, nfs::cplx<R>* p, const 
   cudaGraphExec_t exec = nullptr;
   TRY(cg_chunk_graph<R>(c, x, r, p, &exec));
   const size_t head = offsetof(CGState, part_a);
-  int& last = c->cg_chunks[sizeof(R) == 4][std::min(round, 3)];
-  for (int ahead = std::max(1, std::min(last, maxit / kCgChunk)), ran = 0;; ahead = 1) {
+  for (int ahead = last ? std::max(1, std::min(*last, maxit / kCgChunk)) : 1, ran = 0;; ahead = 1) {
     for (int i = 0; i < ahead; ++i) CK(cudaGraphLaunch(exec, s));
     c->launches += (nfs::kProductKernels * kCgChunk + 1) * ahead;
     ran += ahead;
@@ -453,7 +453,7 @@ int cg_run(nfs_ctx* c, nfs::cplx<R>* x, nfs::cplx<R>* r, nfs::cplx<R>* p, const 
     if (all) {
       int it = 1;
       for (int q = 0; q < c->P; ++q) it = std::max(it, c->st_host[q].it);
-      last = std::min(ran, (it + kCgChunk - 1) / kCgChunk);
+      if (last) *last = std::min(ran, (it + kCgChunk - 1) / kCgChunk);
       break;
     }
     // (a chunk ends a problem or takes kCgChunk of its maxit steps)
@@ -479,25 +479,15 @@ int sub64(nfs_ctx* c, cudaStream_t s, const double2* a, const double2* b, double
   return NFS_OK;
 }
 
-// Whether every entry of the P vectors x is zero (mixed solves: without a start,
-// as the binding's solve without one, the first residual is b itself; its
-// product would cost as much as 20 CG iterations, 1.6 ms at 96^3).
-int is_zero(nfs_ctx* c, cudaStream_t s, const double2* x, bool& zero) {
-  const long long tot = c->P * c->N;
-  TRY(put_flags(c, s, c->P, std::vector<int>(1, 0)));
-  nfs::k_mark_nonzero<<<grid_blocks(tot, 256), 256, 0, s>>>(x, tot, c->d_flags + c->P);
-  CK(cudaGetLastError());
-  c->launches += 1;
-  CK(cudaMemcpyAsync(c->h_flags + c->P, c->d_flags + c->P, sizeof(int), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
-  zero = c->h_flags[c->P] == 0;
-  return NFS_OK;
-}
-
 // Solve A_r x_p = b_p for every problem p with active[p] (b, x: P x N, on the
 // work stream).  FP64 contexts run complex128 CG; MIXED contexts run complex64
-// CG inside FP64 iterative refinement (the residual r = b - A_r x with the
-// complex128 product, scaled to unit norm, demoted; x += |r| d).
+// CG inside FP64 iterative refinement (the residual r = b - A_r x, in complex128
+// for a given start and by the double-single product after each correction,
+// scaled to unit norm, demoted; x += |r| d).  A given start may be zero (what the
+// binding's solve without one passes): it is recognised on the device and needs
+// no product (1.6 ms at 96^3, 20 iterations' time).  Solves from zero differ by an
+// iteration or two and queue their CG steps ahead (cg_run); how many a given start
+// takes is not known.
 struct SolveOut {
   std::vector<int> iters, refines, status;
   std::vector<double> relres;
@@ -517,7 +507,7 @@ int solve(nfs_ctx* c, const double2* b, double2* x, bool x_zero, const std::vect
     std::vector<double> tol2(P);
     for (int q = 0; q < P; ++q) tol2[q] = active[q] ? tol * tol : INFINITY;
     std::vector<int> it, st;
-    TRY(cg_run<double>(c, x, c->r64, c->p64, tol2, c->opt.cg_maxit, it, st, b, 0, 0, true));
+    TRY(cg_run<double>(c, x, c->r64, c->p64, tol2, c->opt.cg_maxit, it, st, &c->cg_chunks[0], b, 0, true));
     for (int q = 0; q < P; ++q) {
       const double bb = c->st_host[q].rr0;
       if (!active[q] || !(bb > 0.0)) continue;
@@ -528,7 +518,18 @@ int solve(nfs_ctx* c, const double2* b, double2* x, bool x_zero, const std::vect
     return NFS_OK;
   }
   std::vector<double> bb;
-  TRY(dots_re(c, s, b, b, bb));
+  TRY(dots_re_start(c, s, b, b, 0));
+  if (!x_zero) {
+    TRY(put_flags(c, s, P, std::vector<int>(1, 0)));
+    nfs::k_mark_nonzero<<<grid_blocks(tot, 256), 256, 0, s>>>(x, tot, c->d_flags + P);
+    CK(cudaGetLastError());
+    c->launches += 1;
+    CK(cudaMemcpyAsync(c->h_flags + P, c->d_flags + P, sizeof(int), cudaMemcpyDeviceToHost, s));
+  }
+  CK(cudaStreamSynchronize(s));
+  dots_re_finish(c, 0, bb);
+  x_zero = x_zero || c->h_flags[P] == 0;
+  int* const chunks = x_zero ? c->cg_chunks : nullptr;
   if (x_zero) {
     CK(cudaMemsetAsync(x, 0, tot * sizeof(double2), s));
     CK(cudaMemcpyAsync(c->r64, b, tot * sizeof(double2), cudaMemcpyDeviceToDevice, s));
@@ -544,7 +545,7 @@ int solve(nfs_ctx* c, const double2* b, double2* x, bool x_zero, const std::vect
     std::vector<double> tol2(P);
     for (int q = 0; q < P; ++q) tol2[q] = need[q] ? tol * tol * bb[q] : INFINITY;
     std::vector<int> it, st;
-    TRY(cg_run<double>(c, x, c->r64, c->p64, tol2, c->opt.cg_maxit, it, st));
+    TRY(cg_run<double>(c, x, c->r64, c->p64, tol2, c->opt.cg_maxit, it, st, chunks));
     for (int q = 0; q < P; ++q) {
       if (!need[q]) continue;
       so.iters[q] = it[q];
@@ -597,7 +598,8 @@ int solve(nfs_ctx* c, const double2* b, double2* x, bool x_zero, const std::vect
     if (!any) break;
     TRY(put_small(c, s, P, inv));
     std::vector<int> it, st;
-    TRY(cg_run<float>(c, c->x32, c->r32, c->p32, itol2, c->opt.cg_maxit, it, st, c->r64, P, round));
+    TRY(cg_run<float>(c, c->x32, c->r32, c->p32, itol2, c->opt.cg_maxit, it, st,
+                      chunks ? &chunks[std::min(round, 3)] : nullptr, c->r64, P));
     TRY(put_small(c, s, 2 * P, nrm));
     nfs::k_axpy_promote<<<nb, 256, 0, s>>>(x, c->d_small + 2 * P, c->x32, c->N, tot);
     CK(cudaGetLastError());
@@ -1922,11 +1924,9 @@ extern "C" int nfs_cg_solve(nfs_ctx* c, const void* b, void* x, nfs_solve_info* 
   const size_t bytes = (size_t)c->P * c->N * sizeof(double2);
   CK(cudaMemcpyAsync(c->t64b, b, bytes, cudaMemcpyDeviceToDevice, c->work));
   CK(cudaMemcpyAsync(c->t64, x, bytes, cudaMemcpyDeviceToDevice, c->work));
-  bool x_zero = false;
-  if (c->opt.precision == NFS_PREC_MIXED) TRY(is_zero(c, c->work, c->t64, x_zero));
   SolveOut so;
   std::vector<int> active(c->P, 1);
-  TRY(solve(c, c->t64b, c->t64, x_zero, active, so));
+  TRY(solve(c, c->t64b, c->t64, false, active, so));
   CK(cudaMemcpyAsync(x, c->t64, bytes, cudaMemcpyDeviceToDevice, c->work));
   CK(cudaStreamSynchronize(c->work));
   if (info) {
