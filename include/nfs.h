@@ -130,8 +130,9 @@ typedef struct {
                               * graph nodes included); in a batch, those of the
                               * problem's whole class                                */
   /* host wall-clock split of the call (the class's, in a batch): total; inside
-   * the CG iteration loops; the rest of the linear solves (residual
-   * refinement); host projected eigensolves; then the Lanczos phases. */
+   * the CG iteration loops (with the few vector kernels queued just before one);
+   * the rest of the linear solves (residual refinement); host projected
+   * eigensolves; then the Lanczos phases. */
   double seconds_total;
   double seconds_cg;
   double seconds_refine;

@@ -135,7 +135,7 @@ struct nfs_ctx {
   long long bytes = 0;
   long long mv32 = 0, mv64 = 0;
   long long launches = 0;  // kernels this context has launched (graph nodes included)
-  double sec_cg = 0.0;     // host wall time inside the CG iteration loops
+  double sec_cg = 0.0;     // host wall time of the CG runs (with the few kernels queued just before one)
   double sec_solve = 0.0;  // ... inside whole solves (CG + refinement residuals)
   double sec_ritz = 0.0;   // ... in the host projected eigensolves
   double sec_recur = 0.0, sec_orth = 0.0, sec_vec = 0.0;  // Lanczos phases
@@ -1309,6 +1309,7 @@ int eigs_core(nfs_ctx* c, int nev, double* omega, double2* Y, nfs_eigs_info* inf
     }
     TRY(refresh_products(c, keep + 1, active));
     TRY(refresh_shadows(c, 0, keep + 1));
+    CK(cudaStreamSynchronize(s));  // (not the next solve's time)
     jstart = keep;
     local_lo = 0;
     ++restarts;
