@@ -1182,6 +1182,12 @@ int eigs_core(nfs_ctx* c, int nev, double* omega, double2* Y, nfs_eigs_info* inf
       // very large one (a coupling after a restart) takes a second pass.
       if (local_lo > 0) {
         std::vector<int> reorth(P, 0);
+        // the vector that a thick restart goes on from, whatever it has lost: the
+        // arrow matrix couples it to the kept Ritz vectors by beta alone, and what
+        // is left of a loss near orth_tol comes back in their residuals (96^3
+        // cylinders, four pairs, one restart: 3e-10 to 1.5e-9 where the loss had
+        // been 9e-11 and was left, 2e-11 where it was removed)
+        const bool last = j == m - 1;
         for (int pass = 0; pass < 3; ++pass) {
           if (pass > 0) TRY(exact_dots_start(c, local_lo, w, d_active, off_host_exact(c)));
           CK(cudaStreamSynchronize(s));
@@ -1195,7 +1201,7 @@ int eigs_core(nfs_ctx* c, int nev, double* omega, double2* Y, nfs_eigs_info* inf
               loss = std::max(loss, std::hypot(d[(size_t)p * 2 * local_lo + 2 * i], d[(size_t)p * 2 * local_lo + 2 * i + 1]));
             loss /= std::sqrt(std::max(bb[p], 1e-300));
             if (pass == 0) loss_first[p] = loss;
-            reorth[p] = pass == 0 ? loss > c->opt.orth_tol : loss > 1e-3 * c->opt.orth_tol + 1e-13;
+            reorth[p] = pass == 0 ? loss > c->opt.orth_tol || last : loss > 1e-3 * c->opt.orth_tol + 1e-13;
             any_re = any_re || reorth[p];
             big = big || (reorth[p] && loss > 1e-3);
             big_loss = big_loss || (reorth[p] && loss > kShadowMaxLoss);
