@@ -68,26 +68,19 @@ __device__ __forceinline__ double block_sum(double v) {
   return r;
 }
 
-__device__ __forceinline__ double sum_partials(const double* part, int count = kRedBlocks) {
-  // one block of kRedThreads threads sums `count` partials in fixed order
-  double v = 0.0;
-  for (int i = threadIdx.x; i < count; i += kRedThreads) v += part[i];
-  return block_sum<kRedThreads>(v);
-}
-
 // part[p * pstride + b] = block b's share of Re(conj(x_p) y_p); grid (blocks, P).
-template <typename C>
 __global__ void __launch_bounds__(kRedThreads)
-k_dot_re(const C* __restrict__ x, const C* __restrict__ y, long long N, double* __restrict__ part, long long pstride) {
+k_dot_re(const double2* __restrict__ x, const double2* __restrict__ y, long long N, double* __restrict__ part,
+         long long pstride) {
   const int p = blockIdx.y;
   x += (long long)p * N;
   y += (long long)p * N;
-  Acc<C> acc;
+  double acc = 0.0;
   for (long long i = (long long)blockIdx.x * kRedThreads + threadIdx.x; i < N; i += (long long)gridDim.x * kRedThreads) {
-    const C a = x[i], b = y[i];
-    acc.add(a.x * b.x + a.y * b.y);
+    const double2 a = x[i], b = y[i];
+    acc += a.x * b.x + a.y * b.y;
   }
-  const double s = block_sum<kRedThreads>(acc.total());
+  const double s = block_sum<kRedThreads>(acc);
   if (threadIdx.x == 0) part[(long long)p * pstride + blockIdx.x] = s;
 }
 

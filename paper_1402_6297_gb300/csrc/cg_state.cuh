@@ -42,31 +42,6 @@ struct CGState {
 constexpr long long kStateDoubles = sizeof(CGState) / sizeof(double);
 static_assert(sizeof(CGState) % sizeof(double) == 0, "CGState must be a whole number of doubles");
 
-// Partial sums of complex products: single-precision data accumulate in FP32
-// over short runs that are folded into FP64 (FP64 arithmetic is scarce on
-// this GPU); double-precision data accumulate in FP64.
-template <typename C>
-struct Acc {
-  double d = 0.0;
-  __device__ __forceinline__ void add(double v) { d += v; }
-  __device__ __forceinline__ double total() const { return d; }
-};
-template <>
-struct Acc<float2> {
-  double d = 0.0;
-  float f = 0.f;
-  int k = 0;
-  __device__ __forceinline__ void add(float v) {
-    f += v;
-    if (++k == 16) {
-      d += (double)f;
-      f = 0.f;
-      k = 0;
-    }
-  }
-  __device__ __forceinline__ double total() const { return d + (double)f; }
-};
-
 // Per-thread accumulator and block sum of the CG reductions (the partials
 // of p^* A p and r^* r).  Complex64 runs accumulate in double-single
 // arithmetic on the FP32 units (hi + lo floats, TwoSum: ~1e-14 of the sum of

@@ -76,8 +76,9 @@ struct nfs_ctx {
   // tables (per problem: stride nl) and twiddles (shared)
   double2* lam64 = nullptr;
   float2* lam32 = nullptr;
-  double2* tw64[3] = {nullptr, nullptr, nullptr};
-  float2* tw32[3] = {nullptr, nullptr, nullptr};
+  // twiddles: [0] the plane's edge, [1] z
+  double2* tw64[2] = {nullptr, nullptr};
+  float2* tw32[2] = {nullptr, nullptr};
   // material, per problem (stride mat_len): inv_phi [3n] | gam [3n or n] | inv_mu [3n]
   double* mat64 = nullptr;
   float4* pmat = nullptr;  // complex64 order of the material (mixed contexts and products; stride 3n / 2)
@@ -100,7 +101,7 @@ struct nfs_ctx {
   // double-single copies of the tables, material and basis (mixed contexts:
   // the refinement residual products)
   nfs::dfc* lamdf = nullptr;
-  nfs::dfc* twdf[3] = {nullptr, nullptr, nullptr};
+  nfs::dfc* twdf[2] = {nullptr, nullptr};
   nfs::df* matdf = nullptr;
   nfs::dfc* basisdf = nullptr;
   // workspaces, per problem
@@ -223,7 +224,7 @@ template <>
 nfs::MatvecArgs<double> margs<double>(nfs_ctx* c, const double2* u, double2* Au, const int* skip) {
   nfs::MatvecArgs<double> a{};
   a.u = u; a.Au = Au; a.fld = c->fld; a.lam = c->lam64;
-  a.tw1 = c->tw64[0]; a.tw3 = c->tw64[2];
+  a.tw1 = c->tw64[0]; a.tw3 = c->tw64[1];
   a.inv_phi = c->mat64; a.gam = c->mat64 + 3 * c->n; a.inv_mu = c->has_mu ? c->mat64 + 3 * c->n + c->gam_len : nullptr;
   a.kind = c->kind; a.ax_a = c->ax_a; a.ax_b = c->ax_b;
   a.n1 = c->n1; a.n3 = c->n3; a.alpha = c->opt.alpha; a.beta = c->opt.beta;
@@ -239,7 +240,7 @@ template <>
 nfs::MatvecArgs<float> margs<float>(nfs_ctx* c, const float2* u, float2* Au, const int* skip) {
   nfs::MatvecArgs<float> a{};
   a.u = u; a.Au = Au; a.fld = c->fld; a.lam = c->lam32;
-  a.tw1 = c->tw32[0]; a.tw3 = c->tw32[2];
+  a.tw1 = c->tw32[0]; a.tw3 = c->tw32[1];
   a.pmat = c->pmat; a.pmu = c->pmu;
   a.kind = c->kind; a.ax_a = c->ax_a; a.ax_b = c->ax_b;
   a.n1 = c->n1; a.n3 = c->n3; a.alpha = (float)c->opt.alpha; a.beta = (float)c->opt.beta;
@@ -254,7 +255,7 @@ template <>
 nfs::MatvecArgs<nfs::df> margs<nfs::df>(nfs_ctx* c, const double2* u, double2* Au, const int* skip) {
   nfs::MatvecArgs<nfs::df> a{};
   a.u = u; a.Au = Au; a.fld = c->fld; a.lam = c->lamdf;
-  a.tw1 = c->twdf[0]; a.tw3 = c->twdf[2];
+  a.tw1 = c->twdf[0]; a.tw3 = c->twdf[1];
   a.inv_phi = c->matdf; a.gam = c->matdf + 3 * c->n; a.inv_mu = c->has_mu ? c->matdf + 3 * c->n + c->gam_len : nullptr;
   a.kind = c->kind; a.ax_a = c->ax_a; a.ax_b = c->ax_b;
   a.n1 = c->n1; a.n3 = c->n3; a.alpha = nfs::df(c->opt.alpha); a.beta = nfs::df(c->opt.beta);
@@ -301,10 +302,9 @@ int ensure_scratch(nfs_ctx* c, size_t dlen) {
 
 // Re(x_p^* y_p) for every problem, on the host: the launch and the copy of the
 // partials to hscratch + off, and their sums once the stream has got there
-template <typename C>
-int dots_re_start(nfs_ctx* c, cudaStream_t s, const C* x, const C* y, size_t off) {
+int dots_re_start(nfs_ctx* c, cudaStream_t s, const double2* x, const double2* y, size_t off) {
   const int nb = red_blocks(c->N, c->P);
-  nfs::k_dot_re<C><<<dim3(nb, c->P), kRedThreads, 0, s>>>(x, y, c->N, c->dscratch, nb);
+  nfs::k_dot_re<<<dim3(nb, c->P), kRedThreads, 0, s>>>(x, y, c->N, c->dscratch, nb);
   CK(cudaGetLastError());
   c->launches += 1;
   CK(cudaMemcpyAsync(c->hscratch + off, c->dscratch, (size_t)nb * c->P * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -319,8 +319,7 @@ void dots_re_finish(const nfs_ctx* c, size_t off, std::vector<double>& out) {
     out[p] = t;
   }
 }
-template <typename C>
-int dots_re(nfs_ctx* c, cudaStream_t s, const C* x, const C* y, std::vector<double>& out) {
+int dots_re(nfs_ctx* c, cudaStream_t s, const double2* x, const double2* y, std::vector<double>& out) {
   TRY(dots_re_start(c, s, x, y, 0));
   CK(cudaStreamSynchronize(s));
   dots_re_finish(c, 0, out);
@@ -432,7 +431,7 @@ int cg_run(nfs_ctx* c, nfs::cplx<R>* x, nfs::cplx<R>* r, nfs::cplx<R>* p, const 
     nfs::k_solve_start<<<dim3(nb, c->P), kRedThreads, 0, s>>>(r64, r, x, p, c->N, c->st);
   } else {
     CK(cudaMemsetAsync(p, 0, c->P * c->N * sizeof(C), s));
-    nfs::k_dot_re<C><<<dim3(nb, c->P), kRedThreads, 0, s>>>(r, r, c->N, c->st->part_a, nfs::kStateDoubles);
+    nfs::k_dot_re<<<dim3(nb, c->P), kRedThreads, 0, s>>>(r, r, c->N, c->st->part_a, nfs::kStateDoubles);
   }
   TRY(put_small(c, s, 0, tol2));
   nfs::k_cg_init<R><<<c->P, kRedThreads, 0, s>>>(c->st, c->d_small, relative, maxit, nb,
@@ -1497,8 +1496,8 @@ void free_ctx(nfs_ctx* c) {
   if (!c) return;
   for (GraphEntry& g : c->graphs) cudaGraphExecDestroy(g.exec);
   for (GmresGraph& g : c->gm_graphs) cudaGraphExecDestroy(g.exec);
-  void* ptrs[] = {c->lam64, c->lam32, c->tw64[0], c->tw64[1], c->tw64[2], c->tw32[0], c->tw32[1], c->tw32[2],
-                  c->mat64, c->pmat, c->pmu, c->basis64, c->bloch64, c->lamdf, c->twdf[0], c->twdf[1], c->twdf[2], c->matdf,
+  void* ptrs[] = {c->lam64, c->lam32, c->tw64[0], c->tw64[1], c->tw32[0], c->tw32[1],
+                  c->mat64, c->pmat, c->pmu, c->basis64, c->bloch64, c->lamdf, c->twdf[0], c->twdf[1], c->matdf,
                   c->basisdf, c->fld, c->x64, c->r64, c->p64, c->Ap64, c->t64, c->t64b, c->x32, c->r32,
                   c->p32, c->Ap32, c->st, c->d_small, c->d_flags, c->dscratch, c->V, c->MV, c->V32, c->MV32,
                   c->MV32lo, c->dY, c->binv64, c->root64, c->zv, c->gv, c->zY};
@@ -1709,8 +1708,8 @@ int setup_class(nfs_ctx** out, int P, const int grid[3], const nfs_material* con
     CKC(cudaMemcpy(c->lam32, lam32.data(), lam32.size() * sizeof(float2), cudaMemcpyHostToDevice));
   }
   const int nn[3] = {n1, n2, n3};
-  for (int l = 0; l < 3; ++l) {
-    const int m = nn[l];
+  for (int l = 0; l < 2; ++l) {
+    const int m = l == 0 ? n1 : n3;
     std::vector<double2> t(m);
     std::vector<float2> t32(m);
     for (int i = 0; i < m; ++i) {
@@ -1753,10 +1752,11 @@ int setup_class(nfs_ctx** out, int P, const int grid[3], const nfs_material* con
     TRYC(dalloc(c, &c->lamdf, (size_t)P * nl));
     CKC(nfs::double_to_df(reinterpret_cast<const double*>(c->lam64), reinterpret_cast<nfs::df*>(c->lamdf),
                           2LL * P * nl, 0));
-    for (int l = 0; l < 3; ++l) {
-      TRYC(dalloc(c, &c->twdf[l], nn[l]));
+    for (int l = 0; l < 2; ++l) {
+      const int m = l == 0 ? n1 : n3;
+      TRYC(dalloc(c, &c->twdf[l], m));
       CKC(nfs::double_to_df(reinterpret_cast<const double*>(c->tw64[l]), reinterpret_cast<nfs::df*>(c->twdf[l]),
-                            2LL * nn[l], 0));
+                            2LL * m, 0));
     }
     TRYC(dalloc(c, &c->matdf, (size_t)P * c->mat_len));
     CKC(nfs::double_to_df(c->mat64, c->matdf, (long long)P * c->mat_len, 0));
@@ -2027,7 +2027,7 @@ extern "C" int nfs_eig_grad(nfs_ctx* c, int m, const double* weights, const void
     cudaError_t e = nfs::matvec_launch_mask<double>(a, 1);
     if (e != cudaSuccess) return cuda_fail(e, "grad rows");
     nfs::GradArgs g{};
-    g.fld = c->fld; g.tw1 = c->tw64[0]; g.tw3 = c->tw64[2];
+    g.fld = c->fld; g.tw1 = c->tw64[0]; g.tw3 = c->tw64[1];
     g.inv_phi = c->mat64; g.gam = c->mat64 + 3 * n;
     g.kind = c->kind; g.ax_a = c->ax_a; g.ax_b = c->ax_b;
     g.n1 = c->n1; g.n3 = c->n3;
@@ -2057,7 +2057,7 @@ extern "C" int nfs_eig_fields(nfs_ctx* c, int m, const void* Yv, void* Xv) {
     cudaError_t e = nfs::matvec_launch_mask<double>(a, 1);
     if (e != cudaSuccess) return cuda_fail(e, "fields rows");
     nfs::FieldsArgs f{};
-    f.fld = c->fld; f.tw1 = c->tw64[0]; f.tw3 = c->tw64[2]; f.bloch = c->bloch64;
+    f.fld = c->fld; f.tw1 = c->tw64[0]; f.tw3 = c->tw64[1]; f.bloch = c->bloch64;
     f.inv_phi = a.inv_phi; f.gam = a.gam; f.inv_mu = a.inv_mu;
     f.kind = c->kind; f.ax_a = c->ax_a; f.ax_b = c->ax_b;
     f.n1 = c->n1; f.n3 = c->n3;
@@ -2118,7 +2118,7 @@ int nfsep_apply(nfs_ctx* c, cudaStream_t s, const double2* y, double2* out, nfs:
   a.kr.root = c->root64;
   cudaError_t e = nfs::matvec_launch_mask<double>(a, 1);
   if (e != cudaSuccess) return cuda_fail(e, "nfsep rows");
-  e = nfs::nfsep_columns(c->fld, c->binv64, c->tw64[0], c->tw64[2], c->n1, c->n3, s);
+  e = nfs::nfsep_columns(c->fld, c->binv64, c->tw64[0], c->tw64[1], c->n1, c->n3, s);
   if (e != cudaSuccess) return cuda_fail(e, "nfsep columns");
   e = nfs::matvec_launch_mask<double>(a, 4);
   if (e != cudaSuccess) return cuda_fail(e, "nfsep rows out");
@@ -2189,7 +2189,7 @@ struct DevBasis : virtual nfs::host::KrylovOps {
     return NFS_OK;
   }
   int norm(double& nrm) override {
-    nfs::k_dot_re<double2><<<dim3(kRedBlocks, 1), kRedThreads, 0, s>>>(w, w, N, c->dscratch, kRedBlocks);
+    nfs::k_dot_re<<<dim3(kRedBlocks, 1), kRedThreads, 0, s>>>(w, w, N, c->dscratch, kRedBlocks);
     CK(cudaGetLastError());
     c->launches += 1;
     CK(cudaMemcpyAsync(c->hscratch, c->dscratch, kRedBlocks * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -2618,7 +2618,7 @@ extern "C" int nfs_nfsep_fields(nfs_ctx* c, int m, const void* Yv, void* Xv) {
     a.kr.root = c->root64;
     cudaError_t e = nfs::matvec_launch_mask<double>(a, 1);
     if (e != cudaSuccess) return cuda_fail(e, "nfsep fields rows");
-    e = nfs::nfsep_fields(c->fld, c->binv64, c->tw64[0], c->tw64[2], c->bloch64, c->n1, c->n3,
+    e = nfs::nfsep_fields(c->fld, c->binv64, c->tw64[0], c->tw64[1], c->bloch64, c->n1, c->n3,
                           (double2*)Xv + (long long)j * 6 * n, c->stream);
     if (e != cudaSuccess) return cuda_fail(e, "nfsep fields");
     c->launches += 2;
