@@ -858,6 +858,7 @@ k_rows_out(const typename ElemOf<R>::E* fld, vecc<R>* Au, const cplx<R>* __restr
   constexpr int LINES = 3 * N1;
   constexpr int NV = N1 * N;
   static_assert(3 * N1 * (N / X) <= kMaxPartials, "one partial of p^* A p per CTA of k_columns");
+  static_assert(N2 * NF * 128 <= kMaxPartials, "one partial of r^* r per CTA of this kernel, up to 128 of z");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   E* buf = reinterpret_cast<E*>(smem_raw);
   E* tw = buf + LINES * PITCH;
