@@ -217,18 +217,20 @@ def profiled_traffic(pass_index):
 
 
 def cg_iteration_roofline(n, product_bytes, info, hbm):
+    # of the product's vectors p is its u, and A_r p is not stored; further r is
+    # read and p written at the start, x, r, p read and x, r written at the end
     vec = 4 * n * 8
-    b = product_bytes + 2 * vec + 6 * vec
+    b = product_bytes - vec + 2 * vec + 5 * vec
     us = 1e6 * info.seconds_cg / max(int(info.cg_iterations), 1)
     gbps = b / (us * 1e-6) / 1e9
     return {"bytes": b, "us": us, "GBps": gbps, "frac": gbps / hbm}
 
 
 def bytes_per_pass(n, csize, kind):
-    """Algorithmic HBM bytes of each pass of one A_r product (3-pass model):
-    pass 1 reads u (4n) and writes six fields (6n); pass 2 reads and writes the
-    six fields and reads the material (1/Phi per component and gamma); pass 3
-    reads six fields and writes A_r u (4n)."""
+    """Algorithmic HBM bytes of each kernel of one A_r product: k_rows_in reads u
+    (4n) and writes six fields (6n); k_columns reads and writes the six fields
+    and reads the material (1/Phi per component and gamma); k_rows_out reads six
+    fields and writes A_r u (4n)."""
     rsize = csize // 2
     mat_reals = 6 if kind == "chiral" else 4
     return [10 * n * csize, 12 * n * csize + mat_reals * n * rsize, 10 * n * csize]
@@ -585,8 +587,8 @@ def fields_leg(ctx, omega, Y, n, torch, hbm):
     res = ctx.gep_residual(omega, X)
     res_ms = 1000.0 * (time.perf_counter() - t0)
     per_vec = statistics.median(ms) / m
-    # algorithmic bytes per vector (complex128): pass 1 reads y (4n) and
-    # writes 6n fields; the z pass reads them with the material (3 reals of
+    # algorithmic bytes per vector (complex128): k_rows_in reads y (4n) and
+    # writes 6n fields; k_columns reads them with the material (3 reals of
     # 1/Phi, one gamma) and writes X (6n)
     fbytes = n * (4 * 16 + 6 * 16 + 6 * 16 + 4 * 8 + 6 * 16)
     return {"vectors": m, "fields_ms_per_vector": per_vec,
@@ -815,10 +817,10 @@ def run_ours(args):
         "precision": "mixed: complex64 CG, double-single refinement residuals, FP64 Lanczos",
         "matvecs_per_s": {"c64": 1000.0 / mv64_ms, "c128": 1000.0 / mv128_ms},
         "cg_iters_per_s": cg_its / (statistics.mean(step_ms) / 1000.0),
-        # one complex64 CG iteration, algorithmic bytes (64 n s + material):
-        # the product (3-pass bytes) + pass 1 reading r and writing p + the
-        # x/r step reading x, r, p, A p and writing x, r (vectors of 4n
-        # complex64; the step runs fused into pass 3, which never stores A p)
+        # one complex64 CG iteration, algorithmic bytes (56 n s + material):
+        # the product's three kernels without the store of A_r p, + reading r
+        # and writing p, + reading x, r, p and writing x, r (vectors of 4n
+        # complex64)
         "cg_iteration": cg_iteration_roofline(n, sum(bpp), info, hbm),
         "eigensolve": {"lanczos_steps": info.lanczos_steps, "restarts": info.restarts,
                        "cg_iterations": int(cg_its), "matvecs_c64": int(info.matvecs_c64),

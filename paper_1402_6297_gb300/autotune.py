@@ -78,7 +78,7 @@ for _ in range({reps}):
     e0.record(st); ctx.matvec(u32, out); e1.record(st)
     torch.cuda.synchronize()
     ts.append(e0.elapsed_time(e1))
-# the CG-fused forms of the passes (direction update, curvature partials):
+# the CG forms of the kernels (direction update, curvature partials):
 # one mixed-precision solve, checked by its true complex128 residual
 b = torch.from_numpy(wl.random_complex(4 * n, 3)).cuda()
 x, info = ctx.cg_solve(b)

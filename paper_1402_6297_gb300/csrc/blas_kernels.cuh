@@ -5,8 +5,8 @@
 //
 // Reductions are deterministic: a grid of blocks per problem fixed by the
 // vector length and the problem count (at most kRedBlocks) writes one
-// partial per block, and a one-block kernel sums the partials in a fixed
-// order.
+// partial per block, and a one-block kernel, the host or (in CG) every block of
+// the next kernel sums the partials in a fixed order.
 #pragma once
 #include <algorithm>
 #include <cstdint>
@@ -181,7 +181,7 @@ __global__ void k_add(const double* __restrict__ a, const double* __restrict__ b
 }
 
 // Refinement residual per problem p (skip64, skip32: the masks of the two
-// products just launched): r_p = b_p - Ap64_p where the complex128 product ran
+// products just launched): r_p = b_p - Ap64_p where the double-single product ran
 // (!skip64[p]), else r_p -= s_p Ap32_p where the complex64 product of the
 // correction ran (!skip32[p]), else r_p is left.  Grid-stride over P x N.
 __global__ void k_refine_residual(double2* __restrict__ r, const double2* __restrict__ b,

@@ -21,7 +21,8 @@ constexpr int kMaxPartials = 3072;  // >= kRedBlocks and the CTAs of one problem
 // kernels need.  Flags are written only by kernels that do not read them, so
 // every CTA of a launch sees the same value:
 //   stop   k_rows_in writes, k_columns and k_rows_out read: nothing left to do
-//   halt   k_rows_out writes, k_rows_in reads: stop was set, or a breakdown
+//   halt   k_rows_out writes, k_rows_in and k_cg_check read: stop was set, or a
+//          breakdown
 // `partial` values are doubles (complex128) or (hi, lo) float pairs
 // (complex64), eight bytes either way.
 struct CGState {

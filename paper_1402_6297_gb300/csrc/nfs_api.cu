@@ -347,7 +347,7 @@ int put_flags(nfs_ctx* c, cudaStream_t s, int off, const std::vector<int>& v) {
 
 // --- CG ---------------------------------------------------------------------
 
-// CG iterations per captured chunk (even); the host reads the done flags
+// CG iterations per captured chunk; the host reads the done flags
 // between chunks, and iterations launched after convergence return at once
 #ifndef NFS_CG_CHUNK
 #define NFS_CG_CHUNK 8
@@ -555,8 +555,8 @@ int solve(nfs_ctx* c, const double2* b, double2* x, bool x_zero, const std::vect
   }
   // mixed precision.  Round k: d = A32^{-1} (r_k / |r_k|) by complex64 CG,
   // x += |r_k| d, then the next residual.  While the correction is of the
-  // size of x (|r_k| large) the residual needs the complex128 product,
-  // r = b - A x.  Once |r_k| <= kCheapRefine * tol * |b| it is updated as
+  // size of x (|r_k| large) the residual needs an accurate product, the
+  // double-single one, r = b - A x.  Once |r_k| <= kCheapRefine * tol * |b| it is updated as
   // r -= |r_k| A32 d with the complex64 product of the correction: that
   // product's relative error (~5e-7) then moves r by at most ~1% of the
   // tolerance.  The inner tolerance is inner_tol, or looser where the
@@ -603,7 +603,7 @@ int solve(nfs_ctx* c, const double2* b, double2* x, bool x_zero, const std::vect
     nfs::k_axpy_promote<<<nb, 256, 0, s>>>(x, c->d_small + 2 * P, c->x32, c->N, tot);
     CK(cudaGetLastError());
     c->launches += 1;
-    // next residual: complex128 product of x, or complex64 product of d
+    // next residual: double-single product of x, or complex64 product of d
     TRY(put_flags(c, s, 2 * P, skip64));
     TRY(put_flags(c, s, 3 * P, skip32));
     if (any64) TRY(matvec<nfs::df>(c, s, x, c->Ap64, c->d_flags + 2 * P, 1));
@@ -2335,7 +2335,8 @@ int gmres_steps(nfs_ctx* c, cudaStream_t s, double2 sigma, double2* V, double2* 
 // vectors, and w as workspace), the least-squares problem on the host
 // (GivensLS) from the Hessenberg columns read once per batch of kGmresBatch
 // steps.  Steps enqueued after the one that converged are wasted work (the
-// cycle ends at the converged column); they are counted as iterations.
+// cycle ends at the converged column): those of its own batch are counted as
+// iterations, the batch behind it is thrown away and not counted.
 int dev_gmres(nfs_ctx* c, const double2* b, double2* x, double2 sigma, double2* V, double2* w, int m, double tol,
               double bnorm, int maxit, nfs::host::GmresResult& out) {
   out = nfs::host::GmresResult{};

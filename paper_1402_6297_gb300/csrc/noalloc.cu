@@ -28,7 +28,7 @@ constexpr int kMaxEdge = 128;
 constexpr int kMaxDevices = 64;
 
 // Layout of the scratch array (offsets in bytes, each 256-aligned):
-//   fields   6 n complex128         (the three passes' workspace)
+//   fields   6 n complex128         (the three kernels' workspace)
 //   inv_phi  3 n double             (1 / Phi per component)
 //   gamma    3 n double             (chiral: per component; pseudochiral: first n)
 //   lambda   3 * kMaxEdge complex128 (Lambda_1 | Lambda_2 | Lambda_3)

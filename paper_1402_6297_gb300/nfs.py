@@ -370,7 +370,7 @@ class Context:
         return out
 
     def matvec_passes(self, mask, u, out):
-        """Only the selected passes of the product (timing aid; see nfs.h)."""
+        """Only the selected kernels of the product (timing aid; see nfs.h)."""
         torch = self._torch
         dt = u.dtype
         code = C128 if dt == torch.complex128 else C64
