@@ -97,9 +97,7 @@ struct MatView {
 // depend_begin() lets the next kernel of the stream start, depend_wait() waits
 // for the one before to end with its writes visible.  Every CTA waits before it
 // touches anything but constant tables, and before it returns: a kernel that
-// ended earlier would let its successor run ahead of its predecessor.  (The
-// Gram-Schmidt kernels also read older basis vectors ahead of the wait, see
-// load_l2.)
+// ended earlier would let its successor run ahead of its predecessor.
 //
 // Such a kernel is alive while its predecessor writes, so what any kernel on the
 // stream writes is read by plain loads from plain pointers: __ldg and const

@@ -116,18 +116,6 @@ constexpr int kGsTile = 128;      // elements of w that a block of k_gs_dots hol
 constexpr int kGsMaxChunks = 64;
 constexpr int kGsPerWarp = 2;     // vectors per warp (4: the FP64 work of a block takes 3 us instead of 1.9)
 
-// The kernels fetch what they need of the older basis vectors before they wait
-// for the kernel before them.  All but the newest vector were written by kernels
-// that had ended when the predecessor passed its own wait, which it did before it
-// let this one start; their writes are in the L2 by then, and the load takes
-// them from there (a line of the L1 may be older than they are).  The newest one,
-// which k_rows_out normalises, is read after the wait by a plain load.
-__device__ __forceinline__ double2 load_l2(const double2* p) {
-  double2 v;
-  asm volatile("ld.global.cg.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
-  return v;
-}
-
 // grid (S, ceil(m / 8)): part[(s m + j) 2 + {0, 1}] = chunk s's share of
 // V_j^* w', w' = w - sum_{g < G} tmp_g (written to w2 when G > 0)
 __global__ void __launch_bounds__(kGsTile)
@@ -140,36 +128,31 @@ k_gs_dots(const double2* V, int m, const double2* w, const double2* tmp, int G, 
   const int s = blockIdx.x;
   const long long i0 = (long long)s * chunk, i1 = min(N, i0 + chunk);
   double2 x[kGsPerWarp][PER];
-  auto fetch = [&](long long base, int from, int to, auto load) {
+  auto fetch = [&](long long base) {
 #pragma unroll
     for (int t = 0; t < kGsPerWarp; ++t)
-      if (j0 + t >= from && j0 + t < to)
+      if (j0 + t < m)
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
-          // (past the chunk: any element, which meets a zero of ws)
-          const long long i = min(base + k * 32 + lane, N - 1);
-          x[t][k] = load(V + (long long)(j0 + t) * N + i);
+          const long long i = base + k * 32 + lane;
+          x[t][k] = i < i1 ? V[(long long)(j0 + t) * N + i] : make_double2(0.0, 0.0);
         }
   };
-  auto plain = [](const double2* p) { return *p; };
-  auto older = [](const double2* p) { return load_l2(p); };
-  fetch(i0, 0, m - 1, older);  // (the newest vector may still be being normalised)
   depend_wait();
-  fetch(i0, m - 1, m, plain);
+  fetch(i0);
   double acc[2 * kGsPerWarp];
 #pragma unroll
   for (int t = 0; t < 2 * kGsPerWarp; ++t) acc[t] = 0.0;
   for (long long base = i0; base < i1; base += kGsTile) {
     const long long i = base + threadIdx.x;
+    // (before w' is formed and stored: plain loads stay behind the store)
+    if (base > i0) fetch(base);
     double2 a = make_double2(0.0, 0.0);
     if (i < i1) {
       a = minus_groups(w[i], tmp + i, N, G);
       if (G > 0 && blockIdx.y == 0) w2[i] = a;
     }
-    if (base > i0) {
-      fetch(base, 0, m, plain);
-      __syncthreads();  // the tile before has been read
-    }
+    if (base > i0) __syncthreads();  // the tile before has been read
     ws[threadIdx.x] = a;
     __syncthreads();
 #pragma unroll
@@ -207,23 +190,16 @@ k_gs_dots(const double2* V, int m, const double2* w, const double2* tmp, int G, 
 template <int NT>
 __global__ void __launch_bounds__(NT)
 k_gs_update(const double2* V, long long N, int m, int VB, const double* part, int S, double2* tmp) {
-  constexpr int AHEAD = 12;  // vectors fetched before the wait
+  constexpr int AHEAD = 12;  // vectors fetched before the coefficients are summed
   __shared__ double2 cs[kGmresMax];
   const int j0 = blockIdx.y * VB, nj = min(VB, m - j0);
   const long long i = (long long)blockIdx.x * NT + threadIdx.x;
   const double2* v = V + (long long)j0 * N + (i < N ? i : 0);
   double2 x[AHEAD];
-  // (older vectors of the group; the newest, if it is among the AHEAD, comes
-  // after the wait and is added behind them)
-  const int older = min(nj, m - 1 - j0), fetched = min(older, AHEAD);
-  const bool newest = older < nj && older < AHEAD;
-  if (older > 0) {
-#pragma unroll
-    for (int t = 0; t < AHEAD; ++t) x[t] = load_l2(v + (long long)min(t, older - 1) * N);
-  }
   depend_wait();
-  double2 xn = make_double2(0.0, 0.0);
-  if (newest) xn = v[(long long)older * N];
+#pragma unroll
+  for (int t = 0; t < AHEAD; ++t)
+    if (t < nj) x[t] = v[(long long)t * N];
   // four threads add up one coefficient
   for (int t = threadIdx.x; t < (nj + NT / 4 - 1) / (NT / 4) * NT; t += NT) {
     const int j = t / 4;
@@ -250,13 +226,8 @@ k_gs_update(const double2* V, long long N, int m, int VB, const double* part, in
   double2 a0 = make_double2(0.0, 0.0), a1 = a0;
 #pragma unroll
   for (int t = 0; t < AHEAD; t += 2) {
-    if (t < fetched) a0 = cadd(a0, cmul(cs[t], x[t]));
-    if (t + 1 < fetched) a1 = cadd(a1, cmul(cs[t + 1], x[t + 1]));
-  }
-  if (newest) {
-    const double2 y = cmul(cs[older], xn);
-    if (older % 2 == 0) a0 = cadd(a0, y);
-    else a1 = cadd(a1, y);
+    if (t < nj) a0 = cadd(a0, cmul(cs[t], x[t]));
+    if (t + 1 < nj) a1 = cadd(a1, cmul(cs[t + 1], x[t + 1]));
   }
   int j = AHEAD;
   for (; j + 8 <= nj; j += 8) {
