@@ -110,7 +110,7 @@ __global__ void k_zrotate(double2* __restrict__ V, int m, const double* __restri
 // whose partial sums the next kernel adds up (w - sum_g tmp_g).  One GB300, a
 // step at 8^3: 62 us with fourteen kernels (separate scalings, sums over the
 // groups, norm column and store; 78 with the product they were written for), 39
-// us now; at 16^3 104, where the FP64 pipe takes about half of it.
+// us now; at 16^3 104.
 
 constexpr int kGsThreads = 256;
 constexpr int kGsTile = 128;      // elements of w that a block of k_gs_dots holds
