@@ -66,6 +66,21 @@ static cudaError_t allow_smem(K* kernel, size_t bytes) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+// f(tag) with the column tile of plane edge n1: tag::N2, tag::X, tag::XL
+template <int N2_, int X_, int XL_>
+struct ColumnTile {
+  static constexpr int N2 = N2_, X = X_, XL = XL_;
+};
+template <typename R, typename F>
+static cudaError_t with_column_tile(int n1, F f) {
+  switch (n1) {
+#define NFS_CASE(N) case N: return f(ColumnTile<PlaneSplit<R, N>::N2, PlaneSplit<R, N>::X, PlaneSplit<R, N>::XL>{});
+    NFS_FOR_EACH_SIZE(NFS_CASE)
+#undef NFS_CASE
+  }
+  return cudaErrorInvalidValue;
+}
+
 // Launch with programmatic stream serialisation (see depend_wait), unless the
 // tables were written on the stream a moment ago (`serial`) or it does not pay:
 // CTAs that start early are placed on the SMs that happen to be free, which is
@@ -77,7 +92,12 @@ static cudaError_t allow_smem(K* kernel, size_t bytes) {
 template <typename R>
 static bool overlap(int n1, int n3, int P) {
   if (ElemOf<R>::NF == 1) return n1 < 128;
-  const int N2 = n1 < 24 ? 4 : 8, X = n1 < 24 ? 1 : NFS_X;
+  int N2 = 1, X = 1;
+  with_column_tile<R>(n1, [&](auto tag) {
+    N2 = decltype(tag)::N2;
+    X = decltype(tag)::X;
+    return cudaSuccess;
+  });
   return std::max(2 * N2 * n3, 3 * (n1 / N2) * (n1 / X)) * P <= 152;
 }
 template <typename... P, typename... A>
@@ -94,21 +114,6 @@ static cudaError_t launch_dependent(bool serial, void (*kernel)(P...), dim3 grid
   cfg.attrs = &attr;
   cfg.numAttrs = serial ? 0 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(a)...);
-}
-
-// f(tag) with the column tile of plane edge n1: tag::N2, tag::X, tag::XL
-template <int N2_, int X_, int XL_>
-struct ColumnTile {
-  static constexpr int N2 = N2_, X = X_, XL = XL_;
-};
-template <typename R, typename F>
-static cudaError_t with_column_tile(int n1, F f) {
-  switch (n1) {
-#define NFS_CASE(N) case N: return f(ColumnTile<PlaneSplit<R, N>::N2, PlaneSplit<R, N>::X, PlaneSplit<R, N>::XL>{});
-    NFS_FOR_EACH_SIZE(NFS_CASE)
-#undef NFS_CASE
-  }
-  return cudaErrorInvalidValue;
 }
 
 template <typename R, class Step>

@@ -149,7 +149,13 @@ __device__ __forceinline__ double block_sum_dbl(double v) {
 // 16.7 / 28.4 / 17.9 (products: 63.8 us with XL = 4, 66.8, 67.5).  X = 2 against
 // X = 4: a product of 63.8 against 68.4 us (smaller CTAs, more of them per SM).
 // The smallest grids take N2 = 4 and X = 1 to have CTAs for the whole GPU (8^3:
-// 32 row CTAs and 48 column CTAs).
+// 32 row CTAs and 48 column CTAs), and complex128 at 32 takes X = 1: with X = 2
+// its 192 column CTAs leave one on most SMs and two on some, which take twice as
+// long where the FP64 pipe is what counts.  Columns with X = 2 and X = 1 in us:
+// 32x32 35.1 and 28.9, 32x96 117.6 and 92.3, 32x128 158 and 121; products: 72.0
+// and 65.9, 209 and 183, 269 and 232 (the plane passes before: 90.5, 183, 249).
+// At 48 the two are equal, at 64 X = 1 is slower up to 24 of z and 4% faster from
+// 48 on; the double-single product gains nothing (80 and 79 us at 32x96).
 #ifndef NFS_N2_48
 #define NFS_N2_48 12
 #endif
@@ -166,7 +172,7 @@ constexpr int common_divisor(int a, int b) { return b == 0 ? a : common_divisor(
 template <typename R, int N> struct PlaneSplit {
   static constexpr bool F32 = sizeof(cplx<R>) == 8;
   static constexpr int N2 = N < 24 ? 4 : (F32 && N == 48) ? NFS_N2_48 : (F32 && N == 96) ? NFS_N2_96 : 8, N1 = N / N2;
-  static constexpr int X = N < 24 ? 1 : NFS_X;
+  static constexpr int X = N < 24 || (N == 32 && std::is_same<R, double>::value) ? 1 : NFS_X;
   // (whole runs of whole tiles: the largest part of NFS_XL that divides the
   // edge, but no shorter than a tile.  A run that does not divide it would share
   // its room with the next row's, and leave the workspace at its end)

@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 K = (0.13, -0.21, 0.37)
-SHAPES = [(8, 12), (12, 128), (16, 8), (24, 12), (32, 8), (48, 8), (48, 96), (64, 8), (96, 8), (128, 8), (128, 128)]
+SHAPES = [(8, 12), (12, 128), (16, 8), (24, 12), (32, 8), (32, 96), (48, 8), (48, 96), (64, 8), (96, 8), (128, 8), (128, 128)]
 
 
 def medium(i, grid):
