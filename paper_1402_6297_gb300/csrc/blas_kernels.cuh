@@ -175,11 +175,6 @@ __global__ void k_mark_nonzero(const double2* __restrict__ x, long long total, i
   if (any) *mark = 1;
 }
 
-__global__ void k_add(const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ y, long long n) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    y[i] = a[i] + b[i];
-}
-
 // Refinement residual per problem p (skip64, skip32: the masks of the two
 // products just launched): r_p = b_p - Ap64_p where the double-single product ran
 // (!skip64[p]), else r_p -= s_p Ap32_p where the complex64 product of the

@@ -143,9 +143,11 @@ cudaError_t pair_material_launch(const double* mat, long long smat, int n1, int 
 cudaError_t double_to_df(const double* in, df* out, long long count, cudaStream_t s);
 
 // Gradient accumulation (complex128 only) from the workspace after k_rows_in:
-// per voxel d_eps += scale * dA/deps and the chirality term of each pair:
-// chiral d_gamma[j n + v] += ..., pseudochiral dg[v] += (coupled pair ax_a) and
-// dg[n + v] += (ax_b).  Either output may be nullptr.
+// per voxel d_eps += scale * dA/deps and dg += the chirality term, 3n doubles
+// each (one n per pair) in the column kernel's order; the first vector's call
+// (`first`) sets them.  Either may be nullptr.  grad_natural_launch, after the
+// last vector, writes the caller's d_eps [3n] and d_gamma (chiral [3n],
+// pseudochiral [n]) in natural order.
 struct GradArgs {
   void* fld;
   const double2* tw1;
@@ -157,9 +159,11 @@ struct GradArgs {
   double scale;
   double* d_eps;
   double* dg;
+  bool first;
   cudaStream_t stream;
 };
 cudaError_t grad_launch(const GradArgs& a);
+cudaError_t grad_natural_launch(const GradArgs& a, double* d_eps, double* d_gamma);
 
 // Fields [E; H] = B^{-1} diag(P_r, Q_r) y of one eigenvector from the
 // workspace of y after k_rows_in (matvec_f64.cu).

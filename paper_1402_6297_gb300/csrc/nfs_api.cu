@@ -2007,12 +2007,16 @@ extern "C" int nfs_eig_grad(nfs_ctx* c, int m, const double* weights, const void
   TRY(join_caller(c));
   cudaStream_t s = c->work;
   const long long n = c->n, N = c->N;
-  // the two coupled pairs of a pseudochiral medium accumulate apart (in the
-  // work vector x64, 2n of its 8n doubles) and are added at the end
-  const bool chiral = c->kind == NFS_MEDIUM_CHIRAL;
-  double* dg = chiral ? d_gamma : (d_gamma ? reinterpret_cast<double*>(c->x64) : nullptr);
-  if (d_eps) CK(cudaMemsetAsync(d_eps, 0, 3 * n * sizeof(double), s));
-  if (dg) CK(cudaMemsetAsync(dg, 0, (chiral ? 3 : 2) * n * sizeof(double), s));
+  // the sums over the vectors, in the column kernel's order, in the work vector
+  // x64 (6n of its 8n doubles)
+  nfs::GradArgs g{};
+  g.fld = c->fld; g.tw1 = c->tw64[0]; g.tw3 = c->tw64[1];
+  g.inv_phi = c->mat64; g.gam = c->mat64 + 3 * n;
+  g.kind = c->kind; g.ax_a = c->ax_a; g.ax_b = c->ax_b;
+  g.n1 = c->n1; g.n3 = c->n3;
+  g.d_eps = d_eps ? reinterpret_cast<double*>(c->x64) : nullptr;
+  g.dg = d_gamma ? reinterpret_cast<double*>(c->x64) + 3 * n : nullptr;
+  g.stream = s;
   const double2* Y = (const double2*)Yv;
   std::vector<double> yBy;
   for (int j = 0; j < m; ++j) {
@@ -2026,21 +2030,14 @@ extern "C" int nfs_eig_grad(nfs_ctx* c, int m, const double* weights, const void
     a.stream = s;
     cudaError_t e = nfs::matvec_launch_mask<double>(a, 1);
     if (e != cudaSuccess) return cuda_fail(e, "grad rows");
-    nfs::GradArgs g{};
-    g.fld = c->fld; g.tw1 = c->tw64[0]; g.tw3 = c->tw64[1];
-    g.inv_phi = c->mat64; g.gam = c->mat64 + 3 * n;
-    g.kind = c->kind; g.ax_a = c->ax_a; g.ax_b = c->ax_b;
-    g.n1 = c->n1; g.n3 = c->n3;
-    g.scale = scale; g.d_eps = d_eps; g.dg = dg; g.stream = s;
+    g.scale = scale;
+    g.first = j == 0;
     e = nfs::grad_launch(g);
     if (e != cudaSuccess) return cuda_fail(e, "grad launch");
     c->launches += 3;  // B_r, rows, gradient
   }
-  if (!chiral && d_gamma) {
-    nfs::k_add<<<grid_blocks(n, 256), 256, 0, s>>>(dg, dg + n, d_gamma, n);
-    CK(cudaGetLastError());
-    c->launches += 1;
-  }
+  CK(nfs::grad_natural_launch(g, d_eps, d_gamma));
+  c->launches += 1;
   CK(cudaStreamSynchronize(s));
   return NFS_OK;
 }
